@@ -69,36 +69,25 @@ template <typename T> static void h2d(void *dst, const std::vector<T> &v, cudaSt
 }
 
 // ------------------------------------------------------------ upload -------
-// op code and mask-adjustment fields of a register-kernel gate record
-static uint32_t reg_opcode(uint32_t cls, uint32_t p0, uint32_t p1) {
-    auto enc = [](uint32_t opc, uint32_t sa, uint32_t sb, uint32_t xa, uint32_t xb) {
-        return opc | sa << 8 | sb << 10 | xa << 12 | xb << 13;
-    };
-    const uint32_t R = (uint32_t)REG_BITS;
-    switch (cls) {
-        case GC_SU2: return enc(OP_SU2 + p0, 0, 0, 0, 0);
-        case GC_DENSE1: return enc(OP_DENSE1 + p0, 0, 0, 0, 0);
-        case GC_H: return enc(OP_H + 2 * p0, 1, 0, 0, 0);  // + flip = bit q0 of m
-        case GC_CZ: {
-            if (p0 < R && p1 < R) {
-                const uint32_t lo = std::min(p0, p1), hi = std::max(p0, p1);
-                const uint32_t pp = lo == 0 ? hi - 1 : lo == 1 ? hi + 2 : lo == 2 ? hi + 4 : 9;
-                // want = 1 ^ mask bit; the lower position carries weight 2
-                return p0 < p1 ? enc(OP_CZ_RR + 4 * pp, 2, 1, 1, 1) : enc(OP_CZ_RR + 4 * pp, 1, 2, 1, 1);
-            }
-            if (p0 < R) return enc(OP_CZ_RT + 2 * p0, 1, 0, 1, 0);
-            if (p1 < R) return enc(OP_CZ_RT + 2 * p1, 0, 1, 0, 1);
-            return enc(OP_CZ_TT, 0, 0, 0, 0);
-        }
-        case GC_X: return enc(OP_X, 0, 0, 0, 0);
-        case GC_OMEGA: return enc(OP_OMEGA, 0, 0, 0, 0);
-        case GC_DIAG1: return enc(OP_DIAG1, 0, 0, 0, 0);
-        case GC_DIAG2: return enc(OP_DIAG2, 0, 0, 0, 0);
-        case GC_CX: return enc(OP_CX + std::min(p1, R - 1), 0, 0, 0, 0);
-        case GC_DENSE2: return enc(OP_DENSE2, 0, 0, 0, 0);
-        case GC_SWAP: return enc(OP_SWAP, 0, 0, 0, 0);
-        default: return enc(OP_NOP, 0, 0, 0, 0);
+// tables of the frames (one per pass, or per checkpoint of a resident circuit)
+static void upload_frames(arso_circuit *c, const std::vector<std::vector<std::complex<double>>> &fr) {
+    const int t = (int)c->tile_qubits;
+    std::vector<float2> tab(fr.size() * (size_t)frame_floats2(t));
+    c->frame_trivial.assign(fr.size(), 1);
+    for (size_t i = 0; i < fr.size(); ++i) {
+        frame_table(fr[i], t, tab.data() + i * frame_floats2(t));
+        for (const std::complex<double> &v : fr[i])
+            if (v != 1.0) c->frame_trivial[i] = 0;
     }
+    c->d_frame.ensure(std::max<size_t>(tab.size(), 1) * sizeof(float2));
+    if (!tab.empty())
+        ARSO_CUDA(cudaMemcpy(c->d_frame.ptr, tab.data(), tab.size() * sizeof(float2), cudaMemcpyHostToDevice));
+}
+
+// frame table of a pass's end (streaming), or NULL when it is the identity
+static const float2 *pass_frame(const arso_circuit *c, size_t pass) {
+    return c->frames && !c->frame_trivial[pass] ? c->d_frame.as<float2>() + pass * frame_floats2((int)c->tile_qubits)
+                                                : nullptr;
 }
 
 static void upload_circuit(arso_circuit *c) {
@@ -184,26 +173,16 @@ static void upload_circuit(arso_circuit *c) {
         c->d_ph_R.ensure(std::max<size_t>(c->ph_R.size(), 1) * 4);
         if (!c->ph_R.empty())
             ARSO_CUDA(cudaMemcpy(c->d_ph_R.ptr, c->ph_R.data(), c->ph_R.size() * 4, cudaMemcpyHostToDevice));
-        std::vector<RegOp> ops(std::max<size_t>(dg.size(), 1));
-        for (size_t pos = 0; pos < c->rpos.size(); ++pos) {
-            const DGate &d = dg[pos];
-            RegOp &o = ops[pos];
-            o.w0 = (uint32_t)d.cls | (uint32_t)(c->rpos[pos] & 15u) << 8 | (uint32_t)(c->rpos[pos] >> 4) << 12 |
-                   (uint32_t)d.q0 << 16 | (uint32_t)d.q1 << 24;
-            o.aux = d.mat;
-            const HostGate &h = c->gates[c->perm[pos]];
-            o.pad[0] = reg_opcode(d.cls, c->rpos[pos] & 15u, c->rpos[pos] >> 4);
-            o.pad[1] = c->tensor ? (uint32_t)c->role[pos] : (uint32_t)TR_CORE;
-            if (d.cls == GC_SU2) {
-                o.c0 = make_float2((float)h.m[0].real(), (float)h.m[0].imag());
-                o.c1 = make_float2((float)h.m[1].real(), (float)h.m[1].imag());
-            } else if (d.cls == GC_DIAG1) {
-                o.c0 = make_float2((float)h.m[0].real(), (float)h.m[0].imag());
-                o.c1 = make_float2((float)h.m[3].real(), (float)h.m[3].imag());
-            }
-        }
-        c->d_rops.ensure(ops.size() * sizeof(RegOp));
-        ARSO_CUDA(cudaMemcpy(c->d_rops.ptr, ops.data(), ops.size() * sizeof(RegOp), cudaMemcpyHostToDevice));
+        auto up = [](DeviceBuffer &d, const void *src, size_t bytes) {
+            d.ensure(std::max<size_t>(bytes, 16));
+            if (bytes) ARSO_CUDA(cudaMemcpy(d.ptr, src, bytes, cudaMemcpyHostToDevice));
+        };
+        up(c->d_rops, c->rops.data(), c->rops.size() * sizeof(RegOp));
+        up(c->d_rmats, c->rmats.data(), c->rmats.size() * sizeof(float2));
+        up(c->d_prog, c->prog.data(), c->prog.size() * sizeof(uint4));
+        up(c->d_ph_pg, c->ph_pg.data(), c->ph_pg.size() * 4);
+        up(c->d_evs, c->evs.data(), c->evs.size() * sizeof(EvSlot));
+        if (c->frames && c->engine == 1) upload_frames(c, c->frame);
         if (c->tensor) {
             c->d_ph_t.ensure(std::max<size_t>(c->ph_t.size(), 1) * 4);
             if (!c->ph_t.empty())
@@ -233,10 +212,13 @@ static ResidentArgs resident_args(const arso_circuit *c) {
     a.n_ckpt = c->n_ckpt;
     if (c->reg_blocked) {
         a.n_phases = (uint32_t)c->ph_R.size();
-        a.ph_gb = c->d_ph_gb.as<uint32_t>();
         a.ph_R = c->d_ph_R.as<uint32_t>();
-        a.rops = c->d_rops.as<RegOp>();
         a.phase_of_pos = c->d_phase_of_pos.as<uint32_t>();
+        a.mats = c->d_rmats.ptr;
+        a.prog = c->d_prog.as<uint4>();
+        a.ph_pg = c->d_ph_pg.as<uint32_t>();
+        a.evs = c->d_evs.as<EvSlot>();
+        a.frame = c->d_frame.as<float2>();
     }
     return a;
 }
@@ -255,9 +237,14 @@ static void run_pass(const arso_circuit *c, const PassArgs &a, bool last, uint32
         PassArgs b = a;
         b.pb = c->passes[a.pass].pb;
         b.pe = c->passes[a.pass].pe;
-        b.ph_gb = c->d_ph_gb.as<uint32_t>();
         b.ph_R = c->d_ph_R.as<uint32_t>();
+        b.ph_gb = c->d_ph_gb.as<uint32_t>();
         b.rops = c->d_rops.as<RegOp>();
+        b.mats = c->d_rmats.ptr;
+        b.prog = c->d_prog.as<uint4>();
+        b.ph_pg = c->d_ph_pg.as<uint32_t>();
+        b.evs = c->d_evs.as<EvSlot>();
+        b.frame = pass_frame(c, a.pass);
         if (c->tensor) {
             b.ph_t = c->d_ph_t.as<uint32_t>();
             b.tmats = c->d_tmats.ptr;
@@ -297,6 +284,11 @@ static void ensure_cache(arso_circuit *c, cudaStream_t st) {
         c->ckpt_every = every;
         c->n_ckpt = (uint32_t)(units / every + 1 + (units % every ? 1 : 0));
         c->d_cache.ensure((size_t)c->n_ckpt * sb);
+        if (c->reg_blocked) {
+            std::vector<std::vector<std::complex<double>>> fr;
+            for (uint64_t k = 0; k < c->n_ckpt; ++k) fr.push_back(c->frame[std::min<uint64_t>(k * every, units)]);
+            upload_frames(c, fr);
+        }
         launch_resident_any(c, resident_args(c), 2, (double)c->n_ckpt * sb, st);
     } else {
         const uint32_t P = (uint32_t)c->passes.size();
@@ -1007,7 +999,7 @@ static bool single_error_fidelities(arso_circuit *c, cudaStream_t st, std::vecto
             copy_h2d(d_fl.ptr, fl.data(), G * 4, st);
             copy_h2d(d_seg.ptr, seg.data(), seg.size() * 4, st);
             launch_expect_resident(c->d_gates.as<DGate>(), c->d_mats.ptr, (int)c->n, c->precision, c->d_cache.ptr,
-                                   d_seg.as<uint32_t>(), (uint32_t)(seg.size() - 1), d_fl.as<uint32_t>(),
+                                   c->reg_blocked ? c->d_frame.as<float2>() : nullptr, d_seg.as<uint32_t>(), (uint32_t)(seg.size() - 1), d_fl.as<uint32_t>(),
                                    d_out.as<double>(), st);
             copy_d2h(xyz.data(), d_out.ptr, 3 * L * 8, st);
             ARSO_CUDA(cudaStreamSynchronize(st));
@@ -1410,11 +1402,13 @@ static void run_mixed(const std::vector<size_t> &sel, arso_circuit *const *circu
                 b.n_ckpt = c->n_ckpt;
                 b.ckpt_every = (uint32_t)c->ckpt_every;
                 b.gates = c->d_gates.as<DGate>();
-                b.mats = c->d_mats.as<float2>();
-                b.ph_gb = c->d_ph_gb.as<uint32_t>();
+                b.mats = c->d_rmats.as<float2>();
                 b.ph_R = c->d_ph_R.as<uint32_t>();
                 b.phase_of_pos = c->d_phase_of_pos.as<uint32_t>();
-                b.rops = c->d_rops.as<RegOp>();
+                b.prog = c->d_prog.as<uint4>();
+                b.ph_pg = c->d_ph_pg.as<uint32_t>();
+                b.evs = c->d_evs.as<EvSlot>();
+                b.frame = c->d_frame.as<float2>();
                 b.cache = c->d_cache.as<float2>();
                 b.offsets = e->d_offsets.as<uint64_t>();
                 b.keys = e->d_key.as<uint32_t>();
@@ -1471,10 +1465,11 @@ static void run_mixed(const std::vector<size_t> &sel, arso_circuit *const *circu
         ms.t = (int)c->tile_qubits;
         ms.c = (int)c->low_qubits;
         ms.tiles = tiles;
-        ms.ph_gb = c->d_ph_gb.as<uint32_t>();
         ms.ph_R = c->d_ph_R.as<uint32_t>();
-        ms.rops = c->d_rops.as<RegOp>();
-        ms.mats = c->d_mats.as<float2>();
+        ms.mats = c->d_rmats.as<float2>();
+        ms.prog = c->d_prog.as<uint4>();
+        ms.ph_pg = c->d_ph_pg.as<uint32_t>();
+        ms.evs = c->d_evs.as<EvSlot>();
         ms.cache = c->d_cache.as<float2>();
         ms.ref_cache = overlap ? c->d_bwd.as<float2>() : c->d_cache.as<float2>();
         ms.offsets = e->d_offsets.as<uint64_t>();
@@ -1493,6 +1488,7 @@ static void run_mixed(const std::vector<size_t> &sel, arso_circuit *const *circu
             mp.gb = c->passes[j].gb;
             mp.pb = c->passes[j].pb;
             mp.pe = c->passes[j].pe;
+            mp.frame = pass_frame(c, j);
             spasses.push_back(mp);
         }
         st_cslot_off.push_back(scslot.size());
@@ -1876,11 +1872,13 @@ arso_status arso_run_batch(size_t count, arso_circuit *const *circuits, const ar
                 b.n_ckpt = c->n_ckpt;
                 b.ckpt_every = (uint32_t)c->ckpt_every;
                 b.gates = c->d_gates.as<DGate>();
-                b.mats = c->d_mats.as<float2>();
-                b.ph_gb = c->d_ph_gb.as<uint32_t>();
+                b.mats = c->d_rmats.as<float2>();
                 b.ph_R = c->d_ph_R.as<uint32_t>();
                 b.phase_of_pos = c->d_phase_of_pos.as<uint32_t>();
-                b.rops = c->d_rops.as<RegOp>();
+                b.prog = c->d_prog.as<uint4>();
+                b.ph_pg = c->d_ph_pg.as<uint32_t>();
+                b.evs = c->d_evs.as<EvSlot>();
+                b.frame = c->d_frame.as<float2>();
                 b.cache = c->d_cache.as<float2>();
                 b.offsets = e->d_offsets.as<uint64_t>();
                 b.keys = e->d_key.as<uint32_t>();

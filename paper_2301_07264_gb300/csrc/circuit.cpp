@@ -487,6 +487,40 @@ static void plan_phases(arso_circuit *c) {
             cur = R;
         }
         if (phases.empty()) phases.emplace_back(0u, load_map);
+        if (!c->tensor) {
+            // within a phase: all ready two-qubit gates, then a layer of ready one-qubit gates,
+            // one per qubit, in turn (reg_program gives a layer one dispatch)
+            std::vector<uint32_t> where(G, 0), deg(G, 0), ord;
+            for (size_t k = 0; k < phases.size(); ++k) {
+                const uint32_t b = phases[k].first, e = k + 1 < phases.size() ? phases[k + 1].first : G;
+                std::set<uint32_t> one, two;
+                auto ready = [&](uint32_t g) {
+                    (c->gates[c->perm[ps.gb + g]].arity == 1 ? one : two).insert(g);
+                };
+                for (uint32_t i = b; i < e; ++i) where[S.order[i]] = (uint32_t)k + 1, deg[S.order[i]] = 0;
+                for (uint32_t i = b; i < e; ++i)
+                    for (uint32_t x : S.succ[S.order[i]])
+                        if (where[x] == k + 1) ++deg[x];
+                for (uint32_t i = b; i < e; ++i)
+                    if (!deg[S.order[i]]) ready(S.order[i]);
+                auto emit = [&](uint32_t g) {
+                    ord.push_back(g);
+                    for (uint32_t x : S.succ[g])
+                        if (where[x] == k + 1 && --deg[x] == 0) ready(x);
+                };
+                while (!one.empty() || !two.empty()) {
+                    while (!two.empty()) {
+                        const uint32_t g = *two.begin();
+                        two.erase(two.begin());
+                        emit(g);
+                    }
+                    const std::set<uint32_t> now = one;
+                    one.clear();
+                    for (uint32_t g : now) emit(g);
+                }
+            }
+            S.order = ord;
+        }
         // the pass's new engine order
         std::vector<uint32_t> perm_new(G);
         for (uint32_t k = 0; k < G; ++k) perm_new[k] = c->perm[ps.gb + S.order[k]];
@@ -549,6 +583,386 @@ static void plan_phases(arso_circuit *c) {
         for (uint32_t pos = c->ph_gb[ph]; pos < c->ph_gb[ph + 1]; ++pos) c->phase_of_pos[pos] = (uint32_t)ph;
 }
 
+// ------------------------------------------------------ register program ---
+// op code and mask-adjustment fields of a register-kernel gate record
+static uint32_t reg_opcode(uint32_t cls, uint32_t p0, uint32_t p1) {
+    auto enc = [](uint32_t opc, uint32_t sa, uint32_t sb, uint32_t xa, uint32_t xb) {
+        return opc | sa << 8 | sb << 10 | xa << 12 | xb << 13;
+    };
+    const uint32_t R = (uint32_t)REG_BITS;
+    switch (cls) {
+        case GC_SU2: return enc(OP_SU2 + p0, 0, 0, 0, 0);
+        case GC_DENSE1: return enc(OP_DENSE1 + p0, 0, 0, 0, 0);
+        case GC_H: return enc(OP_H + 2 * p0, 1, 0, 0, 0);  // + flip = bit q0 of m
+        case GC_CZ: {
+            if (p0 < R && p1 < R) {
+                const uint32_t lo = std::min(p0, p1), hi = std::max(p0, p1);
+                const uint32_t pp = lo == 0 ? hi - 1 : lo == 1 ? hi + 2 : lo == 2 ? hi + 4 : 9;
+                // want = 1 ^ mask bit; the lower position carries weight 2
+                return p0 < p1 ? enc(OP_CZ_RR + 4 * pp, 2, 1, 1, 1) : enc(OP_CZ_RR + 4 * pp, 1, 2, 1, 1);
+            }
+            if (p0 < R) return enc(OP_CZ_RT + 2 * p0, 1, 0, 1, 0);
+            if (p1 < R) return enc(OP_CZ_RT + 2 * p1, 0, 1, 0, 1);
+            return enc(OP_CZ_TT, 0, 0, 0, 0);
+        }
+        case GC_X: return enc(OP_X, 0, 0, 0, 0);
+        case GC_OMEGA: return enc(OP_OMEGA, 0, 0, 0, 0);
+        case GC_DIAG1: return enc(OP_DIAG1, 0, 0, 0, 0);
+        case GC_DIAG2: return enc(OP_CP, 0, 0, 0, 0);
+        case GC_CX: return enc(OP_CX + std::min(p1, R - 1), 0, 0, 0, 0);
+        case GC_DENSE2: return enc(OP_DENSE2, 0, 0, 0, 0);
+        case GC_SWAP: return enc(OP_SWAP, 0, 0, 0, 0);
+        default: return enc(OP_NOP, 0, 0, 0, 0);
+    }
+}
+
+static float2 f2(cd v) { return make_float2((float)v.real(), (float)v.imag()); }
+
+static cd omega(int k) {
+    static const double s = std::sqrt(0.5);
+    static const cd w[8] = {cd(1, 0), cd(s, s), cd(0, 1), cd(-s, s), cd(-1, 0), cd(-s, -s), cd(0, -1), cd(s, -s)};
+    return w[k & 7];
+}
+
+// a unit phase: exactly omega^k when within rounding of it (k returned, else -1)
+static int snap(cd &v) {
+    v /= std::abs(v);
+    for (int k = 0; k < 8; ++k)
+        if (std::abs(v - omega(k)) < 1e-13) {
+            v = omega(k);
+            return k;
+        }
+    return -1;
+}
+
+// The frame of a tile: scalar S and phases phi (see RegOpCode in internal.h).
+struct Frame {
+    std::vector<cd> f;  // f[0] = S, f[1 + q] = phi of tile bit q
+    explicit Frame(uint32_t t) : f(1 + t, cd(1, 0)) {}
+    cd &S() { return f[0]; }
+    cd &phi(uint32_t q) { return f[1 + q]; }
+};
+
+// Largest growth of the stored state over the true one before a gate restores its
+// scale with a full matrix: G(x) grows a state by sqrt(1 + |x|^2) <= sqrt 2, so FP32's
+// range would end after some 250 gates; 2^40 keeps 2^86 of headroom above it.
+constexpr double FRAME_GROWTH = 1.0 / (1ull << 40);
+// a matrix counts as unitary (and its frame form as exact) within this
+constexpr double UNITARY_TOL = 1e-12;
+
+// What a one-qubit gate becomes in a frame.
+struct FrameGate {
+    enum { NOP, FLIP, GIV, FULL } kind = NOP;
+    bool flip = false;   // GIV: an index flip X first
+    float2 x{};          // GIV
+    cd m[4];             // FULL: the matrix
+};
+
+// U on a qubit with frame phase phi: what remains of it, and the frame after it
+static FrameGate frame_dense(Frame &F, uint32_t q, const cd *u) {
+    const cd phi = F.phi(q);
+    const cd u00 = u[0], u01 = u[1] * phi, u10 = u[2], u11 = u[3] * phi;
+    const double a = std::abs(u00), b = std::abs(u01);
+    const bool unitary = std::abs(a * a + b * b - 1.0) < UNITARY_TOL && std::abs(std::abs(u10) - b) < UNITARY_TOL &&
+                         std::abs(std::abs(u11) - a) < UNITARY_TOL &&
+                         std::abs(u00 * std::conj(u10) + u01 * std::conj(u11)) < UNITARY_TOL;
+    FrameGate g;
+    auto full = [&](cd m00, cd m01, cd m10, cd m11) {
+        g.kind = FrameGate::FULL;
+        g.m[0] = m00, g.m[1] = m01, g.m[2] = m10, g.m[3] = m11;
+    };
+    if (!unitary) {  // any matrix as it is; the frame phase goes into its columns
+        full(u00, u01, u10, u11);
+        F.phi(q) = 1;
+        return g;
+    }
+    if (b < UNITARY_TOL) {  // diagonal
+        F.S() *= u00;
+        F.phi(q) = u11 / u00;
+        snap(F.phi(q));
+        return g;
+    }
+    if (a < UNITARY_TOL) {  // diag(u01, u10) X
+        F.S() *= u01;
+        F.phi(q) = u10 / u01;
+        snap(F.phi(q));
+        g.kind = FrameGate::FLIP;
+        return g;
+    }
+    // U'' = diag(d0, d1) G(x) X^flip, the larger entry of the first row as d0
+    g.flip = a < b;
+    const cd d0 = g.flip ? u01 : u00, d1 = g.flip ? u10 : u11;
+    float2 x = f2((g.flip ? u00 : u01) / d0);
+    if (std::abs(x.x) < 1e-16f) x.x = 0.f;  // the sine and cosine of a right angle's rounding
+    if (std::abs(x.y) < 1e-16f) x.y = 0.f;
+    const double sc = 1.0 / std::sqrt(1.0 + (double)x.x * x.x + (double)x.y * x.y);  // exact scale of the rounded x
+    F.S() *= d0 / std::abs(d0) * sc;
+    F.phi(q) = d1 / d0;
+    snap(F.phi(q));
+    const double s = std::abs(F.S());
+    if (s < FRAME_GROWTH) {  // rescale: G(x) X^flip times |S|
+        const cd xs(x.x, x.y), o1(s, 0);
+        if (g.flip) full(xs * s, o1, o1, -std::conj(xs) * s);
+        else full(o1, xs * s, -std::conj(xs) * s, o1);
+        F.S() /= s;
+        return g;
+    }
+    g.kind = FrameGate::GIV;
+    g.x = x;
+    return g;
+}
+
+// Macro-ops of one phase, built gate by gate.
+struct ProgWriter {
+    std::vector<uint4> &out;
+    size_t first;                    // first unit of the phase
+    size_t last = SIZE_MAX;          // header of the last macro-op written in the phase
+    bool open = false;               // a layer being collected
+    uint32_t active = 0, real = 0, flips = 0, used = 0, end = 0;
+    float2 x[REG_BITS];
+    std::vector<uint4> czs;          // CZ gates being collected (open is false then)
+    explicit ProgWriter(std::vector<uint4> &o) : out(o), first(o.size()) {}
+    void close() {
+        if (!czs.empty()) {
+            last = out.size();
+            out.push_back(make_uint4(OP_CZS | (uint32_t)(czs.size() + 1) << 24, end, 0, 0));
+            out.insert(out.end(), czs.begin(), czs.end());
+            czs.clear();
+        }
+        if (!open) return;
+        open = false;
+        uint32_t n = 1;
+        for (int p = 0; p < REG_BITS; ++p) n += active >> p & 1;
+        last = out.size();
+        out.push_back(make_uint4(OP_LAYER | active << 8 | real << 13 | n << 24, end, 0, flips));
+        for (int p = 0; p < REG_BITS; ++p) {
+            if (!(active >> p & 1)) continue;
+            const float v[4] = {x[p].x, p ? x[p].x : -x[p].x, x[p].y, x[p].y};
+            uint32_t b[4];
+            std::memcpy(b, v, 16);
+            out.push_back(make_uint4(b[0], b[1], b[2], b[3]));
+        }
+    }
+    void start(uint32_t tile_bit) {  // a layer that has no gate on tile_bit yet
+        if (!czs.empty() || (open && (used >> tile_bit & 1))) close();
+        if (!open) open = true, active = real = flips = used = 0;
+        used |= 1u << tile_bit;
+    }
+    void nop(uint32_t tile_bit, uint32_t pos) {  // absorbed: only its events are left
+        if (open || !czs.empty()) used |= 1u << tile_bit, end = pos + 1;
+        else if (last != SIZE_MAX) out[last].y = pos + 1;
+        else start(tile_bit), end = pos + 1;
+    }
+    void flip(uint32_t tile_bit, uint32_t pos) {
+        start(tile_bit);
+        flips |= 1u << tile_bit;
+        end = pos + 1;
+    }
+    void giv(uint32_t tile_bit, uint32_t p, const FrameGate &g, uint32_t pos) {
+        start(tile_bit);
+        active |= 1u << p;
+        if (g.x.y == 0.f) real |= 1u << p;
+        if (g.flip) flips |= 1u << tile_bit;
+        x[p] = g.x;
+        end = pos + 1;
+    }
+    void cz(uint32_t q0, uint32_t q1, uint32_t p0, uint32_t p1, uint32_t pos) {
+        static const uint32_t pat[5] = {0xAAAAAAAAu, 0xCCCCCCCCu, 0xF0F0F0F0u, 0xFF00FF00u, 0xFFFF0000u};
+        const uint32_t both = 1u << q0 | 1u << q1;
+        if (open || (!czs.empty() && (used & both))) close();
+        if (czs.empty()) used = 0;
+        used |= both;
+        czs.push_back(make_uint4(p0 < 5 ? pat[p0] : 0u, p1 < 5 ? pat[p1] : 0u, 31 - q0, 31 - q1));
+        end = pos + 1;
+    }
+    // any other op, after the open layer; `before`: it may precede the open layer
+    void op(uint32_t code, uint32_t pos_end, uint32_t z, const uint32_t *c = nullptr, bool before = false) {
+        if (!before) close();
+        last = out.size();
+        out.push_back(make_uint4(code | (c ? 2u : 1u) << 24, pos_end, z, 0));
+        if (c) out.push_back(make_uint4(c[0], c[1], 0, 0));
+    }
+    // the frame phase of q applied to the state, before the gate at `pos`
+    void flush(Frame &F, uint32_t q, uint32_t p, uint32_t pos) {
+        const int k = snap(F.phi(q));
+        if (k == 0) return;
+        const bool collecting = open || !czs.empty();
+        const bool before = collecting && !(used >> q & 1);
+        if (!before) close();
+        if (k > 0) {
+            op(OP_OMEGA | (uint32_t)k << 20, before ? 0 : pos, q | p << 16, nullptr, true);
+        } else {
+            // diag(1, phi) = h diag(conj h, h), h^2 = phi: the rounded h scales both halves alike, and
+            // the host takes that scale out (a rounded phi would scale one half of the state)
+            const cd h = std::sqrt(F.phi(q));
+            const float2 hf = f2(h);
+            uint32_t c[2];
+            std::memcpy(c, &hf, 8);
+            op(OP_PHASE, before ? 0 : pos, q | p << 16, c, true);
+            F.S() *= h / std::abs(cd(hf.x, hf.y));
+        }
+        F.phi(q) = 1;
+    }
+};
+
+// Records of a circuit with tensor phases: each gate's own matrix.
+static void tensor_records(arso_circuit *c) {
+    c->rops.resize(c->perm.size());
+    for (const Pass &ps : c->passes) {
+        std::vector<int> local(c->n, -1);
+        for (size_t i = 0; i < ps.tile_qubits.size(); ++i) local[ps.tile_qubits[i]] = (int)i;
+        for (uint32_t pos = ps.gb; pos < ps.ge; ++pos) {
+            const HostGate &h = c->gates[c->perm[pos]];
+            const uint32_t p0 = c->rpos[pos] & 15u, p1 = c->rpos[pos] >> 4;
+            RegOp &o = c->rops[pos];
+            o = RegOp{};
+            uint8_t cls = h.cls;
+            o.aux = cls == GC_OMEGA ? h.omega_k : (uint32_t)c->rmats.size();
+            if (cls == GC_DENSE1) {
+                // a dense gate whose complex64 entries have the special unitary form
+                // [[a, b], [-conj b, conj a]] exactly runs on a and b alone
+                for (int i = 0; i < 4; ++i) c->rmats.push_back(f2(h.m[i]));
+                const float2 *m = c->rmats.data() + o.aux;
+                if (m[2].x == -m[1].x && m[2].y == m[1].y && m[3].x == m[0].x && m[3].y == -m[0].y) {
+                    cls = GC_SU2;
+                    o.c0 = m[0];
+                    o.c1 = m[1];
+                }
+            } else if (cls == GC_DENSE2) {
+                for (int i = 0; i < 16; ++i) c->rmats.push_back(f2(h.m[i]));
+            } else if (cls == GC_DIAG1) {
+                o.c0 = f2(h.m[0]);
+                o.c1 = f2(h.m[3]);
+            } else if (cls == GC_DIAG2) {
+                o.c0 = f2(h.m[15]);
+            }
+            o.pad[0] = reg_opcode(cls, p0, p1);
+            o.pad[1] = (uint32_t)c->role[pos];
+            o.w0 = (uint32_t)cls | p0 << 8 | p1 << 12 | (uint32_t)local[h.q0] << 16 | (uint32_t)local[h.q1] << 24;
+        }
+    }
+}
+
+// The register program of every phase (internal.h), its event table and frames: the
+// frames start from the identity in every pass (streaming) or once (resident, recorded at
+// every phase boundary).
+static void reg_program(arso_circuit *c) {
+    c->frames = c->reg_blocked && !c->tensor;
+    c->rops.clear();
+    c->prog.clear();
+    c->ph_pg.clear();
+    c->rmats.clear();
+    c->evs.clear();
+    c->frame.clear();
+    if (!c->reg_blocked) return;
+    if (!c->frames) return tensor_records(c);
+    c->evs.resize(2 * c->perm.size());
+    for (const Pass &ps : c->passes) {
+        std::vector<int> local(c->n, -1);
+        for (size_t i = 0; i < ps.tile_qubits.size(); ++i) local[ps.tile_qubits[i]] = (int)i;
+        Frame F(c->tile_qubits);
+        for (uint32_t ph = ps.pb; ph < ps.pe; ++ph) {
+            if (c->engine == 0) c->frame.push_back(F.f);
+            c->ph_pg.push_back((uint32_t)c->prog.size());
+            ProgWriter W(c->prog);
+            for (uint32_t pos = c->ph_gb[ph]; pos < c->ph_gb[ph + 1]; ++pos) {
+                const HostGate &h = c->gates[c->perm[pos]];
+                const uint32_t q0 = (uint32_t)local[h.q0], q1 = (uint32_t)local[h.q1];
+                const uint32_t p0 = c->rpos[pos] & 15u, p1 = c->rpos[pos] >> 4;
+                const uint32_t z = q0 | q1 << 8 | p0 << 16 | p1 << 20, code = reg_opcode(h.cls, p0, p1);
+                switch (h.cls) {
+                    case GC_H: {
+                        // an odd power of omega would make x a rounded constant: the same rounding
+                        // in every such gate of a Clifford+T circuit, so it is applied (compensated) first
+                        const int k = snap(F.phi(q0));
+                        if (k > 0 && (k & 1)) W.flush(F, q0, p0, pos);
+                    }  // fall through
+                    case GC_DENSE1: {
+                        const FrameGate g = frame_dense(F, q0, h.m);
+                        if (g.kind == FrameGate::NOP) {
+                            W.nop(q0, pos);
+                        } else if (g.kind == FrameGate::FLIP) {
+                            W.flip(q0, pos);
+                        } else if (g.kind == FrameGate::GIV) {
+                            W.giv(q0, p0, g, pos);
+                        } else {
+                            const uint32_t aux[2] = {(uint32_t)c->rmats.size(), 0};
+                            for (const cd &v : g.m) c->rmats.push_back(f2(v));
+                            W.op(reg_opcode(GC_DENSE1, p0, p1), pos + 1, z, aux);
+                        }
+                        break;
+                    }
+                    case GC_DIAG1:
+                    case GC_OMEGA:
+                        F.S() *= h.m[0];
+                        F.phi(q0) *= h.m[3] / h.m[0];
+                        snap(F.phi(q0));
+                        W.nop(q0, pos);
+                        break;
+                    case GC_X:  // X diag(1, phi) X = phi diag(1, conj phi)
+                        F.S() *= F.phi(q0);
+                        F.phi(q0) = std::conj(F.phi(q0));
+                        W.flip(q0, pos);
+                        break;
+                    case GC_CX:
+                        if (snap(F.phi(q1)) == 4) F.phi(q0) = -F.phi(q0);  // CX Z_t = Z_c Z_t CX
+                        else W.flush(F, q1, p1, pos);
+                        W.op(code, pos + 1, z);
+                        break;
+                    case GC_SWAP:
+                        std::swap(F.phi(q0), F.phi(q1));
+                        W.op(code, pos + 1, z);
+                        break;
+                    case GC_DENSE2: {
+                        const uint32_t aux[2] = {(uint32_t)c->rmats.size(), 0};
+                        const cd col[4] = {1.0, F.phi(q0), F.phi(q1), F.phi(q0) * F.phi(q1)};
+                        for (int i = 0; i < 16; ++i) c->rmats.push_back(f2(h.m[i] * col[i & 3]));
+                        F.phi(q0) = F.phi(q1) = 1;
+                        W.op(code, pos + 1, z, aux);
+                        break;
+                    }
+                    case GC_DIAG2: {  // commutes with the frame
+                        const float2 f = f2(h.m[15]);
+                        uint32_t cst[2];
+                        std::memcpy(cst, &f, 8);
+                        W.op(code, pos + 1, z, cst);
+                        break;
+                    }
+                    case GC_CZ: W.cz(q0, q1, p0, p1, pos); break;
+                    default: W.nop(q0, pos); break;
+                }
+                c->evs[2 * pos] = {f2(F.phi(q0)), q0, 0};
+                c->evs[2 * pos + 1] = {f2(F.phi(q1)), q1, 0};
+            }
+            W.close();
+        }
+        c->frame.push_back(F.f);  // streaming: the pass's end; resident: the circuit's
+    }
+    c->ph_pg.push_back((uint32_t)c->prog.size());
+}
+
+// The kernels' table of frame f (internal.h), in the load/store mapping {0, t-4, ..., t-1}.
+void frame_table(const std::vector<cd> &f, int t, float2 *out) {
+    const int nt = 1 << (t - REG_BITS);
+    for (int i = 0; i < nt; ++i) {
+        cd v = f[0];
+        for (int b = 0; b < t - REG_BITS; ++b)
+            if (i >> b & 1) v *= f[1 + 1 + b];
+        out[i] = f2(v);
+    }
+    auto reg = [&](int r) {
+        cd v = r & 1 ? f[1] : cd(1, 0);
+        for (int b = 0; b < 4; ++b)
+            if (r >> (1 + b) & 1) v *= f[1 + t - 4 + b];
+        return f2(v);
+    };
+    for (int k = 0; k < 16; ++k) {
+        const float2 a = reg(2 * k), b = reg(2 * k + 1);
+        out[nt + 2 * k] = make_float2(a.x, b.x);
+        out[nt + 2 * k + 1] = make_float2(a.y, b.y);
+    }
+}
+
 void build_circuit(arso_circuit *c, uint32_t n, const arso_gate *gates, size_t n_gates,
                    const arso_compile_opts *opts) {
     ARSO_REQUIRE(n >= 1 && n <= 30, "n_qubits must be in [1, 30]");
@@ -605,6 +1019,7 @@ void build_circuit(arso_circuit *c, uint32_t n, const arso_gate *gates, size_t n
         schedule_streaming(c);
     }
     plan_phases(c);  // may reorder gates within a pass
+    reg_program(c);
     c->flops_prefix.assign(n_gates + 1, 0.0);
     for (size_t pos = 0; pos < n_gates; ++pos) c->flops_prefix[pos + 1] = c->flops_prefix[pos] + gate_flops(c->gates[c->perm[pos]]);
     c->pos_of.assign(n_gates, 0);

@@ -60,6 +60,8 @@ constexpr int RB_MIN_TILE = 10;                   // 32 threads x 32 amplitudes
 // gates per phase at most: the register kernels stage a phase's gate records
 // in shared memory (double-buffered: the next phase's copy overlaps this one)
 constexpr int MAX_PHASE_OPS = 64;
+constexpr int MAX_PHASE_UNITS = 4 * MAX_PHASE_OPS;  // of the register program: a gate takes at most two, and
+                                                    // two for a phase before it
 inline uint32_t pack_rbits(const uint32_t *p) {   // 5 local bit positions, 5 bits each
     uint32_t r = 0;
     for (int b = 0; b < REG_BITS; ++b) r |= p[b] << (5 * b);
@@ -82,40 +84,75 @@ struct DGate {
     uint32_t mat;   // offset (in complex entries) into the matrix pool
 };
 
-// One gate as the register-blocked kernels see it: everything in one 32-byte
-// record (two 16-byte loads, no dependent second load for the common gates).
+// One gate of a circuit with tensor phases as the register-blocked kernels see it:
+// everything in one 32-byte record (two 16-byte loads).
 //   w0  = cls | p0 << 8 | p1 << 12 | q0 << 16 | q1 << 24, with p0/p1 the
 //         register positions of q0/q1 in the gate's phase (15: thread bit)
-//   aux = matrix-pool offset (dense and two-qubit diagonal gates) or the
-//         exponent k of GC_OMEGA
-//   c0, c1 = inline constants: (a, b) of GC_SU2, (d0, d1) of GC_DIAG1
+//   aux = matrix-pool offset (dense gates) or the exponent k of GC_OMEGA
+//   c0, c1 = inline constants: (a, b) of GC_SU2, (d0, d1) of GC_DIAG1, c0 of OP_CP
 struct __align__(16) RegOp {
     uint32_t w0, aux;
     float2 c0, c1;
     uint32_t pad[2];
 };
 
-// Register-kernel op codes (RegOp::pad[0] bits 0-7): the gate class with its
-// register positions resolved on the host, so the kernel dispatches once.
-// Mask-dependent variants follow their base code: the kernel adds
+// Register-kernel op codes (RegOp::pad[0] bits 0-7, or a macro-op's header): the gate
+// class with its register positions resolved on the host, so the kernel dispatches once.
+// Mask-dependent CZ variants follow their base code: the kernel adds
 // sa * (bit q0 of m ^ xa) + sb * (bit q1 of m ^ xb), with sa (bits 8-9),
-// sb (bits 10-11), xa (bit 12), xb (bit 13) of pad[0].
+// sb (bits 10-11), xa (bit 12), xb (bit 13).
 enum RegOpCode : uint32_t {
-    OP_SU2 = 0,      // + register position 0..4 (0: the packed lanes)
+    OP_SU2 = 0,      // + position 0..4 (0: the packed lanes); tensor circuits only
     OP_DENSE1 = 5,   // + position
-    OP_H = 10,       // + 2 * position + mask bit of q0
+    OP_H = 10,       // + 2 * position + mask bit of q0; tensor circuits only
     OP_CZ_RR = 20,   // + 4 * pair index of (lower, higher) position + 2 * want(lower) + want(higher)
     OP_CZ_RT = 60,   // + 2 * register position + want(register qubit); the other qubit is a thread bit
     OP_CZ_TT = 70,   // both qubits thread bits
-    OP_X = 71,
-    OP_OMEGA = 72,
-    OP_DIAG1 = 73,
-    OP_DIAG2 = 74,
+    OP_X = 71,       // tensor circuits only
+    OP_OMEGA = 72,   // diag(1, omega^k), omega = e^{i pi/4}
+    OP_DIAG1 = 73,   // tensor circuits only
+    OP_CP = 74,      // diag(1, 1, 1, f)
     OP_CX = 75,      // + target position
     OP_DENSE2 = 80,
     OP_SWAP = 81,
     OP_NOP = 82,
+    OP_PHASE = 83,   // diag(conj f, f)
+    OP_LAYER = 84,   // one-qubit gates on distinct qubits (below)
+    OP_CZS = 85,     // CZ gates on distinct qubits (below)
 };
+
+// Register program of a phase (circuits without tensor phases): macro-ops of 16-byte units.
+//   header: x = op code | k of OP_OMEGA (bits 20-22) | units << 24
+//           y = end: engine positions below it are done after this macro-op (their error
+//               events are applied then; a macro-op's gates act on distinct qubits, so an
+//               event commutes with the macro-op's other gates)
+//           z = q0 | q1 << 8 | p0 << 16 | p1 << 20 (tile bits and register positions)
+//           w = tile bits whose index-mask bit flips before the op (X)
+//   second unit where the op has constants: x, y = f, or x = matrix-pool offset
+//   OP_LAYER: bits 8-12 of x the register positions that hold a gate G(x), bits 13-17
+//           those whose x is real; one unit (Re x, Re x, Im x, Im x) for each, in order
+//           (position 0: (Re x, -Re x, Im x, Im x), the lanes of a packed register)
+//   OP_CZS: one unit for each CZ: the registers whose bit q0, and q1, is 1 as 32-bit masks
+//           (0 for a thread bit), and 31 - q0, 31 - q1
+// Frames: the true state is S * prod_q diag(1, phi_q) * X^m * stored, with the scalar S
+// and the unit phases phi_q the same for every trajectory and tracked on the host in FP64
+// from gate to gate (reg_program in circuit.cpp). A unitary U diag(1, phi) equals, up to
+// such a frame, G(x) = [[1, x], [-conj x, 1]] with |x| <= 1, after an index flip X
+// when |u00| < |u01|: half the multiplications of the full matrix, none at all for
+// one-qubit diagonal gates, and no rounded 1/sqrt2 for H (x = +-1). The gates of a layer
+// share one dispatch.
+
+// What an error event at an engine position and slot needs: the frame phase of its qubit
+// after the gate, and the qubit's tile bit.
+struct __align__(16) EvSlot {
+    float2 phi;
+    uint32_t q, pad;
+};
+
+// A frame as the kernels apply it, in the load/store register mapping of a t-qubit
+// tile: 2^(t-5) thread factors (S times the phases of tile bits 1..t-5), then the 32
+// register factors as 16 float4 (re, re, im, im) of registers 2k and 2k+1.
+constexpr int frame_floats2(int t) { return (1 << (t - REG_BITS)) + 32; }
 
 // Tensor-core phases (streaming complex64 circuits compiled with
 // ARSO_OPT_TENSOR_PHASES, tiles of 2^12..2^14 amplitudes). A phase whose gates on
@@ -218,6 +255,18 @@ struct arso_circuit {
     std::vector<uint32_t> phase_of_pos;     // engine position -> phase
     std::vector<double> flops_prefix;       // engine position k -> algorithmic FP32 flops per amplitude of
                                             // gates [0, k) (the tracing counts of arso.h)
+    // register program (reg_program) with its matrix pool and event table, and the frames at pass ends (streaming) or at
+    // every phase boundary (resident): 1 + t values (S, then phi of each tile bit)
+    bool frames = false;
+    std::vector<arso::RegOp> rops;          // tensor circuits: one record per gate
+    std::vector<uint4> prog;                // the others: macro-ops of all phases
+    std::vector<uint32_t> ph_pg;            // phase -> first unit of prog (plus a sentinel)
+    std::vector<float2> rmats;
+    std::vector<arso::EvSlot> evs;          // 2 per engine position
+    std::vector<std::vector<std::complex<double>>> frame;
+    arso::DeviceBuffer d_rmats, d_evs, d_prog, d_ph_pg;
+    arso::DeviceBuffer d_frame;             // tables of `frame` per pass, or per checkpoint (resident)
+    std::vector<uint8_t> frame_trivial;     // streaming: per pass
     std::vector<uint32_t> chg_prefix;       // phase k -> phases 1 <= p < k whose register set differs from p-1's
     // tensor-core phases (ARSO_OPT_TENSOR_PHASES on a streaming complex64 circuit)
     bool tensor = false;
@@ -263,6 +312,7 @@ namespace arso {
 // circuit.cpp
 void matrix_for(const arso_gate &g, HostGate &h);  // h.arity must be set
 std::vector<float> circuit_features(const arso_circuit *c, const arso_criterion *crit);
+void frame_table(const std::vector<std::complex<double>> &f, int t, float2 *out);
 void build_circuit(arso_circuit *c, uint32_t n, const arso_gate *gates, size_t n_gates,
                    const arso_compile_opts *opts);
 }  // namespace arso

@@ -47,9 +47,12 @@ struct ResidentArgs {
     void *states_out;            // non-null: store final states (count * 2^n) instead of scoring
     // register-blocked execution: checkpoints sit at phase boundaries
     uint32_t n_phases;
-    const uint32_t *ph_gb, *ph_R;
-    const RegOp *rops;
+    const uint32_t *ph_R;
     const uint32_t *phase_of_pos;  // gate position -> phase
+    const uint4 *prog;             // register program (internal.h)
+    const uint32_t *ph_pg;         // phase -> first unit of prog
+    const EvSlot *evs;             // 2 per gate position
+    const float2 *frame;           // frame tables per checkpoint (frame_floats2(n) values each)
 };
 
 // mode: 0 = score trajectories, 1 = store final states, 2 = error-free run filling the cache
@@ -85,9 +88,13 @@ struct PassArgs {
     int store_last;              // last pass stores the state instead of reducing
     // register-blocked execution
     uint32_t pb, pe;             // phases of this pass
-    const uint32_t *ph_gb;       // phase -> first engine position (with sentinel)
     const uint32_t *ph_R;        // phase -> packed register bits
-    const RegOp *rops;           // engine position -> register-kernel gate record
+    const uint32_t *ph_gb;       // tensor circuits: phase -> first engine position (with sentinel)
+    const RegOp *rops;           // tensor circuits: engine position -> gate record
+    const uint4 *prog;           // register program (internal.h)
+    const uint32_t *ph_pg;       // phase -> first unit of prog
+    const EvSlot *evs;           // 2 per gate position
+    const float2 *frame;         // frame table of the pass's end; NULL: the identity
     // tensor-core phases (NULL: every phase runs gate by gate)
     const uint32_t *ph_t;        // phase -> operand-image index or NO_TENSOR
     const void *tmats;           // TENSOR_IMAGE_HALVES fp16 values per image
@@ -105,8 +112,11 @@ struct BatchCircuit {
     uint32_t n_phases, n_ckpt, ckpt_every;
     const DGate *gates;
     const float2 *mats;
-    const uint32_t *ph_gb, *ph_R, *phase_of_pos;
-    const RegOp *rops;
+    const uint32_t *ph_R, *phase_of_pos;
+    const uint4 *prog;  // as in ResidentArgs
+    const uint32_t *ph_pg;
+    const EvSlot *evs;
+    const float2 *frame;
     const float2 *cache;
     const uint64_t *offsets;
     const uint32_t *keys;
@@ -170,6 +180,7 @@ struct MixSmall {            // resident circuit of n <= 9 qubits, gate-indexed 
 struct MixPass {
     uint64_t rest_mask;      // global bits outside the pass's tiles
     const uint32_t *offs;    // tile-high offsets of the pass
+    const float2 *frame;     // frame table of the pass's end; NULL: the identity
     uint32_t gb, pb, pe, pad;
 };
 struct MixTraj {
@@ -182,9 +193,11 @@ struct MixStream {
     int n, t, c;
     uint32_t tiles;
     const MixPass *passes;
-    const uint32_t *ph_gb, *ph_R;
-    const RegOp *rops;
+    const uint32_t *ph_R;
     const float2 *mats;
+    const uint4 *prog;
+    const uint32_t *ph_pg;
+    const EvSlot *evs;
     const float2 *cache;       // cached error-free boundary states
     const float2 *ref_cache;   // states the scored pass is compared with, same entries
     const uint32_t *cache_slot;
@@ -236,8 +249,9 @@ void launch_init_zero_state(void *psi, int n, int precision, cudaStream_t st);
 // gate: resident circuits run one CTA per cached checkpoint segment
 // (engine positions seg_pos[b] .. seg_pos[b + 1]; out[3 * location + k]), or a
 // complex64 state in HBM (launch_gate_expect below).
+// frame: the checkpoints' frame tables (register-blocked circuits) or NULL
 void launch_expect_resident(const DGate *gates, const void *mats, int n, int precision, const void *ckpt,
-                            const uint32_t *seg_pos, uint32_t n_seg, const uint32_t *first_loc, double *out,
+                            const float2 *frame, const uint32_t *seg_pos, uint32_t n_seg, const uint32_t *first_loc, double *out,
                             cudaStream_t st);
 uint32_t expect_hbm_blocks(int n);
 // One gate fused with the expectations of its qubits on the updated state; block

@@ -83,9 +83,11 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 
 // ------------------------------------------------------- register gates ---
-// Code size matters: the whole phase loop must stay resident in the
-// instruction cache, so only dense one-qubit gates, H, phase gates and CZ are
-// specialised per register position; everything else is position-free.
+// Code size matters: warps stall for instructions more than for anything else
+// when the phase loop outgrows the instruction cache (with CZ specialised per pair
+// of positions 2.9 of 9.2 warps per issue waited for them, with the mask form 1.4 of
+// 8.4), so only dense one-qubit gates and odd phases are specialised per register
+// position; everything else is position-free.
 
 // U on register bit P >= 1: packed registers k and k | 2^(P-1) hold the pairs
 template <int P>
@@ -103,6 +105,55 @@ __device__ __forceinline__ void rg_dense1(Amps &a, float2 u00, float2 u01, float
         a.im[k] = fma2(u01i, r1, fma2(u01r, i1, fma2(u00i, r0, mul2(u00r, i0))));
         a.re[k1] = fma2(n11i, i1, fma2(u11r, r1, fma2(n10i, i0, mul2(u10r, r0))));
         a.im[k1] = fma2(u11i, r1, fma2(u11r, i1, fma2(u10i, r0, mul2(u10r, i0))));
+    }
+}
+
+// G(x) = [[1, x], [-conj x, 1]] on register bit P >= 1 (the frame form of a one-qubit
+// unitary, RegOpCode in internal.h): half the instructions of the full matrix and four
+// broadcast constants instead of seven.
+template <int P> __device__ __forceinline__ void rg_giv(Amps &a, float2 xr, float2 xi) {
+    const float2 nxr = make_float2(-xr.x, -xr.y), nxi = make_float2(-xi.x, -xi.y);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        if (k & (1 << (P - 1))) continue;
+        const int k1 = k | (1 << (P - 1));
+        const float2 r0 = a.re[k], i0 = a.im[k], r1 = a.re[k1], i1 = a.im[k1];
+        a.re[k] = fma2(nxi, i1, fma2(xr, r1, r0));
+        a.im[k] = fma2(xi, r1, fma2(xr, i1, i0));
+        a.re[k1] = fma2(nxi, i0, fma2(nxr, r0, r1));
+        a.im[k1] = fma2(xi, r0, fma2(nxr, i0, i1));
+    }
+}
+// the same for a real x
+template <int P> __device__ __forceinline__ void rg_givr(Amps &a, float2 xr) {
+    const float2 nxr = make_float2(-xr.x, -xr.y);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        if (k & (1 << (P - 1))) continue;
+        const int k1 = k | (1 << (P - 1));
+        const float2 r0 = a.re[k], i0 = a.im[k], r1 = a.re[k1], i1 = a.im[k1];
+        a.re[k] = fma2(xr, r1, r0);
+        a.im[k] = fma2(xr, i1, i0);
+        a.re[k1] = fma2(nxr, r0, r1);
+        a.im[k1] = fma2(nxr, i0, i1);
+    }
+}
+// on register bit 0 (the two lanes of each packed register): xr = (Re x, -Re x)
+__device__ __forceinline__ void rg_giv_lanes(Amps &a, float2 xr, float2 xi) {
+    const float2 nxi = make_float2(-xi.x, -xi.y);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const float2 r = a.re[k], i = a.im[k], rs = swp2(r), is = swp2(i);
+        a.re[k] = fma2(nxi, is, fma2(xr, rs, r));
+        a.im[k] = fma2(xi, rs, fma2(xr, is, i));
+    }
+}
+__device__ __forceinline__ void rg_givr_lanes(Amps &a, float2 xr) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const float2 r = a.re[k], i = a.im[k];
+        a.re[k] = fma2(xr, swp2(r), r);
+        a.im[k] = fma2(xr, swp2(i), i);
     }
 }
 
@@ -349,17 +400,35 @@ template <int IDX> __device__ __forceinline__ void cz_case(Amps &a) {
     neg_quarter<cz_pa(IDX >> 2), cz_pb(IDX >> 2), (IDX >> 1) & 1, IDX & 1>(a);
 }
 
-__device__ __forceinline__ void rg_diag2(Amps &a, const TileCtx &c, uint32_t qa, uint32_t qb,
-                                         const float2 *__restrict__ d) {
-    const uint32_t pa = reg_pos(c, qa), ma = (c.m >> qa) & 1u, ta = thread_bit(c, qa);
-    const uint32_t pb = reg_pos(c, qb), mb = (c.m >> qb) & 1u, tb = thread_bit(c, qb);
-    const float2 d0 = d[0], d1 = d[1], d2 = d[2], d3 = d[3];
+// multiply the registers selected by mask by f
+__device__ __forceinline__ void phase_masked(Amps &a, uint32_t mask, float2 f) {
 #pragma unroll
-    for (int ri = 0; ri < 32; ++ri) {
-        const uint32_t k = bit_of(ri, pa, ma, ta) | (bit_of(ri, pb, mb, tb) << 1);
-        const float2 f = k == 0 ? d0 : (k == 1 ? d1 : (k == 2 ? d2 : d3));
-        amp_set(a, ri, cmul(f, amp_get(a, ri)));
+    for (int k = 0; k < 16; ++k) {
+        const bool x = (mask >> (2 * k)) & 1u, y = (mask >> (2 * k + 1)) & 1u;
+        const float2 fr = make_float2(x ? f.x : 1.f, y ? f.x : 1.f), fi = make_float2(x ? f.y : 0.f, y ? f.y : 0.f);
+        const float2 nfi = make_float2(-fi.x, -fi.y);
+        const float2 r = a.re[k], i = a.im[k];
+        a.re[k] = fma2(nfi, i, mul2(fr, r));
+        a.im[k] = fma2(fi, r, mul2(fr, i));
     }
+}
+// multiply the registers selected by mask by f, the others by its conjugate
+__device__ __forceinline__ void phase_pair(Amps &a, uint32_t mask, float2 f) {
+    const float2 fr = bc2(f.x);
+    const uint32_t b = __float_as_uint(f.y) ^ 0x80000000u;  // -f.y, the sign flipped by the mask
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const float2 fi = make_float2(__uint_as_float(b ^ sign_bit(mask, 2 * k)), __uint_as_float(b ^ sign_bit(mask, 2 * k + 1)));
+        const float2 nfi = make_float2(-fi.x, -fi.y);
+        const float2 r = a.re[k], i = a.im[k];
+        a.re[k] = fma2(nfi, i, mul2(fr, r));
+        a.im[k] = fma2(fi, r, mul2(fr, i));
+    }
+}
+// diag(1, 1, 1, f) on tile bits qa, qb
+__device__ __forceinline__ void rg_cp(Amps &a, const TileCtx &c, uint32_t qa, uint32_t qb, float2 f) {
+    const uint32_t mask = bit_mask(c, qa) & bit_mask(c, qb);
+    if (mask) phase_masked(a, mask, f);
 }
 
 // Pauli error on tile bit q of the true state (Eq. (2)): Z -> phase -1 on
@@ -477,9 +546,8 @@ __device__ __forceinline__ void smem_dense2(float2 *sm, int t, uint32_t q0, uint
 // sign pattern (want = 1 ^ mask bit).
 #define ARSO_CZ_CASE(i) case OP_CZ_RR + (i): cz_case<(i)>(a); break;
 #define ARSO_CZ_CASE4(i) ARSO_CZ_CASE(4 * (i)) ARSO_CZ_CASE(4 * (i) + 1) ARSO_CZ_CASE(4 * (i) + 2) ARSO_CZ_CASE(4 * (i) + 3)
-__device__ __forceinline__ void rg_cz_code(Amps &a, const TileCtx &c, const RegOp &op, uint32_t q0, uint32_t q1,
+__device__ __forceinline__ void rg_cz_code(Amps &a, const TileCtx &c, uint32_t x, uint32_t q0, uint32_t q1,
                                            uint32_t p0) {
-    const uint32_t x = op.pad[0];
     const uint32_t ba = ((c.m >> q0) ^ (x >> 12)) & 1u, bb = ((c.m >> q1) ^ (x >> 13)) & 1u;
     const uint32_t code = (x & 255u) + ba * ((x >> 8) & 3u) + bb * ((x >> 10) & 3u);
     if (code >= (uint32_t)OP_CZ_RT) {
@@ -517,6 +585,38 @@ __device__ __forceinline__ void rg_cz_code(Amps &a, const TileCtx &c, const RegO
 }
 #undef ARSO_CZ_CASE
 #undef ARSO_CZ_CASE4
+
+// Dense two-qubit gate M (or SWAP) on tile bits q0, q1, through shared memory
+__device__ __forceinline__ void tile_two(Amps &a, TileCtx &c, bool swap, uint32_t q0, uint32_t q1,
+                                         const float2 *__restrict__ M, float2 *sm, float2 *ubuf, int t) {
+    const uint32_t mab = ((c.m >> q0) & 1u) | (((c.m >> q1) & 1u) << 1);
+    if (c.tid < 16) {
+        const uint32_t k = c.tid >> 2, l = c.tid & 3u;
+        float2 u;
+        if (swap) {
+            const uint32_t perm[4] = {0, 2, 1, 3};
+            u = make_float2(perm[k] == l ? 1.f : 0.f, 0.f);
+        } else {
+            u = M[4 * (k ^ mab) + (l ^ mab)];
+        }
+        ubuf[c.tid] = u;
+    }
+    __syncthreads();
+    to_smem(a, sm, c, t);
+    __syncthreads();
+    smem_dense2(sm, t, q0, q1, ubuf, c.tid, c.nthr);
+    __syncthreads();
+    from_smem(a, sm, c, t);
+    __syncthreads();
+    // SWAP X^m = X^{m with bits q0, q1 exchanged} SWAP
+    if (swap && (((c.m >> q0) ^ (c.m >> q1)) & 1u)) c.m ^= (1u << q0) | (1u << q1);
+}
+
+#define ARSO_CZ_ALL \
+    case OP_CZ_RR + 0: case OP_CZ_RR + 4: case OP_CZ_RR + 8: case OP_CZ_RR + 12: case OP_CZ_RR + 16: \
+    case OP_CZ_RR + 20: case OP_CZ_RR + 24: case OP_CZ_RR + 28: case OP_CZ_RR + 32: case OP_CZ_RR + 36: \
+    case OP_CZ_RT + 0: case OP_CZ_RT + 2: case OP_CZ_RT + 4: case OP_CZ_RT + 6: case OP_CZ_RT + 8: \
+    case OP_CZ_TT
 
 // One dispatch per gate on the host-resolved base op code (class and
 // register positions); mask-dependent details (H on a flipped qubit, the CZ
@@ -562,63 +662,105 @@ __device__ __forceinline__ void apply_op(Amps &a, TileCtx &c, const RegOp &op, c
         case OP_H + 4: ARSO_HADAMARD(2); break;
         case OP_H + 6: ARSO_HADAMARD(3); break;
         case OP_H + 8: ARSO_HADAMARD(4); break;
-        case OP_CZ_RR + 0: case OP_CZ_RR + 4: case OP_CZ_RR + 8: case OP_CZ_RR + 12: case OP_CZ_RR + 16:
-        case OP_CZ_RR + 20: case OP_CZ_RR + 24: case OP_CZ_RR + 28: case OP_CZ_RR + 32: case OP_CZ_RR + 36:
-        case OP_CZ_RT + 0: case OP_CZ_RT + 2: case OP_CZ_RT + 4: case OP_CZ_RT + 6: case OP_CZ_RT + 8:
-        case OP_CZ_TT: rg_cz_code(a, c, op, q0, q1, p0); break;
+        ARSO_CZ_ALL: rg_cz_code(a, c, op.pad[0], q0, q1, p0); break;
         case OP_X: c.m ^= 1u << q0; break;
         case OP_OMEGA: rg_omega(a, c, q0, p0, op.aux); break;
         case OP_DIAG1: rg_diag1(a, c, q0, p0, op.c0, op.c1); break;
-        case OP_DIAG2: rg_diag2(a, c, q0, q1, M); break;
+        case OP_CP: rg_cp(a, c, q0, q1, op.c0); break;
         case OP_CX: ARSO_CX(0); break;
         ARSO_P4(OP_CX, ARSO_CX)
         case OP_DENSE2:
-        case OP_SWAP: {
-            const bool swap = (op.pad[0] & 255u) == OP_SWAP;
-            const uint32_t mab = ((c.m >> q0) & 1u) | (((c.m >> q1) & 1u) << 1);
-            if (c.tid < 16) {
-                const uint32_t k = c.tid >> 2, l = c.tid & 3u;
-                float2 u;
-                if (swap) {
-                    const uint32_t perm[4] = {0, 2, 1, 3};
-                    u = make_float2(perm[k] == l ? 1.f : 0.f, 0.f);
-                } else {
-                    u = M[4 * (k ^ mab) + (l ^ mab)];
-                }
-                ubuf[c.tid] = u;
-            }
-            __syncthreads();
-            to_smem(a, sm, c, t);
-            __syncthreads();
-            smem_dense2(sm, t, q0, q1, ubuf, c.tid, c.nthr);
-            __syncthreads();
-            from_smem(a, sm, c, t);
-            __syncthreads();
-            // SWAP X^m = X^{m with bits q0, q1 exchanged} SWAP
-            if (swap && (((c.m >> q0) ^ (c.m >> q1)) & 1u)) c.m ^= (1u << q0) | (1u << q1);
-            break;
-        }
+        case OP_SWAP: tile_two(a, c, (op.pad[0] & 255u) == OP_SWAP, q0, q1, M, sm, ubuf, t); break;
         default: break;
     }
-#undef ARSO_FLIP
 #undef ARSO_UA
 #undef ARSO_UB
 #undef ARSO_SU2
-#undef ARSO_D1
 #undef ARSO_HADAMARD
-#undef ARSO_CX
 }
+
+// One macro-op of a register program (internal.h): h its header, u its further units.
+__device__ __forceinline__ void apply_macro(Amps &a, TileCtx &c, const uint4 h, const uint4 *u,
+                                            const float2 *__restrict__ mats, float2 *sm, float2 *ubuf, int t) {
+    const uint32_t code = h.x & 255u;
+    if (code == OP_LAYER) {
+        c.m ^= h.w;
+        // X G(x) X = G(-conj x): the mask bit of the qubit flips the sign of Re x
+#define ARSO_LAYER_X                                                           \
+    const uint4 w = *u++;                                                      \
+    const uint32_t f = ((c.m >> rbit(c.R, P)) & 1u) << 31;                     \
+    const float2 xr = make_float2(__uint_as_float(w.x ^ f), __uint_as_float(w.y ^ f)); \
+    const float2 xi = make_float2(__uint_as_float(w.z), __uint_as_float(w.w));
+        if (h.x & 0x100u) {
+            constexpr int P = 0;
+            ARSO_LAYER_X
+            if (h.x & 0x2000u) rg_givr_lanes(a, xr);
+            else rg_giv_lanes(a, xr, xi);
+        }
+#define ARSO_LAYER_P(PP)                                        \
+        if (h.x & (0x100u << PP)) {                             \
+            constexpr int P = PP;                               \
+            ARSO_LAYER_X                                        \
+            if (h.x & (0x2000u << PP)) rg_givr<P>(a, xr);       \
+            else rg_giv<P>(a, xr, xi);                          \
+        }
+        ARSO_LAYER_P(1)
+        ARSO_LAYER_P(2)
+        ARSO_LAYER_P(3)
+        ARSO_LAYER_P(4)
+#undef ARSO_LAYER_X
+#undef ARSO_LAYER_P
+        return;
+    }
+    const uint32_t q0 = h.z & 255u, q1 = (h.z >> 8) & 255u, p0 = (h.z >> 16) & 15u;
+    switch (code) {
+        case OP_CZS: {
+            // every CZ of the layer as one sign per register: 96 ALU instructions and 10 a CZ, in
+            // code that fits the instruction cache where one block per pair of positions does not
+            const uint32_t tm = c.tpart ^ c.m;
+            uint32_t mask = 0;
+            for (const uint4 *e = u + (h.x >> 24) - 1; u < e; ++u) {
+                const uint4 w = *u;
+                const uint32_t s0 = (uint32_t)((int)(tm << w.z) >> 31), s1 = (uint32_t)((int)(tm << w.w) >> 31);
+                mask ^= (w.x ^ s0) & (w.y ^ s1);
+            }
+            negate_masked(a, mask);
+            break;
+        }
+        case OP_OMEGA: rg_omega(a, c, q0, p0, (h.x >> 20) & 7u); break;
+        case OP_PHASE: phase_pair(a, bit_mask(c, q0), make_float2(__uint_as_float(u->x), __uint_as_float(u->y))); break;
+        case OP_CP: rg_cp(a, c, q0, q1, make_float2(__uint_as_float(u->x), __uint_as_float(u->y))); break;
+        case OP_CX: ARSO_CX(0); break;
+        ARSO_P4(OP_CX, ARSO_CX)
+        case OP_DENSE1: {
+            const float2 *M = mats + u->x;
+            const uint32_t f = ARSO_FLIP;
+            rg_dense1_lanes(a, M[f ? 3 : 0], M[f ? 2 : 1], M[f ? 1 : 2], M[f ? 0 : 3]);
+            break;
+        }
+        case OP_DENSE1 + 1: { const float2 *M = mats + u->x; ARSO_D1(1); break; }
+        case OP_DENSE1 + 2: { const float2 *M = mats + u->x; ARSO_D1(2); break; }
+        case OP_DENSE1 + 3: { const float2 *M = mats + u->x; ARSO_D1(3); break; }
+        case OP_DENSE1 + 4: { const float2 *M = mats + u->x; ARSO_D1(4); break; }
+        case OP_DENSE2: tile_two(a, c, false, q0, q1, mats + u->x, sm, ubuf, t); break;
+        case OP_SWAP: tile_two(a, c, true, q0, q1, nullptr, sm, ubuf, t); break;
+        default: break;
+    }
+}
+#undef ARSO_FLIP
+#undef ARSO_D1
+#undef ARSO_CX
+#undef ARSO_CZ_ALL
 #undef ARSO_P4
 
-// Gates [g, ge) of one phase with the Pauli events that fall inside them;
-// ops[0] is the record of gate g0 (the phase's first gate). The inner loop
+// Gates [g, ge) of one phase of a tensor circuit with the Pauli events that fall inside
+// them; ops[0] is the record of gate g0 (the phase's first gate). The inner loop
 // runs up to and including the next event's gate without touching the event
 // state, which stays out of the hot registers. Records whose tensor role has
 // its bit set in `skip` are passed over (tensor phases, which hold no event).
 __device__ __forceinline__ void run_gates(Amps &v, TileCtx &c, uint32_t g, uint32_t ge, const RegOp *ops, uint32_t g0,
                                           const float2 *__restrict__ mats, float2 *sm, float2 *ubuf, int t,
-                                          const uint32_t *&ev, const uint32_t *ev_end, uint32_t &next,
-                                          uint32_t skip = 0u) {
+                                          const uint32_t *&ev, const uint32_t *ev_end, uint32_t &next, uint32_t skip) {
     while (g < ge) {
         const uint32_t np = next == NO_EVENT ? ge : ev_pos(next);
         const uint32_t stop = np < ge ? np + 1 : ge;
@@ -637,16 +779,38 @@ __device__ __forceinline__ void run_gates(Amps &v, TileCtx &c, uint32_t g, uint3
     }
 }
 
-// A phase's gate records are staged in shared memory: stage_ops starts
-// cp.async copies of the next phase's records (at most MAX_PHASE_OPS, 16 bytes
-// per copy) while the current phase runs; stage_wait waits for this thread's
-// copies and syncs the CTA, after which the staged records are visible to all
-// threads and the other buffer is free again.
-__device__ __forceinline__ void stage_ops(RegOp *dst, const RegOp *src, uint32_t n, uint32_t tid, uint32_t nthr) {
-    n = n < (uint32_t)MAX_PHASE_OPS ? n : (uint32_t)MAX_PHASE_OPS;
-    const char *s = reinterpret_cast<const char *>(src);
+// The macro-ops [u, ue) of one phase with the Pauli events that fall inside them. An X
+// or Y error would turn the frame's diag(1, phi) on its qubit into diag(phi, 1);
+// diag(phi, conj phi) on the flipped state keeps the frame the same for every trajectory.
+__device__ __forceinline__ void run_prog(Amps &v, TileCtx &c, const uint4 *u, const uint4 *ue,
+                                         const float2 *__restrict__ mats, float2 *sm, float2 *ubuf, int t,
+                                         const uint32_t *&ev, const uint32_t *ev_end, uint32_t &next,
+                                         const EvSlot *__restrict__ evs) {
+    while (u < ue) {
+        const uint4 h = *u;
+        apply_macro(v, c, h, u + 1, mats, sm, ubuf, t);
+        u += h.x >> 24;
+        while (ev_pos(next) < h.y) {
+            const float4 e = __ldg(reinterpret_cast<const float4 *>(evs + 2 * ev_pos(next) + ev_slot(next)));
+            const uint32_t q = __float_as_uint(e.z), pc = ev_code(next);
+            rg_pauli(v, c, q, pc);
+            if ((pc & 1u) && e.x != 1.f) phase_pair(v, ~bit_mask(c, q), make_float2(e.x, e.y));
+            ++ev;
+            next = ev < ev_end ? *ev : NO_EVENT;
+        }
+    }
+}
+
+// A phase's program is staged in shared memory: stage_units starts cp.async copies of
+// the next phase's 16-byte units while the current phase runs (a tensor circuit's gate
+// records are two units each); stage_wait waits for this thread's copies and syncs the
+// CTA, after which the staged units are visible to all threads and the other buffer is
+// free again.
+__device__ __forceinline__ void stage_units(uint4 *dst, const void *src, uint32_t n, uint32_t tid, uint32_t nthr) {
+    n = n < (uint32_t)MAX_PHASE_UNITS ? n : (uint32_t)MAX_PHASE_UNITS;
+    const char *s = static_cast<const char *>(src);
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-    for (uint32_t i = tid; i < 2 * n; i += nthr)
+    for (uint32_t i = tid; i < n; i += nthr)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d + 16 * i), "l"(s + 16 * i) : "memory");
     asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
@@ -780,37 +944,178 @@ __device__ __forceinline__ bool tensor_apply(Amps &v, unsigned char *abuf, const
     return ok;
 }
 
-// Criterion partial of one thread's 32 amplitudes (true index of register ri:
-// (tpart | register part) ^ m, mapped to memory by idx). Fidelity overlaps and
-// outcome/binning probabilities are summed over the 32 registers in FP32 and
-// then added to the FP64 partial (GB300's FP64 rate is a small fraction of its
-// FP32 rate; the block and trajectory sums stay FP64); argmax compares FP64
-// probabilities amplitude by amplitude.
-template <class Index>
-__device__ __forceinline__ void score_registers(Partial &acc, const DCrit &crit, const Amps &v, const TileCtx &c,
-                                                const float2 *__restrict__ ref, Index idx) {
+// Addresses of a thread's packed registers in the load mapping under an index mask:
+// packed register k holds the true tile indices j and j + 1 (swapped when the mask has
+// bit 0), j = (k ^ mr) << (t-4) | (tid ^ mt) << 1. The tile bits map to disjoint bits of
+// the state's index, so k's part is an XOR of four offsets and each register costs one XOR.
+struct LoadAt {
+    uint32_t base;   // the tile's base, the thread's part and the mask's
+    uint32_t ho[4];  // index offset of tile bits t-4 .. t-1
+    __device__ __forceinline__ uint32_t operator()(int k) const {
+        uint32_t i = base;
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+            if ((k >> b) & 1) i ^= ho[b];
+        return i;
+    }
+    __device__ __forceinline__ void mask(uint32_t mr) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+            if ((mr >> b) & 1u) base ^= ho[b];
+    }
+};
+__device__ __forceinline__ LoadAt linear_at(int t, uint32_t tid, uint32_t m) {
+    LoadAt at;
+    at.base = (tid << 1) ^ (m & ~1u);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) at.ho[b] = 1u << (t - 4 + b);
+    return at;
+}
+// of a streaming tile: offs the pass's tile-high offsets, c its contiguous low bits
+__device__ __forceinline__ LoadAt tile_at(uint32_t base, const uint32_t *__restrict__ offs, int t, int c, uint32_t tid,
+                                          uint32_t m) {
+    const uint32_t cm = (1u << c) - 1u, j = (tid ^ ((m >> 1) & ((1u << (t - REG_BITS)) - 1u))) << 1;
+    LoadAt at;
+    at.base = base + __ldg(offs + (j >> c)) + (j & cm);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        const uint32_t x = 1u << (t - 4 + b);
+        at.ho[b] = __ldg(offs + (x >> c)) + (x & cm);
+    }
+    at.mask((m >> (t - 4)) & 15u);
+    return at;
+}
+
+// Criterion partial of one thread's 32 amplitudes, in the load mapping with mask m and
+// addresses `at`. Fidelity overlaps and outcome/binning probabilities are summed over
+// the 32 registers in FP32 and then added to the FP64 partial (GB300's FP64 rate is a
+// small fraction of its FP32 rate; the block and trajectory sums stay FP64); argmax
+// compares FP64 probabilities amplitude by amplitude. The FP32 sum is a tree over the
+// register bits: the mask only swaps the branches of its nodes, so a score does not
+// depend on the checkpoint its trajectory started from. The reference is read two
+// neighbours (16 bytes) at a time.
+__device__ __forceinline__ void score_registers(Partial &acc, const DCrit &crit, const Amps &v, uint32_t m,
+                                                const float2 *__restrict__ ref, const LoadAt &at) {
+    const uint32_t flip0 = m & 1u;
     if (crit.kind == ARSO_CRIT_ARGMAX) {
 #pragma unroll
-        for (int ri = 0; ri < 32; ++ri) accumulate(acc, crit, amp_get(v, ri), ref, idx((c.tpart | reg_part(ri, c.R)) ^ c.m));
+        for (int ri = 0; ri < 32; ++ri)
+            accumulate(acc, crit, amp_get(v, ri), ref, (uint64_t)(at(ri >> 1) + ((ri & 1) ^ flip0)));
         return;
     }
-    float fa = 0.f, fb = 0.f;
+    float2 ta[5], tb[5];  // partial sums of the tree's levels
 #pragma unroll
-    for (int ri = 0; ri < 32; ++ri) {
-        const uint64_t gi = idx((c.tpart | reg_part(ri, c.R)) ^ c.m);
-        const float2 x = amp_get(v, ri);
+    for (int k = 0; k < 16; ++k) {
+        const uint32_t gi = at(k);
+        float2 sa, sb = make_float2(0.f, 0.f);
         if (crit.kind == ARSO_CRIT_FIDELITY) {
-            const float2 r = ref[gi];
-            fa = fmaf(r.x, x.x, fmaf(r.y, x.y, fa));
-            fb = fmaf(r.x, x.y, fmaf(-r.y, x.x, fb));
+            const float4 w = __ldg(reinterpret_cast<const float4 *>(ref + gi));
+            const float2 rr = flip0 ? make_float2(w.z, w.x) : make_float2(w.x, w.z);
+            const float2 ri = flip0 ? make_float2(w.w, w.y) : make_float2(w.y, w.w);
+            sa = fma2(rr, v.re[k], mul2(ri, v.im[k]));
+            sb = fma2(rr, v.im[k], mul2(make_float2(-ri.x, -ri.y), v.re[k]));
         } else {
-            const bool in = crit.kind == ARSO_CRIT_OUTCOME ? gi == crit.target
-                                                            : ((crit.bitmap[gi >> 5] >> (gi & 31)) & 1u) != 0;
-            if (in) fa = fmaf(x.x, x.x, fmaf(x.y, x.y, fa));
+            uint32_t in;  // bits 0 and 1: whether gi and gi + 1 count
+            if (crit.kind == ARSO_CRIT_OUTCOME) in = gi == (crit.target & ~1ull) ? 1u << (crit.target & 1u) : 0u;
+            else in = crit.bitmap[gi >> 5] >> (gi & 31);
+            sa = fma2(v.re[k], v.re[k], mul2(v.im[k], v.im[k]));
+            sa.x = (in >> flip0) & 1u ? sa.x : 0.f;
+            sa.y = (in >> (flip0 ^ 1u)) & 1u ? sa.y : 0.f;
+        }
+#pragma unroll
+        for (int l = 0; l < 5; ++l) {
+            if (!((k >> l) & 1)) {
+                ta[l] = sa;
+                tb[l] = sb;
+                break;
+            }
+            sa = add2(ta[l], sa);
+            sb = add2(tb[l], sb);
         }
     }
-    acc.a += (double)fa;
-    acc.b += (double)fb;
+    acc.a += (double)(ta[4].x + ta[4].y);
+    acc.b += (double)(tb[4].x + tb[4].y);
+}
+
+// the tile's amplitudes from / to memory, in the load mapping
+template <bool L2ONLY>
+__device__ __forceinline__ void load_tile(Amps &v, const float2 *__restrict__ src, const LoadAt &at) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const float4 *p = reinterpret_cast<const float4 *>(src + at(k));
+        const float4 w = L2ONLY ? __ldcg(p) : __ldg(p);
+        v.re[k] = make_float2(w.x, w.z);
+        v.im[k] = make_float2(w.y, w.w);
+    }
+}
+__device__ __forceinline__ void store_tile(const Amps &v, float2 *dst, uint32_t m, const LoadAt &at) {
+    const uint32_t flip0 = m & 1u;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const float2 r = flip0 ? swp2(v.re[k]) : v.re[k], i = flip0 ? swp2(v.im[k]) : v.im[k];
+        *reinterpret_cast<float4 *>(dst + at(k)) = make_float4(r.x, i.x, r.y, i.y);
+    }
+}
+
+// v (in the load mapping, mask c.m) times the frame table (internal.h) and i^gp
+__device__ __forceinline__ void apply_frame(Amps &v, TileCtx &c, const float2 *__restrict__ frame, int t) {
+    const uint32_t nt = 1u << (t - REG_BITS);
+    const float4 *T = reinterpret_cast<const float4 *>(frame + nt);
+    float2 F = __ldg(frame + (c.tid ^ ((c.m >> 1) & (nt - 1u))));
+    if (c.gp & 1u) F = make_float2(-F.y, F.x);
+    if (c.gp & 2u) F = make_float2(-F.x, -F.y);
+    c.gp = 0;
+    const uint32_t mr = (c.m >> (t - 4)) & 15u, flip0 = c.m & 1u;
+    const float2 fr = bc2(F.x), fi = bc2(F.y), nfi = bc2(-F.y);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const float4 w = __ldg(T + ((uint32_t)k ^ mr));
+        const float2 tr = flip0 ? make_float2(w.y, w.x) : make_float2(w.x, w.y);
+        const float2 ti = flip0 ? make_float2(w.w, w.z) : make_float2(w.z, w.w);
+        const float2 gr = fma2(nfi, ti, mul2(fr, tr)), gi = fma2(fi, tr, mul2(fr, ti));
+        const float2 ngi = make_float2(-gi.x, -gi.y);
+        const float2 r = v.re[k], i = v.im[k];
+        v.re[k] = fma2(ngi, i, mul2(gr, r));
+        v.im[k] = fma2(gi, r, mul2(gr, i));
+    }
+}
+
+// register set of the load/store mapping {0, t-4, ..., t-1}
+__device__ __forceinline__ uint32_t load_set(int t) {
+    return ((uint32_t)(t - 4) << 5) | ((uint32_t)(t - 3) << 10) | ((uint32_t)(t - 2) << 15) | ((uint32_t)(t - 1) << 20);
+}
+// the true state up to its mask, in the load mapping
+__device__ __forceinline__ void finish_tile(Amps &v, float2 *sm, TileCtx &c, const float2 *__restrict__ frame, int t) {
+    if (c.R != load_set(t)) remap(v, sm, c, load_set(t), t);
+    if (frame) apply_frame(v, c, frame, t);
+    else apply_global_phase(v, c);
+}
+
+// Per-group sums of a criterion partial: `group` threads (a power of two, at least a
+// warp) each; the group's first thread gets its sum. Ends with red[] free to reuse only
+// after the caller's next barrier.
+__device__ __forceinline__ Partial group_reduce_partial(Partial acc, Partial *red, uint32_t group) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double a2 = __shfl_down_sync(0xffffffffu, acc.a, o);
+        const double b2 = __shfl_down_sync(0xffffffffu, acc.b, o);
+        const double mp = __shfl_down_sync(0xffffffffu, acc.maxp, o);
+        const unsigned long long mi = __shfl_down_sync(0xffffffffu, acc.idx, o);
+        acc.a += a2;
+        acc.b += b2;
+        argmax_merge(acc.maxp, acc.idx, mp, mi);
+    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if ((threadIdx.x & (group - 1)) == 0) {
+        const uint32_t w0 = threadIdx.x >> 5, nw = group >> 5;
+        for (uint32_t w = w0 + 1; w < w0 + nw; ++w) {
+            acc.a += red[w].a;
+            acc.b += red[w].b;
+            argmax_merge(acc.maxp, acc.idx, red[w].maxp, red[w].idx);
+        }
+    }
+    return acc;
 }
 
 // global offset of the tile's first amplitude: the tile index deposited into
@@ -824,191 +1129,198 @@ __device__ __forceinline__ uint64_t tile_base(uint64_t rest_mask, uint64_t tile)
     return base;
 }
 
+// where a slot's tile comes from, and its events from the pass's first gate on; false
+// when the slot does not run this pass
+__device__ __forceinline__ bool pass_source(const PassArgs &a, uint32_t slot, const float2 *&src, const uint32_t *&ev,
+                                            const uint32_t *&ev_end) {
+    const uint64_t N = 1ull << a.n;
+    ev = ev_end = nullptr;
+    if (a.ideal) {
+        src = static_cast<const float2 *>(a.ideal_src);
+        return true;
+    }
+    const int start = a.start_pass[slot];
+    if (a.pass < start || a.pass > a.end_pass[slot]) return false;
+    src = a.pass == start ? static_cast<const float2 *>(a.cache) + (size_t)a.cache_slot[start] * N
+                          : static_cast<const float2 *>(a.work) + (size_t)slot * N;
+    // binary search for the first key at or after the pass's first gate
+    const uint64_t tr = a.slot_traj[slot];
+    const uint32_t *lo = a.keys + a.offsets[tr], *hi = a.keys + a.offsets[tr + 1];
+    ev_end = hi;
+    const uint32_t key_lo = a.gb << 3;
+    while (lo < hi) {
+        const uint32_t *mid = lo + (hi - lo) / 2;
+        if (*mid < key_lo) lo = mid + 1;
+        else hi = mid;
+    }
+    ev = lo;
+    return true;
+}
+
+// end of a pass: the tile scored against the cached state at the boundary, or stored
+__device__ __forceinline__ void pass_finish(const PassArgs &a, Amps &v, TileCtx &c, uint32_t slot, uint32_t tile,
+                                            uint32_t tiles, Partial *red) {
+    const uint64_t N = 1ull << a.n;
+    if (a.frame) apply_frame(v, c, a.frame, a.t);
+    else apply_global_phase(v, c);
+    const LoadAt at = tile_at((uint32_t)tile_base(a.rest_mask, tile), a.offs, a.t, a.c, c.tid, c.m);
+    if (!a.ideal && !a.store_last && a.pass == a.end_pass[slot]) {
+        const float2 *ref = static_cast<const float2 *>(a.ref_cache ? a.ref_cache : a.cache) +
+                            (size_t)a.cache_slot[a.pass + 1] * N;
+        Partial acc = empty_partial();
+        score_registers(acc, a.crit, v, c.m, ref, at);
+        acc = group_reduce_partial(acc, red, c.nthr);
+        if (c.tid == 0) a.partials[(size_t)slot * tiles + tile] = acc;
+        return;
+    }
+    store_tile(v, a.ideal ? static_cast<float2 *>(a.ideal_dst) : static_cast<float2 *>(a.work) + (size_t)slot * N, c.m, at);
+}
+
+// One pass over tiles of 2^t amplitudes: a CTA runs THREADS / 2^(t-5) neighbouring tiles
+// of one slot side by side.
 // The phase loop holds the 64 amplitude registers; everything needed only
 // before or after it (addresses, slot data) is recomputed there instead of
 // being kept live.
-// TENSOR: the launch has tensor phases (a separate instantiation, so that the
-// gate-by-gate kernel's code is not shaped by the contraction path). SMALL:
-// tiles of at most 2^12 amplitudes (at most 128 threads), compiled for five
-// CTAs per SM (96 registers, a few more spills) instead of four: measured 5%
-// faster on the 24-qubit benchmark at 12-qubit tiles.
-template <bool LAST, bool TENSOR, bool SMALL = false>
-__global__ void __launch_bounds__(SMALL ? 128 : 512, SMALL ? 5 : 1) pass_rb_kernel(PassArgs a) {
+template <int THREADS, int MINB>
+__global__ void __launch_bounds__(THREADS, MINB) pass_rb_kernel(PassArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *sm = reinterpret_cast<float2 *>(smem_raw);
-    __shared__ Partial red[32];
-    __shared__ float2 ubuf[16];
-    __shared__ RegOp s_ops[2][MAX_PHASE_OPS];
+    __shared__ Partial red[THREADS / 32];
+    __shared__ float2 ubuf[THREADS / 32][16];
+    __shared__ uint4 s_ops[2][MAX_PHASE_UNITS];
     const int t = a.t;
-    const uint32_t slot = blockIdx.y;
-    const uint64_t N = 1ull << a.n;
-    const uint32_t cmask = (1u << a.c) - 1u;
-    auto gidx = [&](uint64_t base, uint32_t j) -> uint64_t { return base + a.offs[j >> a.c] + (j & cmask); };
-
-    // load mapping R = {0, t-4, ..., t-1}: register ri = b0 | hi << 1 holds j = hi << (t-4) | tid << 1 | b0
-    const uint32_t load_packed = 0u | ((uint32_t)(t - 4) << 5) | ((uint32_t)(t - 3) << 10) |
-                                 ((uint32_t)(t - 2) << 15) | ((uint32_t)(t - 1) << 20);
+    TileCtx c;
+    c.m = 0;
+    c.gp = 0;
+    c.nthr = 1u << (t - REG_BITS);
+    c.tid = threadIdx.x & (c.nthr - 1u);
+    const uint32_t sg = threadIdx.x >> (t - REG_BITS), groups = blockDim.x >> (t - REG_BITS);
+    float2 *sm = reinterpret_cast<float2 *>(smem_raw) + ((size_t)sg << t);
     Amps v;
-    const uint32_t *ev = nullptr, *ev_end = nullptr;
+    const uint32_t *ev, *ev_end;
     {
         const float2 *src;
-        if (a.ideal) {
-            src = static_cast<const float2 *>(a.ideal_src);
-        } else {
-            const int start = a.start_pass[slot];
-            if (a.pass < start || a.pass > a.end_pass[slot]) return;
-            src = a.pass == start ? static_cast<const float2 *>(a.cache) + (size_t)a.cache_slot[start] * N
-                                  : static_cast<const float2 *>(a.work) + (size_t)slot * N;
-            // this pass's events: binary search for the first key at or after the pass's first gate
-            const uint64_t tr = a.slot_traj[slot];
-            const uint32_t *lo = a.keys + a.offsets[tr];
-            const uint32_t *hi = a.keys + a.offsets[tr + 1];
-            ev_end = hi;
-            const uint32_t key_lo = a.gb << 3;
-            while (lo < hi) {
-                const uint32_t *mid = lo + (hi - lo) / 2;
-                if (*mid < key_lo) lo = mid + 1;
-                else hi = mid;
-            }
-            ev = lo;
-        }
-        const uint64_t base = tile_base(a.rest_mask, blockIdx.x);
-#pragma unroll
-        for (int hi = 0; hi < 16; ++hi) {
-            const uint32_t j = ((uint32_t)hi << (t - 4)) | (threadIdx.x << 1);
-            const float4 w = __ldg(reinterpret_cast<const float4 *>(src + gidx(base, j)));
-            v.re[hi] = make_float2(w.x, w.z);
-            v.im[hi] = make_float2(w.y, w.w);
-        }
+        if (!pass_source(a, blockIdx.y, src, ev, ev_end)) return;
+        const uint32_t tile = blockIdx.x * groups + sg;
+        load_tile<false>(v, src, tile_at((uint32_t)tile_base(a.rest_mask, tile), a.offs, t, a.c, c.tid, 0u));
     }
+    set_phase(c, load_set(t), t);
+    uint32_t next = ev < ev_end ? *ev : NO_EVENT;
+    const float2 *mats = static_cast<const float2 *>(a.mats);
+    if (a.pb < a.pe)
+        stage_units(s_ops[0], a.prog + a.ph_pg[a.pb], a.ph_pg[a.pb + 1] - a.ph_pg[a.pb], threadIdx.x, blockDim.x);
+    for (uint32_t ph = a.pb; ph <= a.pe; ++ph) {  // and back to the load mapping: one copy of the remap's code
+        const uint32_t buf = (ph - a.pb) & 1u;
+        stage_wait();
+        if (ph + 1 < a.pe)
+            stage_units(s_ops[buf ^ 1u], a.prog + a.ph_pg[ph + 1], a.ph_pg[ph + 2] - a.ph_pg[ph + 1], threadIdx.x,
+                        blockDim.x);
+        const uint32_t R = ph < a.pe ? a.ph_R[ph] : load_set(t);
+        if (R != c.R) remap<true>(v, sm, c, R, t);
+        if (ph == a.pe) break;
+        run_prog(v, c, s_ops[buf], s_ops[buf] + (a.ph_pg[ph + 1] - a.ph_pg[ph]), mats, sm, ubuf[sg], t, ev, ev_end, next,
+                 a.evs);
+    }
+    pass_finish(a, v, c, blockIdx.y, blockIdx.x * groups + sg, gridDim.x * groups, red);
+}
+
+// The same for circuits with tensor phases: one tile per CTA, gate records instead of the
+// register program, and the contraction above for the phases that qualify.
+__global__ void __launch_bounds__(512, 1) pass_tensor_kernel(PassArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float2 *sm = reinterpret_cast<float2 *>(smem_raw);
+    __shared__ Partial red[16];
+    __shared__ float2 ubuf[16];
+    __shared__ uint4 s_ops[2][2 * MAX_PHASE_OPS];
+    const int t = a.t;
     TileCtx c;
     c.m = 0;
     c.gp = 0;
     c.tid = threadIdx.x;
     c.nthr = blockDim.x;
-    set_phase(c, load_packed, t);
-
+    Amps v;
+    const uint32_t *ev, *ev_end;
+    {
+        const float2 *src;
+        if (!pass_source(a, blockIdx.y, src, ev, ev_end)) return;
+        load_tile<false>(v, src, tile_at((uint32_t)tile_base(a.rest_mask, blockIdx.x), a.offs, t, a.c, c.tid, 0u));
+    }
+    set_phase(c, load_set(t), t);
     uint32_t next = ev < ev_end ? *ev : NO_EVENT;
     const float2 *mats = static_cast<const float2 *>(a.mats);
-    // tensor phases: tensor memory for D0 and D1 (128 columns per block of 128 rows), one mbarrier
+    // tensor memory for D0 and D1 (128 columns per block of 128 rows), one mbarrier
     // for the contractions' completion, and two 16 KiB buffers for the staged B images
     __shared__ uint64_t s_tbar[4];  // one per block of 128 rows
     __shared__ uint32_t s_tmem;
-    constexpr bool tensor = TENSOR;
     const uint32_t nblk = blockDim.x / TP_ROWS;
     unsigned char *img = smem_raw + ((size_t)1 << t) * sizeof(float2);
     const unsigned char *tmats = static_cast<const unsigned char *>(a.tmats);
-    uint32_t tmem = 0, tpar = 0;
-    if (tensor) {
-        if (threadIdx.x < 32) tmem_alloc(&s_tmem, nblk * 128u);
-        if (threadIdx.x < nblk) {
-            mbar_init(&s_tbar[threadIdx.x], 1);
-            fence_mbar_init();
-        }
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        tmem = s_tmem;
+    uint32_t tpar = 0;
+    if (threadIdx.x < 32) tmem_alloc(&s_tmem, nblk * 128u);
+    if (threadIdx.x < nblk) {
+        mbar_init(&s_tbar[threadIdx.x], 1);
+        fence_mbar_init();
     }
-    if (a.pb < a.pe) {
-        if (tensor && a.ph_t[a.pb] != NO_TENSOR)
-            stage_image(img, tmats + (size_t)a.ph_t[a.pb] * TP_IMAGE_BYTES, threadIdx.x, blockDim.x);
-        stage_ops(s_ops[0], a.rops + a.ph_gb[a.pb], a.ph_gb[a.pb + 1] - a.ph_gb[a.pb], threadIdx.x, blockDim.x);
-    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+    auto stage = [&](uint32_t ph, uint32_t buf) {
+        if (a.ph_t[ph] != NO_TENSOR)
+            stage_image(img + buf * TP_IMAGE_BYTES, tmats + (size_t)a.ph_t[ph] * TP_IMAGE_BYTES, threadIdx.x, blockDim.x);
+        stage_units(s_ops[buf], a.rops + a.ph_gb[ph], 2 * (a.ph_gb[ph + 1] - a.ph_gb[ph]), threadIdx.x, blockDim.x);
+    };
+    if (a.pb < a.pe) stage(a.pb, 0);
     for (uint32_t ph = a.pb; ph < a.pe; ++ph) {
         const uint32_t buf = (ph - a.pb) & 1u;
         stage_wait();
-        if (ph + 1 < a.pe) {
-            if (tensor && a.ph_t[ph + 1] != NO_TENSOR)
-                stage_image(img + (buf ^ 1u) * TP_IMAGE_BYTES, tmats + (size_t)a.ph_t[ph + 1] * TP_IMAGE_BYTES,
-                            threadIdx.x, blockDim.x);
-            stage_ops(s_ops[buf ^ 1u], a.rops + a.ph_gb[ph + 1], a.ph_gb[ph + 2] - a.ph_gb[ph + 1], threadIdx.x,
-                      blockDim.x);
-        }
+        if (ph + 1 < a.pe) stage(ph + 1, buf ^ 1u);
         const uint32_t R = a.ph_R[ph];
         if (R != c.R) remap<true>(v, sm, c, R, t);
         const uint32_t g0 = a.ph_gb[ph], ge = a.ph_gb[ph + 1];
-        if constexpr (TENSOR) {
-            // the contraction applies U to the true amplitudes: no event of this trajectory in
-            // the phase and no mask bit on a register bit (the CTA takes the same branch)
-            uint32_t rm = 0;
+        // the contraction applies U to the true amplitudes: no event of this trajectory in
+        // the phase and no mask bit on a register bit (the CTA takes the same branch)
+        uint32_t rm = 0;
 #pragma unroll
-            for (int b = 0; b < REG_BITS; ++b) rm |= 1u << rbit(R, b);
-            const bool tp =
-                a.ph_t[ph] != NO_TENSOR && (next == NO_EVENT || ev_pos(next) >= ge) && (c.m & rm) == 0u;
-            const int rounds = tp ? 2 : 1;
+        for (int b = 0; b < REG_BITS; ++b) rm |= 1u << rbit(R, b);
+        const bool tp = a.ph_t[ph] != NO_TENSOR && (next == NO_EVENT || ev_pos(next) >= ge) && (c.m & rm) == 0u;
+        const int rounds = tp ? 2 : 1;
 #pragma unroll 1
-            for (int rd = 0; rd < rounds; ++rd) {
-                if (rd == 1) {
-                    __syncthreads();  // every thread's reads of the tile buffer are done
-                    if (!tensor_apply(v, smem_raw, img + buf * TP_IMAGE_BYTES, nblk, tmem, s_tbar, tpar))
-                        atomicOr(a.terr, 1u);
-                }
-                const uint32_t skip =
-                    tp ? (rd == 0 ? (1u << TR_CORE) | (1u << TR_AFTER) : (1u << TR_CORE) | (1u << TR_BEFORE)) : 0u;
-                run_gates(v, c, g0, ge, s_ops[buf], g0, mats, sm, ubuf, t, ev, ev_end, next, skip);
+        for (int rd = 0; rd < rounds; ++rd) {
+            if (rd == 1) {
+                __syncthreads();  // every thread's reads of the tile buffer are done
+                if (!tensor_apply(v, smem_raw, img + buf * TP_IMAGE_BYTES, nblk, tmem, s_tbar, tpar))
+                    atomicOr(a.terr, 1u);
             }
-        } else {
-            run_gates(v, c, g0, ge, s_ops[buf], g0, mats, sm, ubuf, t, ev, ev_end, next);
+            const uint32_t skip =
+                tp ? (rd == 0 ? (1u << TR_CORE) | (1u << TR_AFTER) : (1u << TR_CORE) | (1u << TR_BEFORE)) : 0u;
+            run_gates(v, c, g0, ge, reinterpret_cast<const RegOp *>(s_ops[buf]), g0, mats, sm, ubuf, t, ev, ev_end, next,
+                      skip);
         }
     }
-    if (tensor) {
-        tc_fence_before();
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            tc_fence_after();
-            tmem_free(tmem, nblk * 128u);
-        }
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        tc_fence_after();
+        tmem_free(tmem, nblk * 128u);
     }
-    apply_global_phase(v, c);  // global phase i^gp
-    const uint64_t base = tile_base(a.rest_mask, blockIdx.x);
-    if (!a.ideal && !a.store_last && a.pass == a.end_pass[slot]) {
-        const float2 *ref = static_cast<const float2 *>(a.ref_cache ? a.ref_cache : a.cache) +
-                            (size_t)a.cache_slot[a.pass + 1] * N;
-        Partial acc = empty_partial();
-        score_registers(acc, a.crit, v, c, ref, [&](uint32_t j) { return gidx(base, j); });
-        acc = block_reduce_partial(acc, red);
-        if (threadIdx.x == 0) a.partials[(size_t)slot * gridDim.x + blockIdx.x] = acc;
-        return;
-    }
-    if (c.R != load_packed) remap(v, sm, c, load_packed, t);
-    float2 *dst = a.ideal ? static_cast<float2 *>(a.ideal_dst) : static_cast<float2 *>(a.work) + (size_t)slot * N;
-    const uint32_t flip0 = c.m & 1u;
-#pragma unroll
-    for (int hi = 0; hi < 16; ++hi) {
-        const uint32_t j = (((uint32_t)hi << (t - 4)) | (threadIdx.x << 1)) ^ (c.m & ~1u);
-        const float2 r = flip0 ? swp2(v.re[hi]) : v.re[hi], i = flip0 ? swp2(v.im[hi]) : v.im[hi];
-        reinterpret_cast<float4 *>(dst + gidx(base, j))[0] = make_float4(r.x, i.x, r.y, i.y);
-    }
+    if (c.R != load_set(t)) remap(v, sm, c, load_set(t), t);
+    pass_finish(a, v, c, blockIdx.y, blockIdx.x, gridDim.x, red);
 }
 
 // ------------------------------------------------------------- resident ---
 // Whole state (2^n, 10 <= n <= 13) in one CTA: each trajectory restarts from
 // the cached error-free state at the checkpoint (phase boundary) at or before
-// its first error and runs the remaining phases; ckpt_every counts phases.
+// its first error and runs the remaining phases; ckpt_every counts phases. The
+// checkpoints before the last are in their boundary's frame (RegOpCode, internal.h), so
+// that a run from any of them has the bits of a run through it; the last is the true psi_R.
 
-__device__ __forceinline__ void rb_load_linear(Amps &v, const float2 *src, int t, uint32_t tid) {
-#pragma unroll
-    for (int hi = 0; hi < 16; ++hi) {
-        const uint32_t j = ((uint32_t)hi << (t - 4)) | (tid << 1);
-        const float4 w = __ldg(reinterpret_cast<const float4 *>(src + j));
-        v.re[hi] = make_float2(w.x, w.z);
-        v.im[hi] = make_float2(w.y, w.w);
-    }
-}
-
-// store the true state (mask and global phase applied); leaves v in the load mapping
-__device__ __forceinline__ void rb_store_linear(Amps &v, float2 *sm, TileCtx &c, uint32_t load_packed, float2 *dst,
-                                                int t) {
-    if (c.R != load_packed) remap(v, sm, c, load_packed, t);
-    apply_global_phase(v, c);
-    const uint32_t flip0 = c.m & 1u;
-#pragma unroll
-    for (int hi = 0; hi < 16; ++hi) {
-        const uint32_t j = (((uint32_t)hi << (t - 4)) | (c.tid << 1)) ^ (c.m & ~1u);
-        const float2 r = flip0 ? swp2(v.re[hi]) : v.re[hi], i = flip0 ? swp2(v.im[hi]) : v.im[hi];
-        reinterpret_cast<float4 *>(dst + j)[0] = make_float4(r.x, i.x, r.y, i.y);
-    }
+// store the state (mask applied) to dst, times the frame when one is given; without one
+// v stays as it is (in the load mapping)
+__device__ __forceinline__ void rb_store_linear(Amps &v, float2 *sm, TileCtx &c, float2 *dst, int t,
+                                                const float2 *__restrict__ frame) {
+    if (c.R != load_set(t)) remap(v, sm, c, load_set(t), t);
+    if (frame) apply_frame(v, c, frame, t);
+    store_tile(v, dst, c.m, linear_at(t, c.tid, c.m));
 }
 
 template <int MODE>
@@ -1017,13 +1329,11 @@ __global__ void __launch_bounds__(512, 1) resident_rb_kernel(ResidentArgs a) {
     float2 *sm = reinterpret_cast<float2 *>(smem_raw);
     __shared__ Partial red[32];
     __shared__ float2 ubuf[16];
-    __shared__ RegOp s_ops[2][MAX_PHASE_OPS];
+    __shared__ uint4 s_ops[2][MAX_PHASE_UNITS];
     const int t = a.n;
     const uint32_t N = 1u << t;
     const float2 *cache = static_cast<const float2 *>(a.cache);
     const float2 *mats = static_cast<const float2 *>(a.mats);
-    const uint32_t load_packed = 0u | ((uint32_t)(t - 4) << 5) | ((uint32_t)(t - 3) << 10) |
-                                 ((uint32_t)(t - 2) << 15) | ((uint32_t)(t - 1) << 20);
     const uint64_t count = MODE == 2 ? 1 : a.count;
     for (uint64_t b = blockIdx.x; b < count; b += gridDim.x) {
         Amps v;
@@ -1032,7 +1342,7 @@ __global__ void __launch_bounds__(512, 1) resident_rb_kernel(ResidentArgs a) {
         c.gp = 0;
         c.tid = threadIdx.x;
         c.nthr = blockDim.x;
-        set_phase(c, load_packed, t);
+        set_phase(c, load_set(t), t);
         uint32_t ph0 = 0;
         const uint32_t *ev = nullptr, *ev_end = nullptr;
         uint64_t tr = 0;
@@ -1058,38 +1368,39 @@ __global__ void __launch_bounds__(512, 1) resident_rb_kernel(ResidentArgs a) {
                 ck = a.phase_of_pos[first] / (uint32_t)a.ckpt_every;
                 ph0 = ck * (uint32_t)a.ckpt_every;
             }
-            rb_load_linear(v, cache + (size_t)ck * N, t, c.tid);
+            load_tile<false>(v, cache + (size_t)ck * N, linear_at(t, c.tid, 0u));
             ev = a.keys + a.offsets[tr];
             ev_end = a.keys + a.offsets[tr + 1];
         }
         uint32_t next = ev && ev < ev_end ? *ev : NO_EVENT;
         if (ph0 < a.n_phases)
-            stage_ops(s_ops[0], a.rops + a.ph_gb[ph0], a.ph_gb[ph0 + 1] - a.ph_gb[ph0], threadIdx.x, blockDim.x);
+            stage_units(s_ops[0], a.prog + a.ph_pg[ph0], a.ph_pg[ph0 + 1] - a.ph_pg[ph0], threadIdx.x, blockDim.x);
         for (uint32_t ph = ph0; ph < a.n_phases; ++ph) {
             const uint32_t buf = (ph - ph0) & 1u;
             stage_wait();
             if (ph + 1 < a.n_phases)
-                stage_ops(s_ops[buf ^ 1u], a.rops + a.ph_gb[ph + 1], a.ph_gb[ph + 2] - a.ph_gb[ph + 1], threadIdx.x,
-                          blockDim.x);
+                stage_units(s_ops[buf ^ 1u], a.prog + a.ph_pg[ph + 1], a.ph_pg[ph + 2] - a.ph_pg[ph + 1], threadIdx.x,
+                            blockDim.x);
             if (MODE == 2 && ph % (uint32_t)a.ckpt_every == 0) {
                 float2 *dst = const_cast<float2 *>(cache) + (size_t)(ph / (uint32_t)a.ckpt_every) * N;
-                rb_store_linear(v, sm, c, load_packed, dst, t);
+                rb_store_linear(v, sm, c, dst, t, nullptr);
             }
             const uint32_t R = a.ph_R[ph];
             if (R != c.R) remap<MODE != 2>(v, sm, c, R, t);
-            const uint32_t g0 = a.ph_gb[ph];
-            run_gates(v, c, g0, a.ph_gb[ph + 1], s_ops[buf], g0, mats, sm, ubuf, t, ev, ev_end, next);
+            run_prog(v, c, s_ops[buf], s_ops[buf] + (a.ph_pg[ph + 1] - a.ph_pg[ph]), mats, sm, ubuf, t, ev, ev_end,
+                     next, a.evs);
         }
+        // the last checkpoint is the true psi_R, so a trajectory that starts there ends there too
+        const float2 *frame_end = ph0 < a.n_phases ? a.frame + (size_t)(a.n_ckpt - 1) * frame_floats2(t) : nullptr;
         if (MODE == 2) {
-            rb_store_linear(v, sm, c, load_packed, const_cast<float2 *>(cache) + (size_t)(a.n_ckpt - 1) * N,
-                            t);
+            rb_store_linear(v, sm, c, const_cast<float2 *>(cache) + (size_t)(a.n_ckpt - 1) * N, t, frame_end);
         } else if (MODE == 1) {
-            rb_store_linear(v, sm, c, load_packed, static_cast<float2 *>(a.states_out) + (size_t)b * N, t);
+            rb_store_linear(v, sm, c, static_cast<float2 *>(a.states_out) + (size_t)b * N, t, frame_end);
         } else {
-            apply_global_phase(v, c);
+            finish_tile(v, sm, c, frame_end, t);
             const float2 *ref = cache + (size_t)(a.n_ckpt - 1) * N;
             Partial acc = empty_partial();
-            score_registers(acc, a.crit, v, c, ref, [](uint32_t j) { return (uint64_t)j; });
+            score_registers(acc, a.crit, v, c.m, ref, linear_at(t, c.tid, c.m));
             acc = block_reduce_partial(acc, red);
             if (threadIdx.x == 0) {
                 const double sc = finish_score(a.crit, acc);
@@ -1132,65 +1443,44 @@ constexpr int BATCH_THREADS = 256;
 // One batched resident item (see above) run by the whole CTA.
 __device__ __forceinline__ void batch_item(const BatchItem &it, const BatchCircuit &C, const uint64_t *__restrict__ ids,
                                            unsigned char *smem_raw, Partial *red, float2 (*ubuf)[16],
-                                           RegOp (*s_ops)[MAX_PHASE_OPS]) {
+                                           uint4 (*s_ops)[MAX_PHASE_UNITS]) {
     const int t = C.n;
     const uint32_t N = 1u << t, gsize = 1u << (t - REG_BITS), sg = threadIdx.x / gsize;
     float2 *sm = reinterpret_cast<float2 *>(smem_raw) + (size_t)sg * N;
     const bool active = sg < it.count;
     const uint64_t tr = ids[it.off + (active ? sg : 0)];
-    const uint32_t load_packed = 0u | ((uint32_t)(t - 4) << 5) | ((uint32_t)(t - 3) << 10) |
-                                 ((uint32_t)(t - 2) << 15) | ((uint32_t)(t - 1) << 20);
     TileCtx c;
     c.m = 0;
     c.gp = 0;
     c.tid = threadIdx.x % gsize;
     c.nthr = gsize;
-    set_phase(c, load_packed, t);
+    set_phase(c, load_set(t), t);
     Amps v;
-    rb_load_linear(v, C.cache + (size_t)it.ck * N, t, c.tid);
+    load_tile<false>(v, C.cache + (size_t)it.ck * N, linear_at(t, c.tid, 0u));
     const uint32_t *ev = C.keys + C.offsets[tr];
     const uint32_t *ev_end = C.keys + C.offsets[tr + 1];
     uint32_t next = ev < ev_end ? *ev : NO_EVENT;
     const uint32_t ph0 = it.ck * C.ckpt_every;
     if (ph0 < C.n_phases)
-        stage_ops(s_ops[0], C.rops + C.ph_gb[ph0], C.ph_gb[ph0 + 1] - C.ph_gb[ph0], threadIdx.x, BATCH_THREADS);
+        stage_units(s_ops[0], C.prog + C.ph_pg[ph0], C.ph_pg[ph0 + 1] - C.ph_pg[ph0], threadIdx.x, BATCH_THREADS);
     for (uint32_t ph = ph0; ph < C.n_phases; ++ph) {
         const uint32_t buf = (ph - ph0) & 1u;
         stage_wait();
         if (ph + 1 < C.n_phases)
-            stage_ops(s_ops[buf ^ 1u], C.rops + C.ph_gb[ph + 1], C.ph_gb[ph + 2] - C.ph_gb[ph + 1], threadIdx.x,
-                      BATCH_THREADS);
+            stage_units(s_ops[buf ^ 1u], C.prog + C.ph_pg[ph + 1], C.ph_pg[ph + 2] - C.ph_pg[ph + 1], threadIdx.x,
+                        BATCH_THREADS);
         const uint32_t R = C.ph_R[ph];
         if (R != c.R) remap<true>(v, sm, c, R, t);
-        const uint32_t g0 = C.ph_gb[ph];
-        run_gates(v, c, g0, C.ph_gb[ph + 1], s_ops[buf], g0, C.mats, sm, ubuf[sg], t, ev, ev_end, next);
+        run_prog(v, c, s_ops[buf], s_ops[buf] + (C.ph_pg[ph + 1] - C.ph_pg[ph]), C.mats, sm, ubuf[sg], t, ev, ev_end,
+                 next, C.evs);
     }
-    apply_global_phase(v, c);
+    finish_tile(v, sm, c, C.frame + (size_t)(C.n_ckpt - 1) * frame_floats2(t), t);
     const float2 *ref = C.cache + (size_t)(C.n_ckpt - 1) * N;
     Partial acc = empty_partial();
-    score_registers(acc, C.crit, v, c, ref, [](uint32_t j) { return (uint64_t)j; });
-    // per sub-group reduction: warps reduce by shuffles, the sub-group leader combines its warps
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double a2 = __shfl_down_sync(0xffffffffu, acc.a, o);
-        const double b2 = __shfl_down_sync(0xffffffffu, acc.b, o);
-        const double mp = __shfl_down_sync(0xffffffffu, acc.maxp, o);
-        const unsigned long long mi = __shfl_down_sync(0xffffffffu, acc.idx, o);
-        acc.a += a2;
-        acc.b += b2;
-        argmax_merge(acc.maxp, acc.idx, mp, mi);
-    }
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
+    score_registers(acc, C.crit, v, c.m, ref, linear_at(t, c.tid, c.m));
+    acc = group_reduce_partial(acc, red, gsize);
     if (c.tid == 0 && active) {
-        Partial s = empty_partial();
-        const uint32_t w0 = (sg * gsize) >> 5, nw = gsize >> 5;
-        for (uint32_t w = w0; w < w0 + nw; ++w) {
-            s.a += red[w].a;
-            s.b += red[w].b;
-            argmax_merge(s.maxp, s.idx, red[w].maxp, red[w].idx);
-        }
-        const double sc = finish_score(C.crit, s);
+        const double sc = finish_score(C.crit, acc);
         C.score[tr] = sc;
         if (C.pass_flags) C.pass_flags[tr] = sc >= C.crit.threshold;
     }
@@ -1203,7 +1493,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, 2)
     __shared__ uint32_t s_item;
     __shared__ Partial red[BATCH_THREADS / 32];
     __shared__ float2 ubuf[8][16];
-    __shared__ RegOp s_ops[2][MAX_PHASE_OPS];
+    __shared__ uint4 s_ops[2][MAX_PHASE_UNITS];
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) s_item = atomicAdd(counter, 1u);
@@ -1408,7 +1698,7 @@ __device__ __noinline__ void mix_small(const MixSmall &C, const BatchItem &it, c
 
 __device__ __noinline__ void mix_res(const BatchItem &it, const BatchCircuit &C, const uint64_t *__restrict__ ids,
                                     unsigned char *smem_raw, Partial *red, float2 (*ubuf)[16],
-                                    RegOp (*s_ops)[MAX_PHASE_OPS]) {
+                                    uint4 (*s_ops)[MAX_PHASE_UNITS]) {
     batch_item(it, C, ids, smem_raw, red, ubuf, s_ops);
 }
 
@@ -1421,13 +1711,9 @@ struct MixTile {
     uint32_t k, j, tile;
 };
 
-__device__ __forceinline__ uint64_t mix_gidx(const MixStream &S, uint32_t j, uint64_t base, uint32_t jj) {
-    return base + S.passes[j].offs[jj >> S.c] + (jj & ((1u << S.c) - 1u));
-}
-
 __device__ __forceinline__ void mix_tile(const MixArgs &A, const MixStream &S, const MixTile &it,
                                          unsigned char *smem_raw, Partial *red, float2 *ubuf,
-                                         RegOp (*s_ops)[MAX_PHASE_OPS], uint32_t *s_flag) {
+                                         uint4 (*s_ops)[MAX_PHASE_UNITS], uint32_t *s_flag) {
     float2 *sm = reinterpret_cast<float2 *>(smem_raw);
     if (threadIdx.x == 0) {
         const MixTraj &T = S.trajs[it.k];
@@ -1445,16 +1731,9 @@ __device__ __forceinline__ void mix_tile(const MixArgs &A, const MixStream &S, c
         const uint64_t N = 1ull << S.n;
         const bool from_cache = (int)j == T.start;
         const float2 *src = from_cache ? S.cache + (size_t)S.cache_slot[j] * N : S.work + (size_t)T.slot * N;
-        const uint64_t base = tile_base(S.passes[j].rest_mask, it.tile);
-#pragma unroll
-        for (int hi = 0; hi < 16; ++hi) {
-            const uint32_t jj = ((uint32_t)hi << (t - 4)) | (threadIdx.x << 1);
-            const float4 *pa = reinterpret_cast<const float4 *>(src + mix_gidx(S, j, base, jj));
-            // the working slot was written by other CTAs of this launch: read it through L2
-            const float4 w = from_cache ? __ldg(pa) : __ldcg(pa);
-            v.re[hi] = make_float2(w.x, w.z);
-            v.im[hi] = make_float2(w.y, w.w);
-        }
+        // the working slot was written by other CTAs of this launch: read it through L2
+        load_tile<true>(v, src, tile_at((uint32_t)tile_base(S.passes[j].rest_mask, it.tile), S.passes[j].offs, t, S.c,
+                                        threadIdx.x, 0u));
         // this pass's events: binary search for the first key at or after the pass's first gate
         const uint32_t *lo = S.keys + S.offsets[T.tr], *hi_ = S.keys + S.offsets[T.tr + 1];
         ev_end = hi_;
@@ -1471,49 +1750,37 @@ __device__ __forceinline__ void mix_tile(const MixArgs &A, const MixStream &S, c
     c.gp = 0;
     c.tid = threadIdx.x;
     c.nthr = blockDim.x;
-    set_phase(c, 0u | ((uint32_t)(t - 4) << 5) | ((uint32_t)(t - 3) << 10) | ((uint32_t)(t - 2) << 15) |
-                     ((uint32_t)(t - 1) << 20),
-              t);
+    set_phase(c, load_set(t), t);
     uint32_t next = ev < ev_end ? *ev : NO_EVENT;
     {
         const uint32_t pb = S.passes[it.j].pb;
         if (pb < S.passes[it.j].pe)
-            stage_ops(s_ops[0], S.rops + S.ph_gb[pb], S.ph_gb[pb + 1] - S.ph_gb[pb], threadIdx.x, blockDim.x);
+            stage_units(s_ops[0], S.prog + S.ph_pg[pb], S.ph_pg[pb + 1] - S.ph_pg[pb], threadIdx.x, blockDim.x);
     }
     for (uint32_t ph = S.passes[it.j].pb, buf = 0; ph < S.passes[it.j].pe; ++ph, buf ^= 1u) {
         stage_wait();
         if (ph + 1 < S.passes[it.j].pe)
-            stage_ops(s_ops[buf ^ 1u], S.rops + S.ph_gb[ph + 1], S.ph_gb[ph + 2] - S.ph_gb[ph + 1], threadIdx.x,
-                      blockDim.x);
+            stage_units(s_ops[buf ^ 1u], S.prog + S.ph_pg[ph + 1], S.ph_pg[ph + 2] - S.ph_pg[ph + 1], threadIdx.x,
+                        blockDim.x);
         const uint32_t R = S.ph_R[ph];
         if (R != c.R) remap<true>(v, sm, c, R, t);
-        const uint32_t g0 = S.ph_gb[ph];
-        run_gates(v, c, g0, S.ph_gb[ph + 1], s_ops[buf], g0, S.mats, sm, ubuf, t, ev, ev_end, next);
+        run_prog(v, c, s_ops[buf], s_ops[buf] + (S.ph_pg[ph + 1] - S.ph_pg[ph]), S.mats, sm, ubuf, t, ev, ev_end, next,
+                 S.evs);
     }
-    apply_global_phase(v, c);
+    finish_tile(v, sm, c, S.passes[it.j].frame, t);
     const uint32_t k = it.k, j = it.j;
     const MixTraj &T = S.trajs[k];
     const uint64_t N = 1ull << S.n;
-    const uint64_t base = tile_base(S.passes[j].rest_mask, it.tile);
+    const LoadAt at = tile_at((uint32_t)tile_base(S.passes[j].rest_mask, it.tile), S.passes[j].offs, t, S.c, c.tid, c.m);
     const bool scored = (int)j == T.end;
     if (scored) {
         const float2 *ref = S.ref_cache + (size_t)S.cache_slot[j + 1] * N;
         Partial acc = empty_partial();
-        score_registers(acc, S.crit, v, c, ref, [&](uint32_t jj) { return mix_gidx(S, j, base, jj); });
-        acc = block_reduce_partial(acc, red);
+        score_registers(acc, S.crit, v, c.m, ref, at);
+        acc = group_reduce_partial(acc, red, MIX_THREADS);
         if (threadIdx.x == 0) S.partials[(size_t)k * S.tiles + it.tile] = acc;
     } else {
-        const uint32_t load_packed = 0u | ((uint32_t)(t - 4) << 5) | ((uint32_t)(t - 3) << 10) |
-                                     ((uint32_t)(t - 2) << 15) | ((uint32_t)(t - 1) << 20);
-        if (c.R != load_packed) remap(v, sm, c, load_packed, t);
-        float2 *dst = S.work + (size_t)T.slot * N;
-        const uint32_t flip0 = c.m & 1u;
-#pragma unroll
-        for (int hi = 0; hi < 16; ++hi) {
-            const uint32_t jj = (((uint32_t)hi << (t - 4)) | (threadIdx.x << 1)) ^ (c.m & ~1u);
-            const float2 r = flip0 ? swp2(v.re[hi]) : v.re[hi], i = flip0 ? swp2(v.im[hi]) : v.im[hi];
-            reinterpret_cast<float4 *>(dst + mix_gidx(S, j, base, jj))[0] = make_float4(r.x, i.x, r.y, i.y);
-        }
+        store_tile(v, S.work + (size_t)T.slot * N, c.m, at);
     }
     // publish: the barrier orders every thread's stores before thread 0's fence and
     // counter increments (the release the waiting CTAs acquire)
@@ -1550,7 +1817,7 @@ __global__ void __launch_bounds__(MIX_THREADS, 2) mix_kernel(const __grid_consta
     __shared__ double s_val;
     __shared__ Partial red[MIX_THREADS / 32];
     __shared__ float2 ubuf[8][16];
-    __shared__ RegOp s_ops[2][MAX_PHASE_OPS];
+    __shared__ uint4 s_ops[2][MAX_PHASE_UNITS];
     // the current streaming circuit's descriptor: read from shared memory in the phase loop
     // instead of being held in registers (the loop already uses all 128)
     __shared__ MixStream s_stream;
@@ -1611,39 +1878,46 @@ void launch_mix(const MixArgs &a, double bytes, double flops, double smem_bytes,
     ARSO_CUDA(cudaGetLastError());
 }
 
-// Raise the dynamic shared-memory limit of both pass variants once, before any
+// Raise the dynamic shared-memory limit of the pass kernels once, before any
 // launch (and outside stream capture).
+static const auto pass_128 = pass_rb_kernel<128, 5>;  // 96 registers, five CTAs per SM
+static const auto pass_256 = pass_rb_kernel<256, 3>;  // 80 registers, three CTAs per SM
+static const auto pass_512 = pass_rb_kernel<512, 1>;
 void prepare_pass_rb() {
     static bool done = false;
     if (done) return;
-    const int smem = (1 << MAX_TILE_QUBITS) * (int)sizeof(float2) + 2 * (int)TP_IMAGE_BYTES;
-    ARSO_CUDA(cudaFuncSetAttribute(pass_rb_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ARSO_CUDA(cudaFuncSetAttribute(pass_rb_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ARSO_CUDA(cudaFuncSetAttribute(pass_rb_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ARSO_CUDA(cudaFuncSetAttribute(pass_rb_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ARSO_CUDA(cudaFuncSetAttribute(pass_rb_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ARSO_CUDA(cudaFuncSetAttribute(pass_rb_kernel<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const int tile = (1 << MAX_TILE_QUBITS) * (int)sizeof(float2);
+    ARSO_CUDA(cudaFuncSetAttribute(pass_128, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 256));
+    ARSO_CUDA(cudaFuncSetAttribute(pass_256, cudaFuncAttributeMaxDynamicSharedMemorySize, 256 * 256));
+    ARSO_CUDA(cudaFuncSetAttribute(pass_512, cudaFuncAttributeMaxDynamicSharedMemorySize, tile));
+    ARSO_CUDA(cudaFuncSetAttribute(pass_tensor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   tile + 2 * (int)TP_IMAGE_BYTES));
     done = true;
 }
 
+// Tiles of up to 2^12 amplitudes run in 128-thread CTAs (small tiles several side by side),
+// 2^13 in 256 and 2^14 in 512, each compiled for the registers that fill the SM. Measured
+// (device time of all pass launches): 12-qubit tiles, 24-qubit brickwork, 177 trajectories:
+// five 128-thread CTAs 342 ms, four 353, two tiles in a 256-thread CTA 353 (three per SM) or
+// 376 (two); 13-qubit tiles: three CTAs per SM 6.53 ms against 6.87 with two (16-qubit
+// brickwork, 2,000 trajectories) and 3.12 against 3.41 (20-qubit adder, 500).
 void launch_pass_rb(const PassArgs &a, bool last, uint32_t slots, double bytes, cudaStream_t st, double flops,
                     double smem_bytes) {
     ProfScope ps_(last && !a.store_last ? ARSO_K_PASS_LAST : ARSO_K_PASS, bytes, st, flops, smem_bytes);
     prepare_pass_rb();
     const uint32_t tiles = 1u << (a.n - a.t);
-    const int nt = 1 << (a.t - REG_BITS);
-    const size_t smem = (size_t(1) << a.t) * sizeof(float2) + (a.ph_t ? 2 * TP_IMAGE_BYTES : 0);
-    if (a.ph_t) ARSO_REQUIRE(a.t >= 12 && a.t <= MAX_TILE_QUBITS, "tensor phases need 12-14-qubit tiles");
-    dim3 grid(tiles, slots);
+    const uint32_t nt = 1u << (a.t - REG_BITS);
+    const size_t smem = (size_t(1) << a.t) * sizeof(float2);
     if (a.ph_t) {
-        if (last) pass_rb_kernel<true, true><<<grid, nt, smem, st>>>(a);
-        else pass_rb_kernel<false, true><<<grid, nt, smem, st>>>(a);
-    } else if (nt <= 128) {
-        if (last) pass_rb_kernel<true, false, true><<<grid, nt, smem, st>>>(a);
-        else pass_rb_kernel<false, false, true><<<grid, nt, smem, st>>>(a);
+        ARSO_REQUIRE(a.t >= 12 && a.t <= MAX_TILE_QUBITS, "tensor phases need 12-14-qubit tiles");
+        pass_tensor_kernel<<<dim3(tiles, slots), nt, smem + 2 * TP_IMAGE_BYTES, st>>>(a);
+    } else if (nt == 512) {
+        pass_512<<<dim3(tiles, slots), nt, smem, st>>>(a);
+    } else if (nt == 256) {
+        pass_256<<<dim3(tiles, slots), nt, smem, st>>>(a);
     } else {
-        if (last) pass_rb_kernel<true, false><<<grid, nt, smem, st>>>(a);
-        else pass_rb_kernel<false, false><<<grid, nt, smem, st>>>(a);
+        const uint32_t groups = std::min<uint32_t>(tiles, 128 / nt);
+        pass_128<<<dim3(tiles / groups, slots), nt * groups, smem * groups, st>>>(a);
     }
     ARSO_CUDA(cudaGetLastError());
 }

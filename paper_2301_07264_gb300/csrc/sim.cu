@@ -511,14 +511,29 @@ __device__ __forceinline__ void block_sum3(double &x, double &z, double &y, doub
 // qubits after it to out[3 * location]; the segments run in parallel.
 template <typename T>
 __global__ void expect_resident_kernel(const DGate *__restrict__ gates, const T *__restrict__ mats, int n,
-                                       const T *__restrict__ ckpt, const uint32_t *__restrict__ seg_pos,
+                                       const T *__restrict__ ckpt, const float2 *__restrict__ frame,
+                                       const uint32_t *__restrict__ seg_pos,
                                        const uint32_t *__restrict__ first_loc, double *__restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[3][32];
     T *s = reinterpret_cast<T *>(smem_raw);
     const uint32_t N = 1u << n;
     const T *src = ckpt + (size_t)blockIdx.x * N;
-    for (uint32_t i = threadIdx.x; i < N; i += blockDim.x) s[i] = src[i];
+    if (frame) {  // register-blocked circuits: the checkpoint times its frame (internal.h)
+        const uint32_t nt = N >> REG_BITS;
+        const float2 *F = frame + (size_t)blockIdx.x * frame_floats2(n);
+        const float *R = reinterpret_cast<const float *>(F + nt);
+        for (uint32_t i = threadIdx.x; i < N; i += blockDim.x) {
+            const uint32_t k = 4u * (i >> (n - 4)) + (i & 1u);
+            const T x = src[i];
+            T f, r;
+            f.x = F[(i >> 1) & (nt - 1u)].x, f.y = F[(i >> 1) & (nt - 1u)].y;
+            r.x = R[k], r.y = R[k + 2];
+            s[i] = cmul(cmul(f, r), x);
+        }
+    } else {
+        for (uint32_t i = threadIdx.x; i < N; i += blockDim.x) s[i] = src[i];
+    }
     __syncthreads();
     const uint32_t pe = seg_pos[blockIdx.x + 1];
     for (uint32_t pos = seg_pos[blockIdx.x]; pos < pe; ++pos) {
@@ -544,7 +559,7 @@ __global__ void expect_resident_kernel(const DGate *__restrict__ gates, const T 
 }
 
 void launch_expect_resident(const DGate *gates, const void *mats, int n, int precision, const void *ckpt,
-                            const uint32_t *seg_pos, uint32_t n_seg, const uint32_t *first_loc, double *out,
+                            const float2 *frame, const uint32_t *seg_pos, uint32_t n_seg, const uint32_t *first_loc, double *out,
                             cudaStream_t st) {
     if (!n_seg) return;
     const size_t smem = (size_t(1) << n) * (precision == ARSO_C64 ? 8 : 16);
@@ -554,14 +569,14 @@ void launch_expect_resident(const DGate *gates, const void *mats, int n, int pre
             ARSO_CUDA(cudaFuncSetAttribute(expect_resident_kernel<float2>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         expect_resident_kernel<float2><<<n_seg, 512, smem, st>>>(gates, static_cast<const float2 *>(mats), n,
-                                                                 static_cast<const float2 *>(ckpt), seg_pos,
+                                                                 static_cast<const float2 *>(ckpt), frame, seg_pos,
                                                                  first_loc, out);
     } else {
         if (smem > 48 * 1024)
             ARSO_CUDA(cudaFuncSetAttribute(expect_resident_kernel<double2>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         expect_resident_kernel<double2><<<n_seg, 512, smem, st>>>(gates, static_cast<const double2 *>(mats), n,
-                                                                  static_cast<const double2 *>(ckpt), seg_pos,
+                                                                  static_cast<const double2 *>(ckpt), frame, seg_pos,
                                                                   first_loc, out);
     }
     ARSO_CUDA(cudaGetLastError());
