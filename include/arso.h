@@ -95,12 +95,12 @@ typedef struct {
  * g has fidelity <psi_g|P|psi_g>^2 with psi_R, because the rest of the circuit
  * is unitary and maps psi_g to psi_R, so one error-free sweep of Pauli
  * expectations suffices; it keeps the state in one CTA (resident circuits) or in
- * HBM (streaming complex64 circuits, one launch per gate that applies it and
- * measures its qubits).
+ * HBM (streaming complex64 circuits, one launch per fused pass that applies the
+ * pass's gates and measures their qubits on the tile).
  * Outcome probability: the score is |<phi_g|P|psi_g>|^2 with the backward state
  * phi_g = W^dagger |target> for the rest W of the circuit; one backward sweep
  * carries psi and phi from (psi_R, |target>) with the adjoint gates (one CTA,
- * or one HBM launch per gate for streaming complex64 circuits). This flag
+ * or the fused passes over both states for streaming complex64 circuits). This flag
  * simulates the 3L single-error trajectories instead (for comparisons). */
 /* arso_run_batch runs circuits with ARSO_OPT_NO_PERSISTENT on their own
  * launches instead of the batch's persistent launch (for comparisons). */

@@ -338,7 +338,7 @@ def exhaustive(args):
             t0 = time.perf_counter()
             P, per = arso.exhaustive(cc, crit)
             torch.cuda.synchronize()
-            # streaming fidelity sweep: one zero-state launch, then one launch per gate
+            # streaming fidelity sweep: one zero-state launch, then one launch per fused pass
             sweeps = arso.profile_read(arso.K_OTHER).launches - 1
             res[route] = (time.perf_counter() - t0, P, per, sweeps)
         (ts, Ps, pers, sweeps), (tt, Pt, pert, _) = res["sweep"], res["trajectories"]
@@ -353,14 +353,14 @@ def exhaustive(args):
 
 
 def _hbm_sweep(rows):
-    """Streaming (HBM) sweep of brickwork-24: each launch applies one gate with the
-    expectations of its qubits, reading and writing the 2^24-amplitude complex64 state
-    once: 2 * 8 * 2^n bytes per launch."""
+    """Streaming sweep of brickwork-24: each launch applies one fused pass with the
+    measurements of its gates' qubits, reading and writing the 2^24-amplitude complex64
+    state once: 2 * 8 * 2^n bytes per launch."""
     r = next((r for r in rows if r["circuit"] == "brickwork24"), None)
     if r is None:
         return None
     gb = r["sweeps"] * 2 * 8 * (1 << r["n"]) / 1e9
-    return {"kernel": "gate_expect_kernel", "gates": r["G"], "sweeps": r["sweeps"], "algorithmic_GB": gb,
+    return {"kernel": "probe_kernel", "gates": r["G"], "sweeps": r["sweeps"], "algorithmic_GB": gb,
             "achieved_GBps": gb / r["sweep_s"], "note": "whole sweep time, reductions included"}
 
 

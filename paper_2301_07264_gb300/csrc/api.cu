@@ -976,6 +976,57 @@ static McOut mc_run_memo(arso_circuit *c, const DevCrit &dc, double p, uint64_t 
 // circuit maps psi_g to psi_R). Scores in the exhaustive order (X block, Z
 // block, Y block, each in location order). Returns false where the sweep is
 // not available (streaming complex128), leaving the trajectory route.
+// The sums of every slot of c's probe circuit (kernels.h), swept over `state` in place;
+// passes share a launch of the row sum while their rows fit PROBE_BYTES.
+static void run_probes(const arso_circuit *P, bool dual, float2 *state, cudaStream_t st, std::vector<double> &sums) {
+    constexpr size_t PROBE_BYTES = 256ull << 20;
+    const uint32_t per = dual ? PROBE_SUMS_DUAL : PROBE_SUMS, n_pass = (uint32_t)P->passes.size();
+    const uint32_t tiles = 1u << (P->n - P->tile_qubits), n_rows = probe_rows((int)P->tile_qubits, tiles, dual);
+    sums.assign((size_t)per * P->probe_slots.size() + 1, 0.0);
+    Scratch d_sums(st, sums.size() * 8);
+    for (uint32_t j0 = 0; j0 < n_pass;) {
+        uint32_t j1 = j0 + 1;
+        auto len = [&](uint32_t j) { return per * (P->probe_first[j] - P->probe_first[j0]); };
+        while (j1 < n_pass && (size_t)len(j1 + 1) * n_rows * 8 <= PROBE_BYTES) ++j1;
+        const size_t bytes = std::max<size_t>((size_t)len(j1) * n_rows * 8, 8);
+        Scratch rows(st, bytes);
+        ARSO_CUDA(cudaMemsetAsync(rows.ptr, 0, bytes, st));
+        for (uint32_t j = j0; j < j1; ++j) {
+            const PassArgs p = pass_args(P, j);
+            ProbeArgs a{};
+            a.n = p.n, a.t = p.t, a.c = p.c;
+            a.tiles = tiles;
+            a.rest_mask = p.rest_mask;
+            a.offs = p.offs;
+            a.state = state;
+            a.pb = P->passes[j].pb, a.pe = P->passes[j].pe;
+            a.ph_R = P->d_ph_R.as<uint32_t>();
+            a.ph_pg = P->d_ph_pg.as<uint32_t>();
+            a.prog = P->d_prog.as<uint4>();
+            a.mats = P->d_rmats.as<float2>();
+            a.frame = pass_frame(P, j);
+            a.rows = rows.as<double>() + len(j);
+            a.row_len = len(j1);
+            launch_probe(a, dual, st);
+        }
+        launch_probe_sum(rows.as<double>(), n_rows, len(j1), d_sums.as<double>() + (size_t)per * P->probe_first[j0], st);
+        ARSO_CUDA(cudaStreamSynchronize(st));
+        j0 = j1;
+    }
+    copy_d2h(sums.data(), d_sums.ptr, (sums.size() - 1) * 8, st);
+    ARSO_CUDA(cudaStreamSynchronize(st));
+}
+
+static const arso_circuit *probe_of(arso_circuit *c, bool dual) {
+    std::unique_ptr<arso_circuit> &p = dual ? c->probe_dual : c->probe;
+    if (!p) {
+        std::unique_ptr<arso_circuit> q = build_probe(c, dual);
+        upload_circuit(q.get());
+        p = std::move(q);
+    }
+    return p.get();
+}
+
 static bool single_error_fidelities(arso_circuit *c, cudaStream_t st, std::vector<double> &s) {
     const uint64_t L = c->L, G = c->gates.size();
     if (c->engine != 0 && c->precision != ARSO_C64) return false;
@@ -1004,47 +1055,20 @@ static bool single_error_fidelities(arso_circuit *c, cudaStream_t st, std::vecto
             copy_d2h(xyz.data(), d_out.ptr, 3 * L * 8, st);
             ARSO_CUDA(cudaStreamSynchronize(st));
         } else {
-            // complex64 state in HBM: each gate in engine order fused with the expectations
-            // of its qubits on the amplitudes it writes; block partials of up to CH gates at a
-            // time, then one ordered reduction per chunk
-            const int n = (int)c->n;
-            const uint32_t blocks = expect_hbm_blocks(n);
-            const uint64_t CH = 1024;
-            std::vector<uint32_t> loc(G);
-            std::vector<uint8_t> ar(G);
-            for (uint64_t pos = 0; pos < G; ++pos) {
-                loc[pos] = first[c->perm[pos]];
-                ar[pos] = (uint8_t)c->gates[c->perm[pos]].arity;
+            // complex64 state in HBM: the passes of the probe circuit
+            const arso_circuit *P = probe_of(c, false);
+            Scratch psi(st, c->state_bytes());
+            launch_init_zero_state(psi.ptr, (int)c->n, ARSO_C64, st);
+            std::vector<double> v;
+            run_probes(P, false, psi.as<float2>(), st, v);
+            for (size_t k = 0; k < P->probe_slots.size(); ++k) {
+                // a0 = S s0, a1 = S phi s1: conj(a0) a1 = |S|^2 phi conj(s0) s1
+                const ProbeSlot &q = P->probe_slots[k];
+                const std::complex<double> cc = q.s2 * q.phi * std::complex<double>(v[3 * k + 1], v[3 * k + 2]);
+                xyz[3 * q.loc] = 2.0 * cc.real();
+                xyz[3 * q.loc + 1] = q.s2 * v[3 * k];
+                xyz[3 * q.loc + 2] = 2.0 * cc.imag();
             }
-            Scratch psi(st, c->state_bytes()), part(st, CH * blocks * 6 * 8), d_loc(st, G * 4), d_ar(st, G);
-            copy_h2d(d_loc.ptr, loc.data(), G * 4, st);
-            copy_h2d(d_ar.ptr, ar.data(), G, st);
-            launch_init_zero_state(psi.ptr, n, ARSO_C64, st);
-            for (uint64_t c0 = 0; c0 < G; c0 += CH) {
-                const uint64_t c1 = std::min<uint64_t>(G, c0 + CH);
-                for (uint64_t pos = c0; pos < c1; ++pos) {
-                    const HostGate &h = c->gates[c->perm[pos]];
-                    DGate d{};
-                    d.cls = h.cls == GC_H ? (uint8_t)GC_DENSE1
-                          : h.cls == GC_OMEGA ? (uint8_t)GC_DIAG1 : h.cls == GC_CZ ? (uint8_t)GC_DIAG2 : h.cls;
-                    d.arity = (uint8_t)h.arity;
-                    d.q0 = (uint8_t)h.q0;
-                    d.q1 = (uint8_t)h.q1;
-                    M16 m{};
-                    if (h.arity == 1 && d.cls == GC_DIAG1) {
-                        m.m[0] = make_float2((float)h.m[0].real(), (float)h.m[0].imag());
-                        m.m[1] = make_float2((float)h.m[3].real(), (float)h.m[3].imag());
-                    } else if (h.cls != GC_NOP) {
-                        for (int i = 0; i < (h.arity == 1 ? 4 : 16); ++i)
-                            m.m[i] = make_float2((float)h.m[i].real(), (float)h.m[i].imag());
-                    }
-                    launch_gate_expect(psi.as<float2>(), n, d, m, part.as<double>() + (pos - c0) * blocks * 6, st);
-                }
-                launch_gate_expect_reduce(part.as<double>(), (uint32_t)(c1 - c0), blocks, d_loc.as<uint32_t>() + c0,
-                                          d_ar.as<uint8_t>() + c0, d_out.as<double>(), st);
-            }
-            copy_d2h(xyz.data(), d_out.ptr, 3 * L * 8, st);
-            ARSO_CUDA(cudaStreamSynchronize(st));
         }
     }
     s.assign(3 * L, 0.0);
@@ -1068,11 +1092,7 @@ static bool single_error_outcomes(arso_circuit *c, uint64_t target, cudaStream_t
         std::vector<uint32_t> first(G);
         for (uint64_t l = L; l-- > 0;) first[c->loc_gate[l]] = (uint32_t)l;
         std::vector<uint32_t> loc(G);
-        std::vector<uint8_t> ar(G);
-        for (uint64_t pos = 0; pos < G; ++pos) {
-            loc[pos] = first[c->perm[pos]];
-            ar[pos] = (uint8_t)c->gates[c->perm[pos]].arity;
-        }
+        for (uint64_t pos = 0; pos < G; ++pos) loc[pos] = first[c->perm[pos]];
         Scratch d_out(st, 6 * L * 8), d_loc(st, G * 4);
         copy_h2d(d_loc.ptr, loc.data(), G * 4, st);
         if (c->engine == 0) {
@@ -1116,32 +1136,25 @@ static bool single_error_outcomes(arso_circuit *c, uint64_t target, cudaStream_t
                                         ref_state_ptr(c), target, d_loc.as<uint32_t>(), d_out.as<double>(), st);
             ARSO_CUDA(cudaStreamSynchronize(st));  // host tables above are freed on return
         } else {
-            const int n = (int)c->n;
-            const uint32_t blocks = expect_hbm_blocks(n);
-            const uint64_t CH = 512;
-            Scratch psi(st, c->state_bytes()), phi(st, c->state_bytes()), part(st, CH * blocks * 12 * 8), d_ar(st, G);
-            copy_h2d(d_ar.ptr, ar.data(), G, st);
-            ARSO_CUDA(cudaMemcpyAsync(psi.ptr, ref_state_ptr(c), c->state_bytes(), cudaMemcpyDeviceToDevice, st));
-            const float2 one = make_float2(1.f, 0.f);
-            ARSO_CUDA(cudaMemsetAsync(phi.ptr, 0, c->state_bytes(), st));
-            copy_h2d(phi.as<float2>() + target, &one, sizeof(float2), st);
-            // positions in descending chunks [c0, c1), each walked from c1 - 1 down
-            for (uint64_t c1 = G; c1 > 0;) {
-                const uint64_t c0 = c1 > CH ? c1 - CH : 0;
-                for (uint64_t pos = c1; pos-- > c0;) {
-                    DGate d;
-                    M16 m;
-                    hbm_gate(c->gates[c->perm[pos]], true, d, m);
-                    launch_dual_gate_expect(psi.as<float2>(), phi.as<float2>(), n, d, m,
-                                            part.as<double>() + (pos - c0) * blocks * 12, st);
-                }
-                launch_dual_expect_reduce(part.as<double>(), (uint32_t)(c1 - c0), blocks, d_loc.as<uint32_t>() + c0,
-                                          d_ar.as<uint8_t>() + c0, d_out.as<double>(), st);
-                c1 = c0;
+            const arso_circuit *P = probe_of(c, true);
+            Scratch both(st, 2 * c->state_bytes());
+            launch_interleave(static_cast<const float2 *>(ref_state_ptr(c)), target, (int)c->n, both.as<float2>(), st);
+            std::vector<double> v;
+            run_probes(P, true, both.as<float2>(), st, v);
+            for (size_t k = 0; k < P->probe_slots.size(); ++k) {
+                const ProbeSlot &q = P->probe_slots[k];
+                typedef std::complex<double> cd;
+                const cd I(0, 1), c01 = q.s2 * q.phi * cd(v[6 * k], v[6 * k + 1]),
+                         c10 = q.s2 * std::conj(q.phi) * cd(v[6 * k + 2], v[6 * k + 3]),
+                         z = q.s2 * cd(v[6 * k + 4], v[6 * k + 5]);
+                const cd e[3] = {c01 + c10, z, I * (c10 - c01)};  // X, Z, Y of Eq. (2)
+                for (int i = 0; i < 3; ++i) v6[6 * q.loc + 2 * i] = e[i].real(), v6[6 * q.loc + 2 * i + 1] = e[i].imag();
             }
         }
-        copy_d2h(v6.data(), d_out.ptr, 6 * L * 8, st);
-        ARSO_CUDA(cudaStreamSynchronize(st));
+        if (c->engine == 0) {
+            copy_d2h(v6.data(), d_out.ptr, 6 * L * 8, st);
+            ARSO_CUDA(cudaStreamSynchronize(st));
+        }
     }
     s.assign(3 * L, 0.0);
     for (uint64_t l = 0; l < L; ++l)

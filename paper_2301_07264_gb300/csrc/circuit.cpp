@@ -208,7 +208,7 @@ static constexpr uint32_t NO_NEED = 0xFFFFFFFFu;
 
 static uint32_t need_of(const HostGate &h, uint32_t lq0, uint32_t lq1) {
     switch (h.cls) {
-        case GC_DENSE1: case GC_H: return lq0;
+        case GC_DENSE1: case GC_H: case GC_PROBE: return lq0;
         case GC_CX: return lq1;
         default: return NO_NEED;
     }
@@ -516,7 +516,9 @@ static void plan_phases(arso_circuit *c) {
                     }
                     const std::set<uint32_t> now = one;
                     one.clear();
-                    for (uint32_t g : now) emit(g);
+                    for (int probes = 1; probes >= 0; --probes)
+                        for (uint32_t g : now)
+                            if ((c->gates[c->perm[ps.gb + g]].cls == GC_PROBE) == (probes == 1)) emit(g);
                 }
             }
             S.order = ord;
@@ -721,8 +723,19 @@ struct ProgWriter {
     uint32_t active = 0, real = 0, flips = 0, used = 0, end = 0;
     float2 x[REG_BITS];
     std::vector<uint4> czs;          // CZ gates being collected (open is false then)
+    uint32_t probes = 0;             // register positions being measured (open is false and czs empty then)
+    ProbeSlot probe[REG_BITS];
+    std::vector<ProbeSlot> *slots = nullptr;
+    size_t slot0 = 0;                // the pass's first slot
     explicit ProgWriter(std::vector<uint4> &o) : out(o), first(o.size()) {}
     void close() {
+        if (probes) {
+            last = out.size();
+            out.push_back(make_uint4(OP_PROBE | probes << 8 | 1u << 24, end, (uint32_t)(slots->size() - slot0), 0));
+            for (int p = 0; p < REG_BITS; ++p)
+                if (probes >> p & 1) slots->push_back(probe[p]);
+            probes = 0;
+        }
         if (!czs.empty()) {
             last = out.size();
             out.push_back(make_uint4(OP_CZS | (uint32_t)(czs.size() + 1) << 24, end, 0, 0));
@@ -744,12 +757,12 @@ struct ProgWriter {
         }
     }
     void start(uint32_t tile_bit) {  // a layer that has no gate on tile_bit yet
-        if (!czs.empty() || (open && (used >> tile_bit & 1))) close();
+        if (probes || !czs.empty() || (open && (used >> tile_bit & 1))) close();
         if (!open) open = true, active = real = flips = used = 0;
         used |= 1u << tile_bit;
     }
     void nop(uint32_t tile_bit, uint32_t pos) {  // absorbed: only its events are left
-        if (open || !czs.empty()) used |= 1u << tile_bit, end = pos + 1;
+        if (open || !czs.empty() || probes) used |= 1u << tile_bit, end = pos + 1;
         else if (last != SIZE_MAX) out[last].y = pos + 1;
         else start(tile_bit), end = pos + 1;
     }
@@ -769,10 +782,18 @@ struct ProgWriter {
     void cz(uint32_t q0, uint32_t q1, uint32_t p0, uint32_t p1, uint32_t pos) {
         static const uint32_t pat[5] = {0xAAAAAAAAu, 0xCCCCCCCCu, 0xF0F0F0F0u, 0xFF00FF00u, 0xFFFF0000u};
         const uint32_t both = 1u << q0 | 1u << q1;
-        if (open || (!czs.empty() && (used & both))) close();
+        if (open || probes || (!czs.empty() && (used & both))) close();
         if (czs.empty()) used = 0;
         used |= both;
         czs.push_back(make_uint4(p0 < 5 ? pat[p0] : 0u, p1 < 5 ? pat[p1] : 0u, 31 - q0, 31 - q1));
+        end = pos + 1;
+    }
+    void measure(Frame &F, uint32_t tile_bit, uint32_t p, uint32_t loc, uint32_t pos) {
+        if (open || !czs.empty() || (probes && (used >> tile_bit & 1))) close();
+        if (!probes) used = 0;
+        used |= 1u << tile_bit;
+        probes |= 1u << p;
+        probe[p] = {loc, F.phi(tile_bit), std::norm(F.S())};
         end = pos + 1;
     }
     // any other op, after the open layer; `before`: it may precede the open layer
@@ -787,7 +808,7 @@ struct ProgWriter {
         const int k = snap(F.phi(q));
         if (k == 0) return;
         const bool collecting = open || !czs.empty();
-        const bool before = collecting && !(used >> q & 1);
+        const bool before = collecting && !probes && !(used >> q & 1);
         if (!before) close();
         if (k > 0) {
             op(OP_OMEGA | (uint32_t)k << 20, before ? 0 : pos, q | p << 16, nullptr, true);
@@ -856,15 +877,20 @@ static void reg_program(arso_circuit *c) {
     c->frame.clear();
     if (!c->reg_blocked) return;
     if (!c->frames) return tensor_records(c);
+    c->probe_slots.clear();
+    c->probe_first.clear();
     c->evs.resize(2 * c->perm.size());
     for (const Pass &ps : c->passes) {
         std::vector<int> local(c->n, -1);
         for (size_t i = 0; i < ps.tile_qubits.size(); ++i) local[ps.tile_qubits[i]] = (int)i;
         Frame F(c->tile_qubits);
+        c->probe_first.push_back((uint32_t)c->probe_slots.size());
         for (uint32_t ph = ps.pb; ph < ps.pe; ++ph) {
             if (c->engine == 0) c->frame.push_back(F.f);
             c->ph_pg.push_back((uint32_t)c->prog.size());
             ProgWriter W(c->prog);
+            W.slots = &c->probe_slots;
+            W.slot0 = c->probe_first.back();
             for (uint32_t pos = c->ph_gb[ph]; pos < c->ph_gb[ph + 1]; ++pos) {
                 const HostGate &h = c->gates[c->perm[pos]];
                 const uint32_t q0 = (uint32_t)local[h.q0], q1 = (uint32_t)local[h.q1];
@@ -929,6 +955,7 @@ static void reg_program(arso_circuit *c) {
                         break;
                     }
                     case GC_CZ: W.cz(q0, q1, p0, p1, pos); break;
+                    case GC_PROBE: W.measure(F, q0, p0, c->probe_loc[c->perm[pos]], pos); break;
                     default: W.nop(q0, pos); break;
                 }
                 c->evs[2 * pos] = {f2(F.phi(q0)), q0, 0};
@@ -939,6 +966,84 @@ static void reg_program(arso_circuit *c) {
         c->frame.push_back(F.f);  // streaming: the pass's end; resident: the circuit's
     }
     c->ph_pg.push_back((uint32_t)c->prog.size());
+    c->probe_first.push_back((uint32_t)c->probe_slots.size());
+}
+
+// The circuit that the single-error analysis of a streaming complex64 circuit runs: its
+// gates with a measurement of each error location's qubit right after the location's gate.
+// dual: the adjoint gates in reverse order, each after the measurements of its locations,
+// on one more qubit, 0, that no gate touches: it tells psi (0) from phi (1), so their
+// amplitudes are neighbours and the two lanes of every packed register.
+std::unique_ptr<arso_circuit> build_probe(const arso_circuit *c, bool dual) {
+    std::unique_ptr<arso_circuit> P(new arso_circuit());
+    const size_t G = c->gates.size();
+    std::vector<uint32_t> first(G + 1, 0);  // first location of each gate
+    for (size_t g = 0; g < G; ++g) first[g + 1] = first[g] + (uint32_t)c->gates[g].arity;
+    P->n = c->n + (dual ? 1 : 0);
+    P->engine = 1;
+    // the forward circuit's own passes where they are register-blocked
+    const bool own = !dual && c->reg_blocked && !c->tensor;
+    P->tile_qubits = own ? c->tile_qubits : std::min(13u, P->n);
+    P->low_qubits = own ? c->low_qubits : 4u;
+    std::vector<uint32_t> order;  // gate of each position of the passes
+    if (own) {
+        P->passes = c->passes;
+        order = c->perm;
+    } else {
+        arso_circuit T;
+        T.n = P->n;
+        T.tile_qubits = P->tile_qubits;
+        T.low_qubits = P->low_qubits;
+        T.gates.resize(G);
+        for (size_t k = 0; k < G; ++k) {
+            T.gates[k] = c->gates[dual ? G - 1 - k : k];
+            T.gates[k].q0 += dual;
+            T.gates[k].q1 += dual;
+        }
+        schedule_streaming(&T);
+        P->passes = T.passes;
+        for (uint32_t k : T.perm) order.push_back(dual ? (uint32_t)(G - 1 - k) : k);
+    }
+    for (Pass &ps : P->passes) {
+        const uint32_t gb = (uint32_t)P->gates.size();
+        for (uint32_t pos = ps.gb; pos < ps.ge; ++pos) {
+            HostGate h = c->gates[order[pos]];
+            h.q0 += dual;
+            h.q1 += dual;
+            if (dual) {  // adjoint
+                const int dim = h.arity == 1 ? 2 : 4;
+                HostGate a = h;
+                for (int r = 0; r < dim; ++r)
+                    for (int k = 0; k < dim; ++k) a.m[r * dim + k] = std::conj(h.m[k * dim + r]);
+                a.omega_k = (8u - h.omega_k) & 7u;
+                h = a;
+            } else {
+                P->gates.push_back(h);
+                P->probe_loc.push_back(0);
+            }
+            for (int j = 0; j < h.arity; ++j) {
+                HostGate m{};
+                m.arity = 1;
+                m.cls = GC_PROBE;
+                m.q0 = m.q1 = j ? h.q1 : h.q0;
+                P->gates.push_back(m);
+                P->probe_loc.push_back(first[order[pos]] + j);
+            }
+            if (dual) {
+                P->gates.push_back(h);
+                P->probe_loc.push_back(0);
+            }
+        }
+        ps.gb = gb;
+        ps.ge = (uint32_t)P->gates.size();
+    }
+    P->perm.resize(P->gates.size());
+    for (size_t i = 0; i < P->perm.size(); ++i) P->perm[i] = (uint32_t)i;
+    plan_phases(P.get());
+    reg_program(P.get());
+    P->pos_of.assign(P->gates.size(), 0);
+    for (size_t pos = 0; pos < P->perm.size(); ++pos) P->pos_of[P->perm[pos]] = (uint32_t)pos;
+    return P;
 }
 
 // The kernels' table of frame f (internal.h), in the load/store mapping {0, t-4, ..., t-1}.

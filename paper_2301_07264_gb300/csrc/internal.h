@@ -47,6 +47,7 @@ enum GateClass : uint8_t {
     GC_H = 8,       // Hadamard, 1/sqrt2 applied as a two-float constant (unbiased rounding)
     GC_OMEGA = 9,   // diag(1, e^{i k pi/4}), k in DGate::mat; exact for even k, two-float 1/sqrt2 for odd k
     GC_CZ = 10,     // diag(1, 1, 1, -1)
+    GC_PROBE = 12,  // measurement of its qubit in a probe circuit (build_probe), not a gate
     GC_SU2 = 11,    // 2x2 dense of the form [[a, b], [-conj b, conj a]] (register kernels read a and b)
 };
 
@@ -119,6 +120,7 @@ enum RegOpCode : uint32_t {
     OP_PHASE = 83,   // diag(conj f, f)
     OP_LAYER = 84,   // one-qubit gates on distinct qubits (below)
     OP_CZS = 85,     // CZ gates on distinct qubits (below)
+    OP_PROBE = 86,   // measurements on distinct qubits (below); probe circuits only
 };
 
 // Register program of a phase (circuits without tensor phases): macro-ops of 16-byte units.
@@ -134,6 +136,8 @@ enum RegOpCode : uint32_t {
 //           (position 0: (Re x, -Re x, Im x, Im x), the lanes of a packed register)
 //   OP_CZS: one unit for each CZ: the registers whose bit q0, and q1, is 1 as 32-bit masks
 //           (0 for a thread bit), and 31 - q0, 31 - q1
+//   OP_PROBE: bits 8-12 of x the register positions measured, z the first one's slot in
+//           its pass; the slots follow in order of position
 // Frames: the true state is S * prod_q diag(1, phi_q) * X^m * stored, with the scalar S
 // and the unit phases phi_q the same for every trajectory and tracked on the host in FP64
 // from gate to gate (reg_program in circuit.cpp). A unitary U diag(1, phi) equals, up to
@@ -203,6 +207,13 @@ struct Pass {
     double flops_per_amp = 0.0;        // algorithmic FP32 flops per amplitude of one sweep
     uint32_t remaps = 0;               // register-set changes inside the pass (from the load layout)
     uint32_t end_remap = 0;            // 1 if the last phase's set differs from the load layout
+};
+
+// One measurement of a probe circuit, in the order of the passes' slots.
+struct ProbeSlot {
+    uint32_t loc;               // error location
+    std::complex<double> phi;   // frame phase of its qubit
+    double s2;                  // |S|^2
 };
 
 struct Criterion {
@@ -295,6 +306,11 @@ struct arso_circuit {
     arso::DeviceBuffer d_bwd;
     arso::DeviceBuffer d_offs;              // streaming: per pass, tile-high offsets
     std::vector<uint64_t> offs_base;        // per pass offset of its table in d_offs
+    // single-error analysis of a streaming complex64 circuit (build_probe), built on first use
+    std::unique_ptr<arso_circuit> probe, probe_dual;
+    std::vector<arso::ProbeSlot> probe_slots;   // of a probe circuit
+    std::vector<uint32_t> probe_loc;            // of a probe circuit: location of a GC_PROBE gate
+    std::vector<uint32_t> probe_first;          // of a probe circuit: pass -> its first slot (plus a sentinel)
     size_t state_bytes() const { return (size_t(1) << n) * (precision == ARSO_C128 ? 16 : 8); }
 };
 
@@ -313,6 +329,7 @@ namespace arso {
 void matrix_for(const arso_gate &g, HostGate &h);  // h.arity must be set
 std::vector<float> circuit_features(const arso_circuit *c, const arso_criterion *crit);
 void frame_table(const std::vector<std::complex<double>> &f, int t, float2 *out);
+std::unique_ptr<arso_circuit> build_probe(const arso_circuit *c, bool dual);
 void build_circuit(arso_circuit *c, uint32_t n, const arso_gate *gates, size_t n_gates,
                    const arso_compile_opts *opts);
 }  // namespace arso

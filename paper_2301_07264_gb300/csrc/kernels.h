@@ -247,35 +247,47 @@ uint32_t launch_score_partials(const void *psi, const void *ref, int n, int prec
 void launch_init_zero_state(void *psi, int n, int precision, cudaStream_t st);
 // Pauli expectations (<X_q>, <Z_q>, <Y_q>) of the error-free state after each
 // gate: resident circuits run one CTA per cached checkpoint segment
-// (engine positions seg_pos[b] .. seg_pos[b + 1]; out[3 * location + k]), or a
-// complex64 state in HBM (launch_gate_expect below).
+// (engine positions seg_pos[b] .. seg_pos[b + 1]; out[3 * location + k]).
 // frame: the checkpoints' frame tables (register-blocked circuits) or NULL
 void launch_expect_resident(const DGate *gates, const void *mats, int n, int precision, const void *ckpt,
-                            const float2 *frame, const uint32_t *seg_pos, uint32_t n_seg, const uint32_t *first_loc, double *out,
-                            cudaStream_t st);
-uint32_t expect_hbm_blocks(int n);
-// One gate fused with the expectations of its qubits on the updated state; block
-// partials at partials + pos * expect_hbm_blocks(n) * 6 (the caller offsets), added
-// in order by launch_gate_expect_reduce for `count` positions (block k: position k,
-// locations loc[k] .. loc[k] + arity[k] - 1).
-void launch_gate_expect(float2 *psi, int n, const DGate &g, const M16 &m, double *partials, cudaStream_t st);
-void launch_gate_expect_reduce(const double *partials, uint32_t count, uint32_t blocks, const uint32_t *loc,
-                               const uint8_t *arity, double *out3, cudaStream_t st);
+                            const float2 *frame, const uint32_t *seg_pos, uint32_t n_seg, const uint32_t *first_loc,
+                            double *out, cudaStream_t st);
 
-// Backward single-error sweep for rank-1 criteria (outcome probability): psi and
-// phi carried backward from (psi_R, |target>) with the adjoint gates; out6[6 * location
-// + k] = (Re, Im) of <phi|X|psi>, <phi|Z|psi>, <phi|Y|psi> after the location's gate.
-// Resident: one CTA, both states in shared memory, adj[pos] the adjoint gate at
-// engine position pos (global qubits). HBM (complex64): one launch per gate with
-// partials at partials + pos * expect_hbm_blocks(n) * 12 (the caller offsets), added
-// in order by launch_dual_expect_reduce.
+// Backward single-error sweep for rank-1 criteria (outcome probability) of a resident
+// circuit: psi and phi carried backward from (psi_R, |target>) with the adjoint gates;
+// out6[6 * location + k] = (Re, Im) of <phi|X|psi>, <phi|Z|psi>, <phi|Y|psi> after the
+// location's gate. One CTA, both states in shared memory, adj[pos] the adjoint gate at
+// engine position pos (global qubits).
 void launch_dual_expect_resident(const DGate *adj, const void *mats, uint32_t G, int n, int precision,
                                  const void *psi_R, uint64_t target, const uint32_t *first_loc, double *out6,
                                  cudaStream_t st);
-void launch_dual_gate_expect(float2 *psi, float2 *phi, int n, const DGate &g, const M16 &m, double *partials,
-                             cudaStream_t st);
-void launch_dual_expect_reduce(const double *partials, uint32_t count, uint32_t blocks, const uint32_t *loc,
-                               const uint8_t *arity, double *out6, cudaStream_t st);
+
+// Both sweeps of a streaming complex64 circuit, as passes of its probe circuit (build_probe)
+// over one state in place. Every warp adds its sums of the pass's slots, PROBE_SUMS (6 with
+// the dual circuit) values each, to its own row of `rows` (zeroed before); launch_probe_sum
+// adds the rows in order. The raw sums of a measured qubit, per slot, over the pairs (s0, s1)
+// of stored amplitudes along it: |s0|^2 - |s1|^2, Re and Im of conj(s0) s1; dual, with psi in
+// the even and phi in the odd amplitudes: (Re, Im) of conj(f0) s1, of conj(f1) s0, and of
+// conj(f0) s0 - conj(f1) s1.
+constexpr uint32_t PROBE_SUMS = 3, PROBE_SUMS_DUAL = 6;
+struct ProbeArgs {
+    int n, t, c;
+    uint32_t tiles;
+    uint64_t rest_mask;
+    const uint32_t *offs;
+    float2 *state;
+    uint32_t pb, pe;
+    const uint32_t *ph_R, *ph_pg;
+    const uint4 *prog;
+    const float2 *mats, *frame;
+    double *rows;
+    uint32_t row_len;   // doubles per row
+};
+uint32_t probe_rows(int t, uint32_t tiles, bool dual);  // rows of one launch
+void launch_probe(const ProbeArgs &a, bool dual, cudaStream_t st);
+void launch_probe_sum(const double *rows, uint32_t n_rows, uint32_t row_len, double *out, cudaStream_t st);
+// state[2j] = psi[j], state[2j + 1] = (j == target)
+void launch_interleave(const float2 *psi, uint64_t target, int n, float2 *state, cudaStream_t st);
 
 // sampling (sample.cu)
 struct SampleArgs {

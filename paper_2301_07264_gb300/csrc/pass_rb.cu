@@ -679,6 +679,99 @@ __device__ __forceinline__ void apply_op(Amps &a, TileCtx &c, const RegOp &op, c
 #undef ARSO_HADAMARD
 }
 
+// Raw sums (kernels.h) of the pairs along register bit P of this thread's registers.
+template <int P> __device__ __forceinline__ void rg_probe(const Amps &a, uint32_t flip, float *w) {
+    float2 z = make_float2(0.f, 0.f), cr = z, ci = z;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        if (k & (1 << (P - 1))) continue;
+        const int k1 = k | (1 << (P - 1));
+        const float2 r0 = a.re[k], i0 = a.im[k], r1 = a.re[k1], i1 = a.im[k1];
+        const float2 nr1 = make_float2(-r1.x, -r1.y), ni1 = make_float2(-i1.x, -i1.y), ni0 = make_float2(-i0.x, -i0.y);
+        z = fma2(ni1, i1, fma2(nr1, r1, fma2(i0, i0, fma2(r0, r0, z))));
+        cr = fma2(i0, i1, fma2(r0, r1, cr));
+        ci = fma2(ni0, r1, fma2(r0, i1, ci));
+    }
+    const float zs = z.x + z.y, cs = ci.x + ci.y;
+    w[0] = flip ? -zs : zs;  // a flipped qubit: s0 and s1 change places
+    w[1] = cr.x + cr.y;
+    w[2] = flip ? -cs : cs;
+}
+__device__ __forceinline__ void rg_probe_lanes(const Amps &a, uint32_t flip, float *w) {
+    float z = 0.f, cr = 0.f, ci = 0.f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const float2 r = a.re[k], i = a.im[k];
+        z = fmaf(-i.y, i.y, fmaf(-r.y, r.y, fmaf(i.x, i.x, fmaf(r.x, r.x, z))));
+        cr = fmaf(i.x, i.y, fmaf(r.x, r.y, cr));
+        ci = fmaf(-i.x, r.y, fmaf(r.x, i.y, ci));
+    }
+    w[0] = flip ? -z : z;
+    w[1] = cr;
+    w[2] = flip ? -ci : ci;
+}
+// psi in lane 0, phi in lane 1 of every packed register
+template <int P> __device__ __forceinline__ void rg_probe_dual(const Amps &a, uint32_t flip, float *w) {
+    float x[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        if (k & (1 << (P - 1))) continue;
+        const int k1 = k | (1 << (P - 1));
+        const float ar0 = a.re[k].x, ai0 = a.im[k].x, ar1 = a.re[k1].x, ai1 = a.im[k1].x;
+        const float br0 = a.re[k].y, bi0 = a.im[k].y, br1 = a.re[k1].y, bi1 = a.im[k1].y;
+        x[0] = fmaf(bi0, ai1, fmaf(br0, ar1, x[0]));
+        x[1] = fmaf(-bi0, ar1, fmaf(br0, ai1, x[1]));
+        x[2] = fmaf(bi1, ai0, fmaf(br1, ar0, x[2]));
+        x[3] = fmaf(-bi1, ar0, fmaf(br1, ai0, x[3]));
+        x[4] = fmaf(-bi1, ai1, fmaf(-br1, ar1, fmaf(bi0, ai0, fmaf(br0, ar0, x[4]))));
+        x[5] = fmaf(bi1, ar1, fmaf(-br1, ai1, fmaf(-bi0, ar0, fmaf(br0, ai0, x[5]))));
+    }
+    w[0] = flip ? x[2] : x[0];
+    w[1] = flip ? x[3] : x[1];
+    w[2] = flip ? x[0] : x[2];
+    w[3] = flip ? x[1] : x[3];
+    w[4] = flip ? -x[4] : x[4];
+    w[5] = flip ? -x[5] : x[5];
+}
+// The measurements of one OP_PROBE: the values of all positions summed over the warp by
+// halving exchanges (one shuffle per value instead of five), then added to the warp's row,
+// one value per lane (pair of lanes).
+template <bool DUAL> __device__ __forceinline__ void run_probe(const Amps &a, const TileCtx &c, const uint4 h, double *row) {
+    constexpr int SUMS = DUAL ? 6 : 3, N = DUAL ? 32 : 16, P0 = DUAL ? 1 : 0;
+    float w[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) w[i] = 0.f;
+    const uint32_t act = (h.x >> (8 + P0)) & 31u;
+#define ARSO_PROBE_P(P)                                                          \
+    if (h.x & (0x100u << P)) {                                                   \
+        const uint32_t f = (c.m >> rbit(c.R, P)) & 1u;                           \
+        if constexpr (DUAL) rg_probe_dual<P>(a, f, w + SUMS * (P - P0));         \
+        else rg_probe<P>(a, f, w + SUMS * (P - P0));                             \
+    }
+    if constexpr (!DUAL) {
+        if (h.x & 0x100u) rg_probe_lanes(a, (c.m >> rbit(c.R, 0)) & 1u, w);
+    }
+    ARSO_PROBE_P(1) ARSO_PROBE_P(2) ARSO_PROBE_P(3) ARSO_PROBE_P(4)
+#undef ARSO_PROBE_P
+    const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+    for (int o = 16, n = N / 2; n >= 1; o >>= 1, n >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i) {
+            if (i >= n) break;
+            const float send = up ? w[i] : w[i + n], keep = up ? w[i + n] : w[i];
+            w[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    if constexpr (!DUAL) w[0] += __shfl_xor_sync(0xffffffffu, w[0], 1);
+    const uint32_t v = DUAL ? lane : lane >> 1, p = v / SUMS;
+    if (((DUAL || !(lane & 1u))) && ((act >> p) & 1u)) {
+        const uint32_t slot = h.z + __popc(act & ((1u << p) - 1u));
+        atomicAdd(row + slot * SUMS + v - p * SUMS, (double)w[0]);  // its own row: no result is waited for
+    }
+}
+
 // One macro-op of a register program (internal.h): h its header, u its further units.
 __device__ __forceinline__ void apply_macro(Amps &a, TileCtx &c, const uint4 h, const uint4 *u,
                                             const float2 *__restrict__ mats, float2 *sm, float2 *ubuf, int t) {
@@ -1221,6 +1314,101 @@ __global__ void __launch_bounds__(THREADS, MINB) pass_rb_kernel(PassArgs a) {
                  a.evs);
     }
     pass_finish(a, v, c, blockIdx.y, blockIdx.x * groups + sg, gridDim.x * groups, red);
+}
+
+// One pass of a probe circuit (kernels.h) over a state in place: CTAs loop over the tiles,
+// so that each warp keeps one row of sums. Bound by instruction issue: a measurement is 64
+// packed multiply-adds and about 70 instructions of exchange per warp, next to 64 for the
+// gate before it, and a pass reads and writes the state once for some 40 gates. Whole
+// single-error analysis, before (one HBM sweep per gate) and after: 24-qubit brickwork, 1,880
+// locations, 88.7 -> 23.7 ms; 20-qubit adder, both states, 25.4 -> 1.16 ms.
+template <int THREADS, int MINB, bool DUAL>
+__global__ void __launch_bounds__(THREADS, MINB) probe_kernel(ProbeArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float2 *sm = reinterpret_cast<float2 *>(smem_raw);
+    __shared__ float2 ubuf[16];
+    __shared__ uint4 s_ops[2][MAX_PHASE_UNITS];
+    const int t = a.t;
+    double *row = a.rows + ((size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * a.row_len;
+    for (uint32_t tile = blockIdx.x; tile < a.tiles; tile += gridDim.x) {
+        TileCtx c;
+        c.m = 0;
+        c.gp = 0;
+        c.nthr = blockDim.x;
+        c.tid = threadIdx.x;
+        Amps v;
+        load_tile<true>(v, a.state, tile_at((uint32_t)tile_base(a.rest_mask, tile), a.offs, t, a.c, c.tid, 0u));
+        set_phase(c, load_set(t), t);
+        if (a.pb < a.pe)
+            stage_units(s_ops[0], a.prog + a.ph_pg[a.pb], a.ph_pg[a.pb + 1] - a.ph_pg[a.pb], threadIdx.x, blockDim.x);
+        for (uint32_t ph = a.pb; ph <= a.pe; ++ph) {
+            const uint32_t buf = (ph - a.pb) & 1u;
+            stage_wait();
+            if (ph + 1 < a.pe)
+                stage_units(s_ops[buf ^ 1u], a.prog + a.ph_pg[ph + 1], a.ph_pg[ph + 2] - a.ph_pg[ph + 1], threadIdx.x,
+                            blockDim.x);
+            const uint32_t R = ph < a.pe ? a.ph_R[ph] : load_set(t);
+            if (R != c.R) remap<true>(v, sm, c, R, t);
+            if (ph == a.pe) break;
+            const uint4 *u = s_ops[buf], *ue = u + (a.ph_pg[ph + 1] - a.ph_pg[ph]);
+            while (u < ue) {
+                const uint4 h = *u;
+                if ((h.x & 255u) == OP_PROBE) run_probe<DUAL>(v, c, h, row);
+                else apply_macro(v, c, h, u + 1, a.mats, sm, ubuf, t);
+                u += h.x >> 24;
+            }
+        }
+        if (a.frame) apply_frame(v, c, a.frame, t);
+        store_tile(v, a.state, c.m, tile_at((uint32_t)tile_base(a.rest_mask, tile), a.offs, t, a.c, c.tid, c.m));
+        __syncthreads();  // the shared memory is reused by the next tile
+    }
+}
+
+// rows added in a fixed order: a block sums 32 values, eight rows at a time
+__global__ void probe_sum_kernel(const double *__restrict__ rows, uint32_t n_rows, uint32_t row_len, double *out) {
+    __shared__ double red[8][32];
+    const uint32_t v = blockIdx.x * 32 + (threadIdx.x & 31u), g = threadIdx.x >> 5;
+    double x = 0.0;
+    if (v < row_len)
+        for (uint32_t r = g; r < n_rows; r += 8) x += rows[(size_t)r * row_len + v];
+    red[g][threadIdx.x & 31u] = x;
+    __syncthreads();
+    if (g == 0 && v < row_len) {
+        for (int k = 1; k < 8; ++k) x += red[k][threadIdx.x];
+        out[v] = x;
+    }
+}
+
+static const void *probe_fn(int t, bool dual) {
+    if (dual) return t <= 12 ? (const void *)probe_kernel<128, 4, true> : (const void *)probe_kernel<512, 1, true>;
+    return t <= 12 ? (const void *)probe_kernel<128, 4, false> : (const void *)probe_kernel<512, 1, false>;
+}
+static uint32_t probe_grid(int t, uint32_t tiles, bool dual) {
+    const void *fn = probe_fn(t, dual);
+    const int smem = (1 << t) * (int)sizeof(float2);
+    ARSO_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    int per_sm = 1, dev = 0, sms = 152;
+    ARSO_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 1 << (t - REG_BITS), smem));
+    ARSO_CUDA(cudaGetDevice(&dev));
+    ARSO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    return std::min<uint32_t>(tiles, (uint32_t)std::max(per_sm, 1) * (uint32_t)sms);
+}
+uint32_t probe_rows(int t, uint32_t tiles, bool dual) { return probe_grid(t, tiles, dual) * (1u << (t - REG_BITS - 5)); }
+
+void launch_probe(const ProbeArgs &a, bool dual, cudaStream_t st) {
+    ProfScope ps_(ARSO_K_OTHER, 16.0 * (double)(1ull << a.n), st);
+    const uint32_t grid = probe_grid(a.t, a.tiles, dual);
+    ProbeArgs b = a;
+    void *args[] = {&b};
+    ARSO_CUDA(cudaLaunchKernel(probe_fn(a.t, dual), dim3(grid), dim3(1u << (a.t - REG_BITS)), args,
+                               (size_t(1) << a.t) * sizeof(float2), st));
+}
+
+void launch_probe_sum(const double *rows, uint32_t n_rows, uint32_t row_len, double *out, cudaStream_t st) {
+    if (!row_len) return;
+    ProfScope ps_(ARSO_K_REDUCE, 8.0 * (double)n_rows * row_len, st);
+    probe_sum_kernel<<<(row_len + 31) / 32, 256, 0, st>>>(rows, n_rows, row_len, out);
+    ARSO_CUDA(cudaGetLastError());
 }
 
 // The same for circuits with tensor phases: one tile per CTA, gate records instead of the

@@ -582,167 +582,6 @@ void launch_expect_resident(const DGate *gates, const void *mats, int n, int pre
     ARSO_CUDA(cudaGetLastError());
 }
 
-// One gate on a complex64 state in HBM fused with the Pauli expectations of its
-// qubits on the amplitudes it just wrote (the pairs along each of the gate's
-// qubits lie inside the pair or quad a thread updates). Per-thread FP32 sums,
-// FP64 block sums; block b of position `pos` writes partials[(pos * blocks + b) * 6
-// + 3 j + {0, 1, 2}] = (X, Z, Y) terms of the gate's j-th qubit.
-__device__ __forceinline__ void pauli_terms_f(float2 a0, float2 a1, float &x, float &z, float &y) {
-    z += a0.x * a0.x + a0.y * a0.y - a1.x * a1.x - a1.y * a1.y;
-    x += 2.f * (a0.x * a1.x + a0.y * a1.y);
-    y += 2.f * (a0.x * a1.y - a0.y * a1.x);
-}
-
-// apply the one-qubit class to a pair
-__device__ __forceinline__ void gate1(const DGate &g, float2 m0, float2 m1, float2 m2, float2 m3, float2 &a0,
-                                      float2 &a1) {
-    if (g.cls == GC_X) {
-        const float2 t = a0;
-        a0 = a1;
-        a1 = t;
-    } else if (g.cls == GC_DIAG1) {
-        a0 = cmul(m0, a0);
-        a1 = cmul(m1, a1);
-    } else if (g.cls == GC_DENSE1) {
-        const float2 b0 = cmac2(m0, a0, m1, a1), b1 = cmac2(m2, a0, m3, a1);
-        a0 = b0;
-        a1 = b1;
-    }
-}
-
-// apply the two-qubit class to a quad (local index bit(q0) + 2 bit(q1))
-__device__ __forceinline__ void gate2(const DGate &g, const float2 *m16, float2 (&a)[4]) {
-    float2 b[4];
-    if (g.cls == GC_CX) {
-        b[0] = a[0], b[1] = a[3], b[2] = a[2], b[3] = a[1];
-    } else if (g.cls == GC_SWAP) {
-        b[0] = a[0], b[1] = a[2], b[2] = a[1], b[3] = a[3];
-    } else if (g.cls == GC_DIAG2) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) b[k] = cmul(m16[5 * k], a[k]);
-    } else {  // GC_DENSE2
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            float2 acc = cmac2(m16[4 * k], a[0], m16[4 * k + 1], a[1]);
-            const float2 acc2 = cmac2(m16[4 * k + 2], a[2], m16[4 * k + 3], a[3]);
-            acc.x += acc2.x;
-            acc.y += acc2.y;
-            b[k] = acc;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) a[k] = b[k];
-}
-
-// UNROLL pairs (quads) per thread and round: every load of a round is issued before
-// the first store, so that more of them are in flight (the pairs are disjoint)
-constexpr int GE_UNROLL = 4;
-
-__global__ void gate_expect_kernel(float2 *psi, int n, DGate g, M16 mm, double *partials) {
-    __shared__ double red[3][32];
-    const float2 *m16 = mm.m;
-    const float2 m0 = m16[0], m1 = m16[1], m2 = m16[2], m3 = m16[3];
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    const bool write = g.cls != GC_NOP;
-    float x0 = 0.f, z0 = 0.f, y0 = 0.f, x1 = 0.f, z1 = 0.f, y1 = 0.f;
-    if (g.arity == 1) {
-        const uint64_t bit = 1ull << g.q0, lo = bit - 1, half = 1ull << (n - 1);
-        for (uint64_t p0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p0 < half; p0 += GE_UNROLL * stride) {
-            float2 a0[GE_UNROLL], a1[GE_UNROLL];
-            uint64_t i0[GE_UNROLL];
-#pragma unroll
-            for (int u = 0; u < GE_UNROLL; ++u) {
-                const uint64_t p = p0 + u * stride;
-                i0[u] = ((p & ~lo) << 1) | (p & lo);
-                if (p < half) a0[u] = psi[i0[u]], a1[u] = psi[i0[u] | bit];
-            }
-#pragma unroll
-            for (int u = 0; u < GE_UNROLL; ++u) {
-                if (p0 + u * stride >= half) break;
-                gate1(g, m0, m1, m2, m3, a0[u], a1[u]);
-                if (write) psi[i0[u]] = a0[u], psi[i0[u] | bit] = a1[u];
-                pauli_terms_f(a0[u], a1[u], x0, z0, y0);
-            }
-        }
-    } else {
-        const uint32_t lo = g.q0 < g.q1 ? g.q0 : g.q1, hi = g.q0 < g.q1 ? g.q1 : g.q0;
-        const uint64_t b0 = 1ull << g.q0, b1 = 1ull << g.q1, quarter = 1ull << (n - 2);
-        for (uint64_t p0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p0 < quarter; p0 += 2 * stride) {
-            float2 a[2][4];
-            uint64_t base[2];
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                uint64_t i = p0 + u * stride;
-                if (i >= quarter) continue;
-                i = ((i & ~((1ull << lo) - 1)) << 1) | (i & ((1ull << lo) - 1));
-                i = ((i & ~((1ull << hi) - 1)) << 1) | (i & ((1ull << hi) - 1));
-                base[u] = i;
-                a[u][0] = psi[i], a[u][1] = psi[i | b0], a[u][2] = psi[i | b1], a[u][3] = psi[i | b0 | b1];
-            }
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                if (p0 + u * stride >= quarter) break;
-                if (write) {
-                    gate2(g, m16, a[u]);
-                    const uint64_t i = base[u];
-                    psi[i] = a[u][0], psi[i | b0] = a[u][1], psi[i | b1] = a[u][2], psi[i | b0 | b1] = a[u][3];
-                }
-                pauli_terms_f(a[u][0], a[u][1], x0, z0, y0);  // along q0
-                pauli_terms_f(a[u][2], a[u][3], x0, z0, y0);
-                pauli_terms_f(a[u][0], a[u][2], x1, z1, y1);  // along q1
-                pauli_terms_f(a[u][1], a[u][3], x1, z1, y1);
-            }
-        }
-    }
-    double *out = partials + (size_t)blockIdx.x * 6;
-    double x = x0, z = z0, y = y0;
-    block_sum3(x, z, y, red);
-    if (threadIdx.x == 0) out[0] = x, out[1] = z, out[2] = y;
-    if (g.arity == 2) {
-        x = x1, z = z1, y = y1;
-        block_sum3(x, z, y, red);
-        if (threadIdx.x == 0) out[3] = x, out[4] = z, out[5] = y;
-    }
-}
-
-// Adds the block partials of `count` gate positions in a fixed order: block k
-// reduces position k and writes (X, Z, Y) of its qubits to out3[3 * (loc[k] + j)].
-__global__ void gate_expect_reduce_kernel(const double *__restrict__ partials, uint32_t blocks,
-                                          const uint32_t *__restrict__ loc, const uint8_t *__restrict__ arity,
-                                          double *out3) {
-    __shared__ double red[6][256];
-    const double *p = partials + (size_t)blockIdx.x * blocks * 6;
-    double v[6] = {0, 0, 0, 0, 0, 0};
-    for (uint32_t b = threadIdx.x; b < blocks; b += blockDim.x)
-#pragma unroll
-        for (int k = 0; k < 6; ++k) v[k] += p[(size_t)b * 6 + k];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) red[k][threadIdx.x] = v[k];
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o)
-#pragma unroll
-            for (int k = 0; k < 6; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x < 3u * arity[blockIdx.x]) out3[3 * (size_t)loc[blockIdx.x] + threadIdx.x] = red[threadIdx.x][0];
-}
-
-void launch_gate_expect(float2 *psi, int n, const DGate &g, const M16 &m, double *partials, cudaStream_t st) {
-    const uint32_t blocks = expect_hbm_blocks(n);
-    ProfScope ps_(ARSO_K_OTHER, 16.0 * (double)(1ull << n), st);
-    gate_expect_kernel<<<blocks, 256, 0, st>>>(psi, n, g, m, partials);
-    ARSO_CUDA(cudaGetLastError());
-}
-
-void launch_gate_expect_reduce(const double *partials, uint32_t count, uint32_t blocks, const uint32_t *loc,
-                               const uint8_t *arity, double *out3, cudaStream_t st) {
-    if (!count) return;
-    ProfScope ps_(ARSO_K_REDUCE, 48.0 * count * blocks, st);
-    gate_expect_reduce_kernel<<<count, 256, 0, st>>>(partials, blocks, loc, arity, out3);
-    ARSO_CUDA(cudaGetLastError());
-}
-
 // ------------------------------------------- single-error outcome values ---
 // For a rank-1 criterion |<tau|psi>|^2 (outcome probability: tau = |t>) the final
 // state with one Pauli error P on qubit q after gate g scores |<phi_g|P|psi_g>|^2,
@@ -857,111 +696,17 @@ void launch_dual_expect_resident(const DGate *adj, const void *mats, uint32_t G,
     ARSO_CUDA(cudaGetLastError());
 }
 
-// The same backward step on complex64 states in HBM, one launch per gate: each
-// thread takes the cross terms of its pairs (quads) before undoing the gate on
-// them. Per-thread FP32 sums, FP64 block partials: block b of a position writes
-// partials[b * 12 + 6 j + k] for the gate's j-th qubit.
-__global__ void dual_gate_expect_kernel(float2 *psi, float2 *phi, int n, DGate g, M16 mm, double *partials) {
-    __shared__ double red[6][32];
-    const float2 *m16 = mm.m;
-    const float2 m0 = m16[0], m1 = m16[1], m2 = m16[2], m3 = m16[3];
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    const bool write = g.cls != GC_NOP;
-    float c0[6] = {0, 0, 0, 0, 0, 0}, c1[6] = {0, 0, 0, 0, 0, 0};
-    if (g.arity == 1) {
-        const uint64_t bit = 1ull << g.q0, lo = bit - 1, half = 1ull << (n - 1);
-        for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < half; p += stride) {
-            const uint64_t i0 = ((p & ~lo) << 1) | (p & lo), i1 = i0 | bit;
-            float2 a0 = psi[i0], a1 = psi[i1], b0 = phi[i0], b1 = phi[i1];
-            cross_terms(a0, a1, b0, b1, c0);
-            if (write) {
-                gate1(g, m0, m1, m2, m3, a0, a1);
-                gate1(g, m0, m1, m2, m3, b0, b1);
-                psi[i0] = a0, psi[i1] = a1, phi[i0] = b0, phi[i1] = b1;
-            }
-        }
-    } else {
-        const uint32_t lo = g.q0 < g.q1 ? g.q0 : g.q1, hi = g.q0 < g.q1 ? g.q1 : g.q0;
-        const uint64_t b0 = 1ull << g.q0, b1 = 1ull << g.q1, quarter = 1ull << (n - 2);
-        for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < quarter; p += stride) {
-            uint64_t i = p;
-            i = ((i & ~((1ull << lo) - 1)) << 1) | (i & ((1ull << lo) - 1));
-            i = ((i & ~((1ull << hi) - 1)) << 1) | (i & ((1ull << hi) - 1));
-            const uint64_t idx[4] = {i, i | b0, i | b1, i | b0 | b1};
-            float2 a[4], b[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) a[k] = psi[idx[k]], b[k] = phi[idx[k]];
-            cross_terms(a[0], a[1], b[0], b[1], c0);  // along q0
-            cross_terms(a[2], a[3], b[2], b[3], c0);
-            cross_terms(a[0], a[2], b[0], b[2], c1);  // along q1
-            cross_terms(a[1], a[3], b[1], b[3], c1);
-            if (write) {
-                gate2(g, m16, a);
-                gate2(g, m16, b);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) psi[idx[k]] = a[k], phi[idx[k]] = b[k];
-            }
-        }
-    }
-    double v[6];
-    double *out = partials + (size_t)blockIdx.x * 12;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) v[k] = c0[k];
-    block_sum6(v, red);
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int k = 0; k < 6; ++k) out[k] = v[k];
-    if (g.arity == 2) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) v[k] = c1[k];
-        block_sum6(v, red);
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int k = 0; k < 6; ++k) out[6 + k] = v[k];
-    }
+__global__ void interleave_kernel(const float2 *__restrict__ psi, uint64_t target, uint64_t N, float4 *state) {
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < N; i += (uint64_t)gridDim.x * blockDim.x)
+        state[i] = make_float4(psi[i].x, psi[i].y, i == target ? 1.f : 0.f, 0.f);
 }
 
-// Adds the block partials of `count` positions in a fixed order: block k reduces
-// position k and writes its qubits' six sums to out6[6 * (loc[k] + j)].
-__global__ void dual_expect_reduce_kernel(const double *__restrict__ partials, uint32_t blocks,
-                                          const uint32_t *__restrict__ loc, const uint8_t *__restrict__ arity,
-                                          double *out6) {
-    __shared__ double red[12][128];
-    const double *p = partials + (size_t)blockIdx.x * blocks * 12;
-    double v[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (uint32_t b = threadIdx.x; b < blocks; b += blockDim.x)
-#pragma unroll
-        for (int k = 0; k < 12; ++k) v[k] += p[(size_t)b * 12 + k];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) red[k][threadIdx.x] = v[k];
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o)
-#pragma unroll
-            for (int k = 0; k < 12; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x < 6u * arity[blockIdx.x]) out6[6 * (size_t)loc[blockIdx.x] + threadIdx.x] = red[threadIdx.x][0];
-}
-
-void launch_dual_gate_expect(float2 *psi, float2 *phi, int n, const DGate &g, const M16 &m, double *partials,
-                             cudaStream_t st) {
-    const uint32_t blocks = expect_hbm_blocks(n);
-    ProfScope ps_(ARSO_K_OTHER, 32.0 * (double)(1ull << n), st);
-    dual_gate_expect_kernel<<<blocks, 256, 0, st>>>(psi, phi, n, g, m, partials);
+void launch_interleave(const float2 *psi, uint64_t target, int n, float2 *state, cudaStream_t st) {
+    const uint64_t N = 1ull << n;
+    ProfScope ps_(ARSO_K_OTHER, 24.0 * (double)N, st);
+    interleave_kernel<<<(unsigned)std::min<uint64_t>((N + 255) / 256, 152ull * 16), 256, 0, st>>>(
+        psi, target, N, reinterpret_cast<float4 *>(state));
     ARSO_CUDA(cudaGetLastError());
-}
-
-void launch_dual_expect_reduce(const double *partials, uint32_t count, uint32_t blocks, const uint32_t *loc,
-                               const uint8_t *arity, double *out6, cudaStream_t st) {
-    if (!count) return;
-    ProfScope ps_(ARSO_K_REDUCE, 96.0 * count * blocks, st);
-    dual_expect_reduce_kernel<<<count, 128, 0, st>>>(partials, blocks, loc, arity, out6);
-    ARSO_CUDA(cudaGetLastError());
-}
-
-uint32_t expect_hbm_blocks(int n) {
-    return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(((1ull << (n - 1)) + 255) / 256, 152ull * 8));
 }
 
 }  // namespace arso
