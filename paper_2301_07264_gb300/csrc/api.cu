@@ -47,7 +47,7 @@ struct Scratch {
     void *ptr = nullptr;
     cudaStream_t st;
     explicit Scratch(cudaStream_t s, size_t bytes) : st(s) {
-        if (bytes) ARSO_CUDA(cudaMallocAsync(&ptr, bytes, st));
+        if (bytes) ptr = pool_alloc(bytes, st);
     }
     ~Scratch() {
         if (ptr) cudaFreeAsync(ptr, st);
@@ -400,7 +400,7 @@ static bool suffix_wanted(const arso_circuit *c, const DCrit &crit) {
 struct DevCrit {
     DCrit d{};
     uint32_t aggregate = 0;
-    DeviceBuffer bitmap;
+    ListBuffer bitmap;
 };
 
 static void make_crit(const arso_circuit *c, const arso_criterion *crit, DevCrit &out, cudaStream_t st) {
@@ -422,7 +422,7 @@ static void make_crit(const arso_circuit *c, const arso_criterion *crit, DevCrit
             ARSO_REQUIRE(crit->set[i] < N, "binning outcome out of range");
             bm[crit->set[i] >> 5] |= 1u << (crit->set[i] & 31);
         }
-        out.bitmap.ensure(bm.size() * 4);
+        out.bitmap.ensure(bm.size() * 4, st);
         copy_h2d(out.bitmap.ptr, bm.data(), bm.size() * 4, st);
         ARSO_CUDA(cudaStreamSynchronize(st));
         out.d.bitmap = out.bitmap.as<uint32_t>();
@@ -560,6 +560,17 @@ static void run_streaming(arso_circuit *c, const arso_error_list *e, const std::
     const bool use_graphs = !states_out && c->reg_blocked && !(c->flags & ARSO_OPT_NO_GRAPHS) && st != nullptr &&
                             st != cudaStreamLegacy && st != cudaStreamPerThread;
     if (use_graphs) prepare_pass_rb();
+    // a sequence is worth capturing when a later batch replays it: capturing and instantiating
+    // takes longer than launching the passes once
+    std::map<GraphKey, uint32_t> uses;
+    if (use_graphs)
+        for (size_t b0 = 0; b0 < ids.size(); b0 += B) {
+            const size_t nb = std::min<size_t>(B, ids.size() - b0);
+            GraphKey k{(int)P, 0, (uint32_t)nb};
+            for (size_t i = b0; i < b0 + nb; ++i)
+                k.jmin = std::min(k.jmin, start[order[i]]), k.jmax = std::max(k.jmax, end[order[i]]);
+            ++uses[k];
+        }
     for (size_t b0 = 0; b0 < ids.size(); b0 += B) {
         const size_t nb = std::min<size_t>(B, ids.size() - b0);
         std::vector<uint64_t> st_traj(nb);
@@ -597,7 +608,7 @@ static void run_streaming(arso_circuit *c, const arso_error_list *e, const std::
             ARSO_CUDA(cudaStreamSynchronize(st));
             continue;
         }
-        CaptureGuard capture(st, use_graphs);
+        CaptureGuard capture(st, use_graphs && uses[key] > 1);
         for (uint32_t j = (uint32_t)jmin; j <= (uint32_t)jmax; ++j) {
             PassArgs a = pass_args(c, j);
             a.cache = c->d_cache.ptr;
@@ -669,13 +680,13 @@ static void run_all(arso_circuit *c, const arso_error_list *e, const DevCrit &dc
 }
 
 // ------------------------------------------------------------ sampling -----
-static arso_error_list *new_list(const arso_circuit *c, uint64_t n_traj) {
-    auto *e = new arso_error_list();
+static std::unique_ptr<arso_error_list> new_list(const arso_circuit *c, uint64_t n_traj, cudaStream_t st) {
+    std::unique_ptr<arso_error_list> e(new arso_error_list());
     e->circ = c;
     e->n_traj = n_traj;
-    e->d_offsets.ensure((n_traj + 1) * 8);
-    e->d_first.ensure(std::max<uint64_t>(n_traj, 1) * 4);
-    e->d_last.ensure(std::max<uint64_t>(n_traj, 1) * 4);
+    e->d_offsets.ensure((n_traj + 1) * 8, st);
+    e->d_first.ensure(std::max<uint64_t>(n_traj, 1) * 4, st);
+    e->d_last.ensure(std::max<uint64_t>(n_traj, 1) * 4, st);
     return e;
 }
 
@@ -694,7 +705,8 @@ static void sample(const arso_circuit *c, double px, double pz, double py, uint6
     const double pt = px + pz + py;
     ARSO_REQUIRE(pt <= 1.0, "p_x + p_z + p_y must be <= 1");
     ARSO_REQUIRE(begin + n_traj >= begin, "trajectory range overflows");
-    std::unique_ptr<arso_error_list> e(new_list(c, n_traj));
+    std::unique_ptr<arso_error_list> e = new_list(c, n_traj, st);
+    SyncOnFail wait(st);
     SampleArgs a{};
     a.seed = seed;
     a.traj_begin = begin;
@@ -720,11 +732,12 @@ static void sample(const arso_circuit *c, double px, double pz, double py, uint6
     copy_d2h(&total, e->d_offsets.as<uint64_t>() + n_traj, 8, st);
     ARSO_CUDA(cudaStreamSynchronize(st));
     e->n_events = total;
-    e->d_loc.ensure(std::max<uint64_t>(total, 1) * 4);
-    e->d_key.ensure(std::max<uint64_t>(total, 1) * 4);
+    e->d_loc.ensure(std::max<uint64_t>(total, 1) * 4, st);
+    e->d_key.ensure(std::max<uint64_t>(total, 1) * 4, st);
     if (total) launch_sample_fill(a, e->d_offsets.as<uint64_t>(), c->d_loc_key.as<uint32_t>(), e->d_loc.as<uint32_t>(),
                                   e->d_key.as<uint32_t>(), st);
     finish_list(c, e.get(), st);
+    wait.done = true;
     *out = e.release();
 }
 
@@ -756,6 +769,7 @@ static void sample_batch(size_t count, const arso_circuit *const *circuits, cons
                          const double *py, const uint64_t *seeds, const uint64_t *begins, const uint64_t *n_traj,
                          cudaStream_t st, arso_error_list **out) {
     std::vector<std::unique_ptr<arso_error_list>> lists(count);
+    SyncOnFail wait(st);
     std::vector<SampleJob> jobs(count);
     uint64_t total = 0;
     for (size_t i = 0; i < count; ++i) {
@@ -763,7 +777,7 @@ static void sample_batch(size_t count, const arso_circuit *const *circuits, cons
         ARSO_REQUIRE(c != nullptr, "NULL circuit");
         SampleJob &J = jobs[i];
         J.a = sample_args(c, px[i], pz[i], py[i], seeds[i], begins[i], n_traj[i]);
-        lists[i].reset(new_list(c, n_traj[i]));
+        lists[i] = new_list(c, n_traj[i], st);
         J.traj0 = total;
         total += n_traj[i];
         J.offsets = lists[i]->d_offsets.as<uint64_t>();
@@ -786,8 +800,8 @@ static void sample_batch(size_t count, const arso_circuit *const *circuits, cons
         bool any = false;
         for (size_t i = 0; i < count; ++i) {
             lists[i]->n_events = ev[i];
-            lists[i]->d_loc.ensure(std::max<uint64_t>(ev[i], 1) * 4);
-            lists[i]->d_key.ensure(std::max<uint64_t>(ev[i], 1) * 4);
+            lists[i]->d_loc.ensure(std::max<uint64_t>(ev[i], 1) * 4, st);
+            lists[i]->d_key.ensure(std::max<uint64_t>(ev[i], 1) * 4, st);
             jobs[i].ev_loc = lists[i]->d_loc.as<uint32_t>();
             jobs[i].ev_key = lists[i]->d_key.as<uint32_t>();
             any |= ev[i] > 0;
@@ -796,6 +810,7 @@ static void sample_batch(size_t count, const arso_circuit *const *circuits, cons
         launch_sample_batch_fill(d_jobs.as<SampleJob>(), (uint32_t)count, total, any, st);
         ARSO_CUDA(cudaStreamSynchronize(st));
     }
+    wait.done = true;
     for (size_t i = 0; i < count; ++i) out[i] = lists[i].release();
 }
 
@@ -814,16 +829,18 @@ static void list_from_host(const arso_circuit *c, uint64_t n_traj, const uint64_
     }
     const uint64_t total = offsets[n_traj];
     ARSO_REQUIRE(total == 0 || events != nullptr, "events is NULL");
-    std::unique_ptr<arso_error_list> e(new_list(c, n_traj));
+    std::unique_ptr<arso_error_list> e = new_list(c, n_traj, st);
+    SyncOnFail wait(st);
     e->n_events = total;
-    e->d_loc.ensure(std::max<uint64_t>(total, 1) * 4);
-    e->d_key.ensure(std::max<uint64_t>(total, 1) * 4);
+    e->d_loc.ensure(std::max<uint64_t>(total, 1) * 4, st);
+    e->d_key.ensure(std::max<uint64_t>(total, 1) * 4, st);
     copy_h2d(e->d_offsets.ptr, offsets, (n_traj + 1) * 8, st);
     if (total) {
         copy_h2d(e->d_loc.ptr, events, total * 4, st);
         launch_keys_from_loc(e->d_loc.as<uint32_t>(), total, c->d_loc_key.as<uint32_t>(), e->d_key.as<uint32_t>(), st);
     }
     finish_list(c, e.get(), st);
+    wait.done = true;
     *out = e.release();
 }
 
@@ -1632,11 +1649,16 @@ arso_status arso_compile_circuit(uint32_t n_qubits, const arso_gate *gates, size
         std::unique_ptr<arso_circuit> c(new arso_circuit());
         build_circuit(c.get(), n_qubits, gates, n_gates, opts);
         upload_circuit(c.get());
+        handle_made();
         *out = c.release();
     });
 }
 
-void arso_circuit_free(arso_circuit *c) { delete c; }
+void arso_circuit_free(arso_circuit *c) {
+    if (!c) return;
+    delete c;
+    handle_freed();
+}
 
 arso_status arso_plan_phases(uint32_t n_qubits, const arso_gate *gates, size_t n_gates,
                              const arso_compile_opts *opts, uint32_t *n_phases, uint32_t *n_tensor) {

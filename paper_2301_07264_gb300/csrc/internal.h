@@ -223,6 +223,17 @@ struct Criterion {
     std::vector<uint64_t> set;
 };
 
+// pool.cpp: memory of the library's pool. pool_alloc: usable on `st` from there on;
+// pool_alloc_now: usable on any stream after the call; pool_free_idle: no work that uses
+// the memory may be pending.
+void *pool_alloc(size_t bytes, cudaStream_t st);
+void *pool_alloc_now(size_t bytes);
+void pool_free_idle(void *ptr) noexcept;
+// circuits and surrogates alive: with the last one freed the pool's memory goes back
+void handle_made();
+void handle_freed() noexcept;
+
+// Memory of a handle, used on any stream.
 struct DeviceBuffer {
     void *ptr = nullptr;
     size_t bytes = 0;
@@ -231,17 +242,67 @@ struct DeviceBuffer {
     DeviceBuffer &operator=(const DeviceBuffer &) = delete;
     ~DeviceBuffer() { release(); }
     void release() {
-        if (ptr) cudaFree(ptr);
+        if (ptr) {
+            cudaDeviceSynchronize();  // kernels of any stream may still use it (as cudaFree waits for them)
+            pool_free_idle(ptr);
+        }
         ptr = nullptr;
         bytes = 0;
     }
     void ensure(size_t b) {
         if (b <= bytes) return;
         release();
-        ARSO_CUDA(cudaMalloc(&ptr, b));
+        ptr = pool_alloc_now(b);
         bytes = b;
     }
     template <typename T> T *as() const { return static_cast<T *>(ptr); }
+};
+
+// Memory that only calls which wait for their own work use (error lists, criteria): freed
+// without waiting. A call that fails half-way waits before its buffers go (SyncOnFail).
+struct ListBuffer {
+    void *ptr = nullptr;
+    size_t bytes = 0;
+    ListBuffer() = default;
+    ListBuffer(const ListBuffer &) = delete;
+    ListBuffer &operator=(const ListBuffer &) = delete;
+    ~ListBuffer() { pool_free_idle(ptr); }
+    void ensure(size_t b, cudaStream_t st) {  // once; usable on st
+        if (ptr) throw Error(ARSO_EINVAL, "internal: a list buffer is allocated once");
+        ptr = pool_alloc(b, st);
+        bytes = b;
+    }
+    template <typename T> T *as() const { return static_cast<T *>(ptr); }
+};
+// Working memory of one call on one stream, which frees and reuses it in order.
+struct StreamBuffer {
+    void *ptr = nullptr;
+    size_t bytes = 0;
+    cudaStream_t st;
+    explicit StreamBuffer(cudaStream_t s) : st(s) {}
+    StreamBuffer(const StreamBuffer &) = delete;
+    StreamBuffer &operator=(const StreamBuffer &) = delete;
+    ~StreamBuffer() { release(); }
+    void release() {
+        if (ptr) cudaFreeAsync(ptr, st);
+        ptr = nullptr;
+        bytes = 0;
+    }
+    void ensure(size_t b) {
+        if (b <= bytes) return;
+        release();
+        ptr = pool_alloc(b, st);
+        bytes = b;
+    }
+    template <typename T> T *as() const { return static_cast<T *>(ptr); }
+};
+struct SyncOnFail {
+    cudaStream_t st;
+    bool done = false;
+    explicit SyncOnFail(cudaStream_t s) : st(s) {}
+    ~SyncOnFail() {
+        if (!done) cudaStreamSynchronize(st);
+    }
 };
 
 }  // namespace arso
@@ -317,11 +378,11 @@ struct arso_circuit {
 struct arso_error_list {
     const arso_circuit *circ = nullptr;
     uint64_t n_traj = 0, n_events = 0;
-    arso::DeviceBuffer d_offsets;  // uint64[n_traj + 1]
-    arso::DeviceBuffer d_loc;      // uint32 (loc << 2) | code, location order
-    arso::DeviceBuffer d_key;      // uint32 engine-order keys
-    arso::DeviceBuffer d_first;    // uint32 per trajectory: first engine position with an event, or NO_EVENT
-    arso::DeviceBuffer d_last;     // uint32 per trajectory: last engine position with an event, or NO_EVENT
+    arso::ListBuffer d_offsets;  // uint64[n_traj + 1]
+    arso::ListBuffer d_loc;      // uint32 (loc << 2) | code, location order
+    arso::ListBuffer d_key;      // uint32 engine-order keys
+    arso::ListBuffer d_first;    // uint32 per trajectory: first engine position with an event, or NO_EVENT
+    arso::ListBuffer d_last;     // uint32 per trajectory: last engine position with an event, or NO_EVENT
 };
 
 namespace arso {

@@ -397,7 +397,7 @@ static std::atomic<bool> g_stall_next_gemm{false};
 // the chunks in order (grad_finish_kernel). Returns the number of chunks.
 static int umma_gemm(int M, int N, int K, GemmOperand A, GemmOperand B, float *C, long ldc, int epi,
                      const __nv_bfloat16 *bias, const float *mask, long ldm, const __nv_bfloat16 *w3, float *z,
-                     float *colsum, DeviceBuffer *part, cudaStream_t st) {
+                     float *colsum, StreamBuffer *part, cudaStream_t st) {
     static uint64_t attr_set = 0;  // one bit per device
     int dev = 0;
     ARSO_CUDA(cudaGetDevice(&dev));
@@ -617,9 +617,11 @@ struct arso_surrogate {
 namespace arso {
 
 struct Activations {
-    DeviceBuffer xb, h1, h2, z, dz, dh1, dh2, lsum;
-    DeviceBuffer pw1, pb1, pw2, pb2, pw3, pb3;  // gradient partials, summed by grad_finish_kernel
+    StreamBuffer xb, h1, h2, z, dz, dh1, dh2, lsum;
+    StreamBuffer pw1, pb1, pw2, pb2, pw3, pb3;  // gradient partials, summed by grad_finish_kernel
     int cap = 0;
+    explicit Activations(cudaStream_t s)
+        : xb(s), h1(s), h2(s), z(s), dz(s), dh1(s), dh2(s), lsum(s), pw1(s), pb1(s), pw2(s), pb2(s), pw3(s), pb3(s) {}
     void ensure(int rows) {
         if (rows <= cap) return;
         xb.ensure((size_t)rows * IN * 4);
@@ -740,7 +742,7 @@ static void refresh_bf16(arso_surrogate *s, cudaStream_t st) {
 
 static void ensure_norm(arso_surrogate *s, const float *x, uint64_t n, cudaStream_t st) {
     if (s->norm_set) return;
-    DeviceBuffer mom;
+    StreamBuffer mom(st);
     mom.ensure(2 * IN * sizeof(double));
     {
         ProfScope ps_(ARSO_K_REDUCE, (double)n * IN * 4, st);
@@ -795,6 +797,7 @@ arso_status arso_surrogate_create(uint64_t seed, arso_surrogate **out) {
         upload_norm(s.get());
         refresh_bf16(s.get(), 0);
         ARSO_CUDA(cudaDeviceSynchronize());
+        handle_made();
         *out = s.release();
         return ARSO_OK;
     } catch (const Error &e) {
@@ -803,7 +806,11 @@ arso_status arso_surrogate_create(uint64_t seed, arso_surrogate **out) {
     }
 }
 
-void arso_surrogate_free(arso_surrogate *s) { delete s; }
+void arso_surrogate_free(arso_surrogate *s) {
+    if (!s) return;
+    delete s;
+    handle_freed();
+}
 
 arso_status arso_surrogate_set_norm(arso_surrogate *s, const float *mean, const float *stdev) {
     try {
@@ -852,13 +859,13 @@ arso_status arso_surrogate_grads(const arso_surrogate *s, const float *x, const 
         ARSO_REQUIRE(s && x && y && grads_out, "NULL argument");
         ARSO_REQUIRE(n > 0 && n <= (1u << 20), "n must be in [1, 2^20]");
         cudaStream_t st = (cudaStream_t)stream;
-        Activations a;
+        Activations a(st);
         a.ensure((int)n);
         gather(x, nullptr, 0, (int)n, s, a, st);
         mlp_forward(s, a, (int)n, true, st);
         ARSO_CUDA(cudaMemsetAsync(a.lsum.ptr, 0, 8, st));
         bce(s, a, y, nullptr, 0, (int)n, st);
-        DeviceBuffer g;
+        StreamBuffer g(st);
         g.ensure(N_PARAMS * 4);
         mlp_backward(s, a, (int)n, g.as<float>(), st);
         ARSO_CUDA(cudaMemcpyAsync(grads_out, g.ptr, N_PARAMS * 4, cudaMemcpyDeviceToHost, st));
@@ -883,9 +890,9 @@ arso_status arso_surrogate_train(arso_surrogate *s, const float *x, const float 
         ARSO_REQUIRE(lr > 0, "lr must be > 0");
         cudaStream_t st = (cudaStream_t)stream;
         ensure_norm(s, x, n, st);
-        Activations a;
+        Activations a(st);
         a.ensure((int)std::min<uint64_t>(batch, n));
-        DeviceBuffer d_idx;
+        StreamBuffer d_idx(st);
         d_idx.ensure(n * 4);
         std::vector<uint32_t> idx(n);
         std::mt19937_64 rng(seed);
@@ -925,7 +932,7 @@ arso_status arso_surrogate_predict(const arso_surrogate *s, const float *x, uint
     try {
         ARSO_REQUIRE(s && x && out, "NULL argument");
         cudaStream_t st = (cudaStream_t)stream;
-        Activations a;
+        Activations a(st);
         const uint64_t chunk = 65536;
         a.ensure((int)std::min<uint64_t>(n, chunk));
         for (uint64_t b0 = 0; b0 < n; b0 += chunk) {
