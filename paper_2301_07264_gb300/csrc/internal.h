@@ -58,11 +58,10 @@ enum GateClass : uint8_t {
 // diagonal gates, X gates and Pauli errors act on any bit.
 constexpr int REG_BITS = 5;
 constexpr int RB_MIN_TILE = 10;                   // 32 threads x 32 amplitudes
-// gates per phase at most: the register kernels stage a phase's gate records
-// in shared memory (double-buffered: the next phase's copy overlaps this one)
+// the register kernels stage a phase's program in shared memory (double-buffered: the
+// next phase's copy overlaps this one); gates per phase at most in a tensor circuit:
 constexpr int MAX_PHASE_OPS = 64;
-constexpr int MAX_PHASE_UNITS = 4 * MAX_PHASE_OPS;  // of the register program: a gate takes at most two, and
-                                                    // two for a phase before it
+constexpr int MAX_PHASE_UNITS = 256;  // of the register program
 inline uint32_t pack_rbits(const uint32_t *p) {   // 5 local bit positions, 5 bits each
     uint32_t r = 0;
     for (int b = 0; b < REG_BITS; ++b) r |= p[b] << (5 * b);
@@ -113,7 +112,7 @@ enum RegOpCode : uint32_t {
     OP_OMEGA = 72,   // diag(1, omega^k), omega = e^{i pi/4}
     OP_DIAG1 = 73,   // tensor circuits only
     OP_CP = 74,      // diag(1, 1, 1, f)
-    OP_CX = 75,      // + target position
+    OP_CX = 75,      // + target position; in a register program a flip under a condition (below)
     OP_DENSE2 = 80,
     OP_SWAP = 81,
     OP_NOP = 82,
@@ -121,6 +120,10 @@ enum RegOpCode : uint32_t {
     OP_LAYER = 84,   // one-qubit gates on distinct qubits (below)
     OP_CZS = 85,     // CZ gates on distinct qubits (below)
     OP_PROBE = 86,   // measurements on distinct qubits (below); probe circuits only
+    OP_BLOCK = 87,   // a fused run of gates (below)
+    OP_SIGN = 88,    // the signs of a fused run without a flip (below)
+    OP_PARITY = 89,  // f where q0 ^ q1 = 1, conj f elsewhere (a fused run)
+    OP_SCALE = 90,   // every amplitude times f
 };
 
 // Register program of a phase (circuits without tensor phases): macro-ops of 16-byte units.
@@ -136,6 +139,13 @@ enum RegOpCode : uint32_t {
 //           (position 0: (Re x, -Re x, Im x, Im x), the lanes of a packed register)
 //   OP_CZS: one unit for each CZ: the registers whose bit q0, and q1, is 1 as 32-bit masks
 //           (0 for a thread bit), and 31 - q0, 31 - q1
+//   OP_CX + p, OP_SIGN: one unit: the registers whose bit a, and b, is 1 as 32-bit masks (0
+//           for a thread bit); 31 - a | (31 - b) << 8 | (31 - c) << 16 | p_c << 24; the flip of c
+//           happens where the XOR of the terms of bits 0-2 (a, b, ab) is 1, then the signs
+//           where that of bits 3-6 (ab, ac, bc, abc) is 1 flip
+//   OP_BLOCK: the gates [.., end) fused: z = units after this header and its fused macro-op
+//           that hold the gates one by one. A trajectory with an error event among the gates
+//           runs those, the others the fused macro-op; both end in the same frame
 //   OP_PROBE: bits 8-12 of x the register positions measured, z the first one's slot in
 //           its pass; the slots follow in order of position
 // Frames: the true state is S * prod_q diag(1, phi_q) * X^m * stored, with the scalar S
@@ -339,6 +349,7 @@ struct arso_circuit {
     arso::DeviceBuffer d_rmats, d_evs, d_prog, d_ph_pg;
     arso::DeviceBuffer d_frame;             // tables of `frame` per pass, or per checkpoint (resident)
     std::vector<uint8_t> frame_trivial;     // streaming: per pass
+    std::vector<std::pair<uint32_t, uint32_t>> blocks;  // fused runs: [first, end) engine positions
     std::vector<uint32_t> chg_prefix;       // phase k -> phases 1 <= p < k whose register set differs from p-1's
     // tensor-core phases (ARSO_OPT_TENSOR_PHASES on a streaming complex64 circuit)
     bool tensor = false;

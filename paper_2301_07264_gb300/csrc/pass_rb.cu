@@ -223,6 +223,29 @@ __device__ __forceinline__ void rg_h_lanes(Amps &a, float sg) {
     }
 }
 
+// Exchange the members of the pairs along register bit P where the mask (over registers;
+// both members of a pair have the same bit) is set.
+template <int P> __device__ __forceinline__ void rg_flip_if(Amps &a, uint32_t mask) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        constexpr int bit = P > 0 ? 1 << (P > 0 ? P - 1 : 0) : 0;
+        if (k & bit) continue;
+        const bool x = (mask >> (2 * k)) & 1u, y = P > 0 ? ((mask >> (2 * k + 1)) & 1u) : x;
+        if (P == 0) {
+            const float2 r = a.re[k], i = a.im[k];
+            a.re[k] = make_float2(x ? r.y : r.x, x ? r.x : r.y);
+            a.im[k] = make_float2(x ? i.y : i.x, x ? i.x : i.y);
+        } else {
+            const int k1 = k | bit;
+            const float2 r0 = a.re[k], i0 = a.im[k], r1 = a.re[k1], i1 = a.im[k1];
+            a.re[k] = make_float2(x ? r1.x : r0.x, y ? r1.y : r0.y);
+            a.re[k1] = make_float2(x ? r0.x : r1.x, y ? r0.y : r1.y);
+            a.im[k] = make_float2(x ? i1.x : i0.x, y ? i1.y : i0.y);
+            a.im[k1] = make_float2(x ? i0.x : i1.x, y ? i0.y : i1.y);
+        }
+    }
+}
+
 // CX on stored data, target register bit P; control is register bit cpos
 // (0..4) or, when cpos == 15, the thread-level bit value cth.
 template <int P> __device__ __forceinline__ void rg_cx(Amps &a, uint32_t cpos, uint32_t cth) {
@@ -823,8 +846,47 @@ __device__ __forceinline__ void apply_macro(Amps &a, TileCtx &c, const uint4 h, 
         case OP_OMEGA: rg_omega(a, c, q0, p0, (h.x >> 20) & 7u); break;
         case OP_PHASE: phase_pair(a, bit_mask(c, q0), make_float2(__uint_as_float(u->x), __uint_as_float(u->y))); break;
         case OP_CP: rg_cp(a, c, q0, q1, make_float2(__uint_as_float(u->x), __uint_as_float(u->y))); break;
-        case OP_CX: ARSO_CX(0); break;
-        ARSO_P4(OP_CX, ARSO_CX)
+        case OP_SIGN:
+        case OP_CX: case OP_CX + 1: case OP_CX + 2: case OP_CX + 3: case OP_CX + 4: {
+            const uint4 w = *u;
+            const uint32_t tm = c.tpart ^ c.m;
+            const uint32_t A = w.x ^ (uint32_t)((int)(tm << (w.z & 31u)) >> 31);
+            const uint32_t B = w.y ^ (uint32_t)((int)(tm << ((w.z >> 8) & 31u)) >> 31);
+            const uint32_t mask = (w.w & 1u ? A : 0u) ^ (w.w & 2u ? B : 0u) ^ (w.w & 4u ? A & B : 0u);
+            if (mask) {
+                switch (code) {
+                    case OP_CX: rg_flip_if<0>(a, mask); break;
+                    case OP_CX + 1: rg_flip_if<1>(a, mask); break;
+                    case OP_CX + 2: rg_flip_if<2>(a, mask); break;
+                    case OP_CX + 3: rg_flip_if<3>(a, mask); break;
+                    case OP_CX + 4: rg_flip_if<4>(a, mask); break;
+                    default: break;
+                }
+            }
+            c.m ^= h.w;
+            if (w.w & 0x78u) {
+                const uint32_t pc = w.z >> 24;
+                const uint32_t C = (pc < REG_BITS ? reg_pattern(pc) : 0u) ^
+                                   (uint32_t)((int)((c.tpart ^ c.m) << ((w.z >> 16) & 31u)) >> 31);
+                const uint32_t sg = (w.w & 8u ? A & B : 0u) ^ (w.w & 16u ? A & C : 0u) ^ (w.w & 32u ? B & C : 0u) ^
+                                    (w.w & 64u ? A & B & C : 0u);
+                if (sg) negate_masked(a, sg);
+            }
+            break;
+        }
+        case OP_PARITY:
+            phase_pair(a, bit_mask(c, q0) ^ bit_mask(c, q1), make_float2(__uint_as_float(u->x), __uint_as_float(u->y)));
+            break;
+        case OP_SCALE: {
+            const float2 fr = bc2(__uint_as_float(u->x)), fi = bc2(__uint_as_float(u->y)), nfi = bc2(-__uint_as_float(u->y));
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const float2 r = a.re[k], i = a.im[k];
+                a.re[k] = fma2(nfi, i, mul2(fr, r));
+                a.im[k] = fma2(fi, r, mul2(fr, i));
+            }
+            break;
+        }
         case OP_DENSE1: {
             const float2 *M = mats + u->x;
             const uint32_t f = ARSO_FLIP;
@@ -879,10 +941,17 @@ __device__ __forceinline__ void run_prog(Amps &v, TileCtx &c, const uint4 *u, co
                                          const float2 *__restrict__ mats, float2 *sm, float2 *ubuf, int t,
                                          const uint32_t *&ev, const uint32_t *ev_end, uint32_t &next,
                                          const EvSlot *__restrict__ evs) {
+    uint32_t skip = 0;  // units after the next macro-op
     while (u < ue) {
         const uint4 h = *u;
+        if ((h.x & 255u) == OP_BLOCK) {  // fused, unless an event falls inside
+            if (ev_pos(next) < h.y) u += 1 + (u[1].x >> 24);
+            else ++u, skip = h.z;
+            continue;
+        }
         apply_macro(v, c, h, u + 1, mats, sm, ubuf, t);
-        u += h.x >> 24;
+        u += (h.x >> 24) + skip;
+        skip = 0;
         while (ev_pos(next) < h.y) {
             const float4 e = __ldg(reinterpret_cast<const float4 *>(evs + 2 * ev_pos(next) + ev_slot(next)));
             const uint32_t q = __float_as_uint(e.z), pc = ev_code(next);
@@ -1355,7 +1424,7 @@ __global__ void __launch_bounds__(THREADS, MINB) probe_kernel(ProbeArgs a) {
                 const uint4 h = *u;
                 if ((h.x & 255u) == OP_PROBE) run_probe<DUAL>(v, c, h, row);
                 else apply_macro(v, c, h, u + 1, a.mats, sm, ubuf, t);
-                u += h.x >> 24;
+                u += h.x >> 24;  // a probe circuit has no fused runs
             }
         }
         if (a.frame) apply_frame(v, c, a.frame, t);

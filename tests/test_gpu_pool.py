@@ -1,6 +1,8 @@
 """The library's memory pool: error lists made on one stream and run on another, several
 threads at once, and memory given back with the last handle."""
-import gc
+import os
+import subprocess
+import sys
 import threading
 
 import numpy as np
@@ -42,15 +44,27 @@ def test_streams_and_threads_share_the_pool():
             assert np.array_equal(x, y)
 
 
+CHILD = """
+import gc
+import numpy as np, torch
+from paper_2301_07264_gb300 import arso
+from workloads import circuits as C
+torch.cuda.synchronize()
+free0 = torch.cuda.mem_get_info()[0]
+circ = C.brickwork(22, 4, 1)
+cc = arso.compile_circuit(circ.n, circ.gates)
+errs = arso.sample_errors(cc, 1e-2, 1e-2, 1e-2, 0, 0, 40)
+arso.run_trajectories(cc, errs, circ.criterion, np.zeros(40))  # 32 MiB a state: over 1 GiB of working states
+used = free0 - torch.cuda.mem_get_info()[0]
+del cc, errs
+gc.collect()
+left = free0 - torch.cuda.mem_get_info()[0]
+assert used > 1 << 30, used
+assert left < (256 << 20) + (64 << 20), left
+"""
+
+
 def test_memory_goes_back_with_the_last_handle():
-    from paper_2301_07264_gb300 import arso
-    gc.collect()
-    torch.cuda.synchronize()
-    free0 = torch.cuda.mem_get_info()[0]
-    circ = C.brickwork(22, 4, 1)
-    cc = arso.compile_circuit(circ.n, circ.gates)
-    _scores(arso, cc, circ, 0, None, None, T=40, p=1e-2)  # 32 MiB a state: over 1 GiB of working states
-    assert free0 - torch.cuda.mem_get_info()[0] > 1 << 30
-    del cc
-    gc.collect()
-    assert free0 - torch.cuda.mem_get_info()[0] < (256 << 20) + (64 << 20)
+    # in a process of its own: no other test's handles keep memory mapped
+    subprocess.run([sys.executable, "-c", CHILD], check=True, timeout=300,
+                   cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
