@@ -963,8 +963,7 @@ struct ProgWriter {
     bool open = false;               // a layer being collected
     uint32_t active = 0, real = 0, flips = 0, used = 0, end = 0;
     float2 x[REG_BITS];
-    std::vector<uint4> czs;          // CZ gates being collected (open is false then)
-    uint32_t probes = 0;             // register positions being measured (open is false and czs empty then)
+    uint32_t probes = 0;             // register positions being measured (open is false then)
     ProbeSlot probe[REG_BITS];
     std::vector<ProbeSlot> *slots = nullptr;
     size_t slot0 = 0;                // the pass's first slot
@@ -976,12 +975,6 @@ struct ProgWriter {
             for (int p = 0; p < REG_BITS; ++p)
                 if (probes >> p & 1) slots->push_back(probe[p]);
             probes = 0;
-        }
-        if (!czs.empty()) {
-            last = out.size();
-            out.push_back(make_uint4(OP_CZS | (uint32_t)(czs.size() + 1) << 24, end, 0, 0));
-            out.insert(out.end(), czs.begin(), czs.end());
-            czs.clear();
         }
         if (!open) return;
         open = false;
@@ -998,12 +991,12 @@ struct ProgWriter {
         }
     }
     void start(uint32_t tile_bit) {  // a layer that has no gate on tile_bit yet
-        if (probes || !czs.empty() || (open && (used >> tile_bit & 1))) close();
+        if (probes || (open && (used >> tile_bit & 1))) close();
         if (!open) open = true, active = real = flips = used = 0;
         used |= 1u << tile_bit;
     }
     void nop(uint32_t tile_bit, uint32_t pos) {  // absorbed: only its events are left
-        if (open || !czs.empty() || probes) used |= 1u << tile_bit, end = pos + 1;
+        if (open || probes) used |= 1u << tile_bit, end = pos + 1;
         else if (last != SIZE_MAX) out[last].y = pos + 1;
         else start(tile_bit), end = pos + 1;
     }
@@ -1021,12 +1014,10 @@ struct ProgWriter {
         end = pos + 1;
     }
     void cz(uint32_t q0, uint32_t q1, uint32_t p0, uint32_t p1, uint32_t pos) {
-        const uint32_t both = 1u << q0 | 1u << q1;
-        if (open || probes || (!czs.empty() && (used & both))) close();
-        if (czs.empty()) used = 0;
-        used |= both;
-        czs.push_back(make_uint4(reg_bits(p0), reg_bits(p1), 31 - q0, 31 - q1));
-        end = pos + 1;
+        if (p0 > p1) std::swap(p0, p1), std::swap(q0, q1);
+        const uint32_t R = REG_BITS;
+        const uint32_t pair = p0 == 0 ? p1 - 1 : p0 == 1 ? p1 + 2 : p0 == 2 ? p1 + 4 : 9;
+        op(p1 < R ? OP_CZ_RR + pair : p0 < R ? OP_CZ_RT + p0 : (uint32_t)OP_CZ_TT, pos + 1, q0 | q1 << 8);
     }
     // conditional flip of c (register position pc) and signs: terms (internal.h) over a, b, c
     void flip_if(uint32_t a, uint32_t pa, uint32_t b, uint32_t pb, uint32_t cq, uint32_t pc, uint32_t terms,
@@ -1043,7 +1034,7 @@ struct ProgWriter {
         return p < 5 ? pat[p] : 0u;
     }
     void measure(Frame &F, uint32_t tile_bit, uint32_t p, uint32_t loc, uint32_t pos) {
-        if (open || !czs.empty() || (probes && (used >> tile_bit & 1))) close();
+        if (open || (probes && (used >> tile_bit & 1))) close();
         if (!probes) used = 0;
         used |= 1u << tile_bit;
         probes |= 1u << p;
@@ -1061,8 +1052,7 @@ struct ProgWriter {
     void flush(Frame &F, uint32_t q, uint32_t p, uint32_t pos) {
         const int k = snap(F.phi(q));
         if (k == 0) return;
-        const bool collecting = open || !czs.empty();
-        const bool before = collecting && !probes && !(used >> q & 1);
+        const bool before = open && !(used >> q & 1);
         if (!before) close();
         if (k > 0) {
             op(OP_OMEGA | (uint32_t)k << 20, before ? 0 : pos, q | p << 16, nullptr, true);

@@ -105,6 +105,8 @@ enum RegOpCode : uint32_t {
     OP_SU2 = 0,      // + position 0..4 (0: the packed lanes); tensor circuits only
     OP_DENSE1 = 5,   // + position
     OP_H = 10,       // + 2 * position + mask bit of q0; tensor circuits only
+    // CZ; in a register program the mask plays no part: + pair index for RR, + register
+    // position for RT (q1 the thread bit)
     OP_CZ_RR = 20,   // + 4 * pair index of (lower, higher) position + 2 * want(lower) + want(higher)
     OP_CZ_RT = 60,   // + 2 * register position + want(register qubit); the other qubit is a thread bit
     OP_CZ_TT = 70,   // both qubits thread bits
@@ -118,7 +120,6 @@ enum RegOpCode : uint32_t {
     OP_NOP = 82,
     OP_PHASE = 83,   // diag(conj f, f)
     OP_LAYER = 84,   // one-qubit gates on distinct qubits (below)
-    OP_CZS = 85,     // CZ gates on distinct qubits (below)
     OP_PROBE = 86,   // measurements on distinct qubits (below); probe circuits only
     OP_BLOCK = 87,   // a fused run of gates (below)
     OP_SIGN = 88,    // the signs of a fused run without a flip (below)
@@ -137,8 +138,6 @@ enum RegOpCode : uint32_t {
 //   OP_LAYER: bits 8-12 of x the register positions that hold a gate G(x), bits 13-17
 //           those whose x is real; one unit (Re x, Re x, Im x, Im x) for each, in order
 //           (position 0: (Re x, -Re x, Im x, Im x), the lanes of a packed register)
-//   OP_CZS: one unit for each CZ: the registers whose bit q0, and q1, is 1 as 32-bit masks
-//           (0 for a thread bit), and 31 - q0, 31 - q1
 //   OP_CX + p, OP_SIGN: one unit: the registers whose bit a, and b, is 1 as 32-bit masks (0
 //           for a thread bit); 31 - a | (31 - b) << 8 | (31 - c) << 16 | p_c << 24; the flip of c
 //           happens where the XOR of the terms of bits 0-2 (a, b, ab) is 1, then the signs
@@ -148,9 +147,11 @@ enum RegOpCode : uint32_t {
 //           runs those, the others the fused macro-op; both end in the same frame
 //   OP_PROBE: bits 8-12 of x the register positions measured, z the first one's slot in
 //           its pass; the slots follow in order of position
-// Frames: the true state is S * prod_q diag(1, phi_q) * X^m * stored, with the scalar S
+// Frames: the true state is S * prod_q diag(1, phi_q) * X^m Z^z * stored, with the scalar S
 // and the unit phases phi_q the same for every trajectory and tracked on the host in FP64
-// from gate to gate (reg_program in circuit.cpp). A unitary U diag(1, phi) equals, up to
+// from gate to gate (reg_program in circuit.cpp), and the masks m and z kept by the kernel:
+// X and Z errors only change them, and a CZ is the same signs whatever m is, its effect on
+// X^m going into z. A unitary U diag(1, phi) equals, up to
 // such a frame, G(x) = [[1, x], [-conj x, 1]] with |x| <= 1, after an index flip X
 // when |u00| < |u01|: half the multiplications of the full matrix, none at all for
 // one-qubit diagonal gates, and no rounded 1/sqrt2 for H (x = +-1). The gates of a layer

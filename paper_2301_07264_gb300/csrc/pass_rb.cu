@@ -11,13 +11,11 @@
 //  * dense one-qubit gates, H and CX targets act on register bits, entirely
 //    in registers;
 //  * diagonal gates (T, S, Z, RZ, P, CZ, CP) act on any bit in place;
-//  * X gates and the X part of Pauli errors never move data: the tile keeps
-//    an index mask m with state[j] = stored[j ^ m] (Eq. (2): X swaps the pair
-//    (a0, a1), i.e. flips bit q of the index), later gates act on the stored
-//    data conjugated by the mask, and the final store writes stored[k] to
-//    index k ^ m;
-//  * the Z part of a Pauli error is a phase on bit q; Y = i X Z adds a factor
-//    i tracked as a power gp and applied at the store.
+//  * X gates and Pauli errors never touch the data: the tile keeps masks m and z with
+//    state[j] = (-1)^(z . (j ^ m)) stored[j ^ m] (Eq. (2): X swaps the pair (a0, a1), i.e.
+//    flips bit q of the index; Z is a sign on it), later gates act on the stored
+//    data conjugated by the masks, and the final store writes the signed stored[k] to
+//    index k ^ m; Y = i X Z adds a factor i tracked as a power gp and applied at the store.
 // Global loads and stores are 16-byte vector accesses in the mapping
 // R = {0, t-4, t-3, t-2, t-1}, whose thread bits 1..t-5 are contiguous.
 #include <cuda_fp16.h>
@@ -30,7 +28,8 @@
 
 namespace arso {
 
-__device__ __forceinline__ uint32_t swz(uint32_t j) { return j ^ (((j >> 4) ^ (j >> 8) ^ (j >> 12)) & 15u); }
+// slot of pair J: eight 16-byte slots make a bank row, so the higher bits fold into three
+__device__ __forceinline__ uint32_t swz(uint32_t j) { return j ^ (((j >> 3) ^ (j >> 6) ^ (j >> 9) ^ (j >> 12)) & 7u); }
 
 // register bit b of a packed register set (the five bits are stored in ascending order)
 __device__ __forceinline__ uint32_t rbit(uint32_t packed, int b) { return (packed >> (5 * b)) & 31u; }
@@ -84,10 +83,13 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 
 // ------------------------------------------------------- register gates ---
 // Code size matters: warps stall for instructions more than for anything else
-// when the phase loop outgrows the instruction cache (with CZ specialised per pair
-// of positions 2.9 of 9.2 warps per issue waited for them, with the mask form 1.4 of
-// 8.4), so only dense one-qubit gates and odd phases are specialised per register
-// position; everything else is position-free.
+// when the phase loop outgrows the instruction cache (with 46 CZ variants by
+// positions and mask bits 2.9 of 9.2 warps per issue waited for them, with a
+// position-free form 1.4 of 8.4), so only dense one-qubit gates, odd phases and CZ
+// are specialised per register position; everything else is position-free. CZ has
+// 16 variants of 8 negations since the z mask took the mask bits out of its signs:
+// 24-qubit brickwork, 177 trajectories, passes 336 -> 305 ms against the position-free
+// form (about 165 instructions per warp for a layer of them).
 
 // U on register bit P >= 1: packed registers k and k | 2^(P-1) hold the pairs
 template <int P>
@@ -269,6 +271,7 @@ struct TileCtx {
     uint32_t R;          // register bits of the current phase, 5 bits each (bit 0 of the tile first)
     uint32_t tpart;      // thread part of the local index
     uint32_t m;          // X mask (stored[j] = state[j ^ m])
+    uint32_t z;          // Z mask on stored indices (register programs)
     uint32_t gp;         // global phase i^gp
     uint32_t tid, nthr;  // thread index within the tile's thread group, group size
 };
@@ -415,6 +418,14 @@ template <int P, int W> __device__ __forceinline__ void neg_half(Amps &a) {
         a.im[k] = mul2(s, a.im[k]);
     }
 }
+__device__ __forceinline__ void negate_all(Amps &a) {
+    const float2 m1 = bc2(-1.f);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        a.re[k] = mul2(m1, a.re[k]);
+        a.im[k] = mul2(m1, a.im[k]);
+    }
+}
 __host__ __device__ constexpr int cz_pa(int pp) { return pp < 4 ? 0 : pp < 7 ? 1 : pp < 9 ? 2 : 3; }
 __host__ __device__ constexpr int cz_pb(int pp) {
     return pp < 4 ? pp + 1 : pp < 7 ? pp - 2 : pp < 9 ? pp - 4 : 4;
@@ -485,9 +496,10 @@ __device__ __forceinline__ void set_phase(TileCtx &c, uint32_t packed, int t) {
     c.tpart = thread_part(c.tid, packed);
 }
 
-// Shared memory holds a tile as two planes of packed neighbour pairs:
-// plane_re[swz(J)] = (Re a_2J, Re a_2J+1) and plane_im likewise, plane_im =
-// plane_re + 2^(t-1). The swizzle is linear over XOR, so the slot of packed
+// Shared memory holds a tile as packed neighbour pairs, 16 bytes each: slot swz(J) = (Re a_2J,
+// Re a_2J+1, Im a_2J, Im a_2J+1), so a register set changes with 16 writes and 16 reads a
+// thread instead of 32 and 32 of 8 bytes (the same bytes: half the issue slots). Eight slots
+// are one turn of the banks: the swizzle folds the higher bits into three. It is linear over XOR, so the slot of packed
 // register k is swz(tpart >> 1) ^ (XOR of swz(2^(r[b]-1)) over the set bits
 // b-1 of k); walking the registers in Gray-code order costs one XOR each.
 __host__ __device__ constexpr int ctz4(int x) { return x & 1 ? 0 : x & 2 ? 1 : x & 4 ? 2 : 3; }
@@ -500,24 +512,24 @@ __device__ __forceinline__ void smem_basis(const TileCtx &c, uint32_t &base, uin
 __device__ __forceinline__ void to_smem(const Amps &a, float2 *sm, const TileCtx &c, int t) {
     uint32_t idx, sw[REG_BITS - 1];
     smem_basis(c, idx, sw);
-    float2 *pim = sm + (1u << (t - 1));
+    float4 *p = reinterpret_cast<float4 *>(sm);
 #pragma unroll
     for (int kk = 0; kk < 16; ++kk) {
         const int k = kk ^ (kk >> 1);
-        sm[idx] = a.re[k];
-        pim[idx] = a.im[k];
+        p[idx] = make_float4(a.re[k].x, a.re[k].y, a.im[k].x, a.im[k].y);
         if (kk < 15) idx ^= sw[ctz4(kk + 1)];
     }
 }
 __device__ __forceinline__ void from_smem(Amps &a, const float2 *sm, const TileCtx &c, int t) {
     uint32_t idx, sw[REG_BITS - 1];
     smem_basis(c, idx, sw);
-    const float2 *pim = sm + (1u << (t - 1));
+    const float4 *p = reinterpret_cast<const float4 *>(sm);
 #pragma unroll
     for (int kk = 0; kk < 16; ++kk) {
         const int k = kk ^ (kk >> 1);
-        a.re[k] = sm[idx];
-        a.im[k] = pim[idx];
+        const float4 w = p[idx];
+        a.re[k] = make_float2(w.x, w.y);
+        a.im[k] = make_float2(w.z, w.w);
         if (kk < 15) idx ^= sw[ctz4(kk + 1)];
     }
 }
@@ -537,10 +549,39 @@ __device__ __forceinline__ void remap(Amps &a, float2 *sm, TileCtx &c, uint32_t 
 // the stored data (U already conjugated by the mask) with runtime indices.
 __device__ __forceinline__ void smem_dense2(float2 *sm, int t, uint32_t q0, uint32_t q1, const float2 *__restrict__ U,
                                             uint32_t tid, uint32_t nthr) {
-    float *pre = reinterpret_cast<float *>(sm);
-    float *pim = reinterpret_cast<float *>(sm + (1u << (t - 1)));
+    float *pre = reinterpret_cast<float *>(sm), *pim = pre + 2;
     const uint32_t lo = q0 < q1 ? q0 : q1, hi = q0 < q1 ? q1 : q0;
     const uint32_t m0 = 1u << q0, m1 = 1u << q1;
+    if (lo > 0) {
+        // neither qubit is tile bit 0: both amplitudes of a slot at once, one 16-byte read and write
+        // per slot and packed arithmetic. Bound by shared-memory reads and the 64 FMA of a group (12-qubit
+        // quantum volume, 4,000 trajectories: 1.08 ms with the scalar loop below for all pairs, 0.86 so)
+        float4 *s4 = reinterpret_cast<float4 *>(sm);
+        for (uint32_t p = tid; p < (1u << (t - 3)); p += nthr) {
+            const uint32_t i = insert_zero2(p, lo - 1, hi - 1);
+            const uint32_t ix[4] = {swz(i), swz(i | m0 >> 1), swz(i | m1 >> 1), swz(i | m0 >> 1 | m1 >> 1)};
+            float2 xr[4], xi[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float4 w = s4[ix[k]];
+                xr[k] = make_float2(w.x, w.y);
+                xi[k] = make_float2(w.z, w.w);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float2 r, c;
+#pragma unroll
+                for (int l = 0; l < 4; ++l) {
+                    const float2 u = U[4 * k + l];
+                    const float2 ur = bc2(u.x), ui = bc2(u.y), nui = bc2(-u.y);
+                    r = l ? fma2(nui, xi[l], fma2(ur, xr[l], r)) : fma2(nui, xi[l], mul2(ur, xr[l]));
+                    c = l ? fma2(ui, xr[l], fma2(ur, xi[l], c)) : fma2(ui, xr[l], mul2(ur, xi[l]));
+                }
+                s4[ix[k]] = make_float4(r.x, r.y, c.x, c.y);
+            }
+        }
+        return;
+    }
     float2 M[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) M[k] = U[k];
@@ -551,7 +592,7 @@ __device__ __forceinline__ void smem_dense2(float2 *sm, int t, uint32_t q0, uint
         float2 v[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            ix[k] = 2u * swz(jx[k] >> 1) + (jx[k] & 1u);
+            ix[k] = 4u * swz(jx[k] >> 1) + (jx[k] & 1u);
             v[k] = make_float2(pre[ix[k]], pim[ix[k]]);
         }
 #pragma unroll
@@ -575,14 +616,7 @@ __device__ __forceinline__ void rg_cz_code(Amps &a, const TileCtx &c, uint32_t x
     const uint32_t code = (x & 255u) + ba * ((x >> 8) & 3u) + bb * ((x >> 10) & 3u);
     if (code >= (uint32_t)OP_CZ_RT) {
         if (code == (uint32_t)OP_CZ_TT) {
-            if (thread_bit(c, q0) && thread_bit(c, q1)) {
-                const float2 m1 = bc2(-1.f);
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    a.re[k] = mul2(m1, a.re[k]);
-                    a.im[k] = mul2(m1, a.im[k]);
-                }
-            }
+            if (thread_bit(c, q0) && thread_bit(c, q1)) negate_all(a);
             return;
         }
         if (!thread_bit(c, p0 < REG_BITS ? q1 : q0)) return;
@@ -613,6 +647,7 @@ __device__ __forceinline__ void rg_cz_code(Amps &a, const TileCtx &c, uint32_t x
 __device__ __forceinline__ void tile_two(Amps &a, TileCtx &c, bool swap, uint32_t q0, uint32_t q1,
                                          const float2 *__restrict__ M, float2 *sm, float2 *ubuf, int t) {
     const uint32_t mab = ((c.m >> q0) & 1u) | (((c.m >> q1) & 1u) << 1);
+    const uint32_t zab = ((c.z >> q0) & 1u) | (((c.z >> q1) & 1u) << 1);
     if (c.tid < 16) {
         const uint32_t k = c.tid >> 2, l = c.tid & 3u;
         float2 u;
@@ -621,6 +656,7 @@ __device__ __forceinline__ void tile_two(Amps &a, TileCtx &c, bool swap, uint32_
             u = make_float2(perm[k] == l ? 1.f : 0.f, 0.f);
         } else {
             u = M[4 * (k ^ mab) + (l ^ mab)];
+            if (__popc(zab & (k ^ l)) & 1) u = make_float2(-u.x, -u.y);
         }
         ubuf[c.tid] = u;
     }
@@ -633,6 +669,7 @@ __device__ __forceinline__ void tile_two(Amps &a, TileCtx &c, bool swap, uint32_
     __syncthreads();
     // SWAP X^m = X^{m with bits q0, q1 exchanged} SWAP
     if (swap && (((c.m >> q0) ^ (c.m >> q1)) & 1u)) c.m ^= (1u << q0) | (1u << q1);
+    if (swap && (((c.z >> q0) ^ (c.z >> q1)) & 1u)) c.z ^= (1u << q0) | (1u << q1);
 }
 
 #define ARSO_CZ_ALL \
@@ -703,7 +740,8 @@ __device__ __forceinline__ void apply_op(Amps &a, TileCtx &c, const RegOp &op, c
 }
 
 // Raw sums (kernels.h) of the pairs along register bit P of this thread's registers.
-template <int P> __device__ __forceinline__ void rg_probe(const Amps &a, uint32_t flip, float *w) {
+// flip: the qubit's bit of m (s0 and s1 change places); g: the sign of its bit of z.
+template <int P> __device__ __forceinline__ void rg_probe(const Amps &a, uint32_t flip, float g, float *w) {
     float2 z = make_float2(0.f, 0.f), cr = z, ci = z;
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
@@ -716,11 +754,11 @@ template <int P> __device__ __forceinline__ void rg_probe(const Amps &a, uint32_
         ci = fma2(ni0, r1, fma2(r0, i1, ci));
     }
     const float zs = z.x + z.y, cs = ci.x + ci.y;
-    w[0] = flip ? -zs : zs;  // a flipped qubit: s0 and s1 change places
-    w[1] = cr.x + cr.y;
-    w[2] = flip ? -cs : cs;
+    w[0] = flip ? -zs : zs;
+    w[1] = g * (cr.x + cr.y);
+    w[2] = flip ? -g * cs : g * cs;
 }
-__device__ __forceinline__ void rg_probe_lanes(const Amps &a, uint32_t flip, float *w) {
+__device__ __forceinline__ void rg_probe_lanes(const Amps &a, uint32_t flip, float g, float *w) {
     float z = 0.f, cr = 0.f, ci = 0.f;
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
@@ -730,11 +768,11 @@ __device__ __forceinline__ void rg_probe_lanes(const Amps &a, uint32_t flip, flo
         ci = fmaf(-i.x, r.y, fmaf(r.x, i.y, ci));
     }
     w[0] = flip ? -z : z;
-    w[1] = cr;
-    w[2] = flip ? -ci : ci;
+    w[1] = g * cr;
+    w[2] = flip ? -g * ci : g * ci;
 }
 // psi in lane 0, phi in lane 1 of every packed register
-template <int P> __device__ __forceinline__ void rg_probe_dual(const Amps &a, uint32_t flip, float *w) {
+template <int P> __device__ __forceinline__ void rg_probe_dual(const Amps &a, uint32_t flip, float g, float *w) {
     float x[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
@@ -749,10 +787,10 @@ template <int P> __device__ __forceinline__ void rg_probe_dual(const Amps &a, ui
         x[4] = fmaf(-bi1, ai1, fmaf(-br1, ar1, fmaf(bi0, ai0, fmaf(br0, ar0, x[4]))));
         x[5] = fmaf(bi1, ar1, fmaf(-br1, ai1, fmaf(-bi0, ar0, fmaf(br0, ai0, x[5]))));
     }
-    w[0] = flip ? x[2] : x[0];
-    w[1] = flip ? x[3] : x[1];
-    w[2] = flip ? x[0] : x[2];
-    w[3] = flip ? x[1] : x[3];
+    w[0] = g * (flip ? x[2] : x[0]);
+    w[1] = g * (flip ? x[3] : x[1]);
+    w[2] = g * (flip ? x[0] : x[2]);
+    w[3] = g * (flip ? x[1] : x[3]);
     w[4] = flip ? -x[4] : x[4];
     w[5] = flip ? -x[5] : x[5];
 }
@@ -768,11 +806,12 @@ template <bool DUAL> __device__ __forceinline__ void run_probe(const Amps &a, co
 #define ARSO_PROBE_P(P)                                                          \
     if (h.x & (0x100u << P)) {                                                   \
         const uint32_t f = (c.m >> rbit(c.R, P)) & 1u;                           \
-        if constexpr (DUAL) rg_probe_dual<P>(a, f, w + SUMS * (P - P0));         \
-        else rg_probe<P>(a, f, w + SUMS * (P - P0));                             \
+        const float g = (c.z >> rbit(c.R, P)) & 1u ? -1.f : 1.f;                 \
+        if constexpr (DUAL) rg_probe_dual<P>(a, f, g, w + SUMS * (P - P0));      \
+        else rg_probe<P>(a, f, g, w + SUMS * (P - P0));                          \
     }
     if constexpr (!DUAL) {
-        if (h.x & 0x100u) rg_probe_lanes(a, (c.m >> rbit(c.R, 0)) & 1u, w);
+        if (h.x & 0x100u) rg_probe_lanes(a, c.m & 1u, c.z & 1u ? -1.f : 1.f, w);
     }
     ARSO_PROBE_P(1) ARSO_PROBE_P(2) ARSO_PROBE_P(3) ARSO_PROBE_P(4)
 #undef ARSO_PROBE_P
@@ -801,12 +840,14 @@ __device__ __forceinline__ void apply_macro(Amps &a, TileCtx &c, const uint4 h, 
     const uint32_t code = h.x & 255u;
     if (code == OP_LAYER) {
         c.m ^= h.w;
-        // X G(x) X = G(-conj x): the mask bit of the qubit flips the sign of Re x
+        // X G(x) X = G(-conj x), Z G(x) Z = G(-x): the qubit's bit of z flips the sign of x,
+        // that of m the sign of Re x
+        const uint32_t mz = c.m ^ c.z;
 #define ARSO_LAYER_X                                                           \
     const uint4 w = *u++;                                                      \
-    const uint32_t f = ((c.m >> rbit(c.R, P)) & 1u) << 31;                     \
+    const uint32_t f = (mz >> rbit(c.R, P)) << 31, g = (c.z >> rbit(c.R, P)) << 31; \
     const float2 xr = make_float2(__uint_as_float(w.x ^ f), __uint_as_float(w.y ^ f)); \
-    const float2 xi = make_float2(__uint_as_float(w.z), __uint_as_float(w.w));
+    const float2 xi = make_float2(__uint_as_float(w.z ^ g), __uint_as_float(w.w ^ g));
         if (h.x & 0x100u) {
             constexpr int P = 0;
             ARSO_LAYER_X
@@ -829,20 +870,42 @@ __device__ __forceinline__ void apply_macro(Amps &a, TileCtx &c, const uint4 h, 
         return;
     }
     const uint32_t q0 = h.z & 255u, q1 = (h.z >> 8) & 255u, p0 = (h.z >> 16) & 15u;
+    // Z M Z: the off-diagonal entries change sign
+    const float zs = (c.z >> q0) & 1u ? -1.f : 1.f;
+#define ARSO_ZS(v) make_float2(zs * (v).x, zs * (v).y)
+#define ARSO_D1Z(P)                                                                                     \
+    {                                                                                                   \
+        const float2 *M = mats + u->x;                                                                  \
+        const uint32_t f = ARSO_FLIP;                                                                   \
+        rg_dense1<P>(a, M[f ? 3 : 0], ARSO_ZS(M[f ? 2 : 1]), ARSO_ZS(M[f ? 1 : 2]), M[f ? 0 : 3]);        \
+    }
     switch (code) {
-        case OP_CZS: {
-            // every CZ of the layer as one sign per register: 96 ALU instructions and 10 a CZ, in
-            // code that fits the instruction cache where one block per pair of positions does not
-            const uint32_t tm = c.tpart ^ c.m;
-            uint32_t mask = 0;
-            for (const uint4 *e = u + (h.x >> 24) - 1; u < e; ++u) {
-                const uint4 w = *u;
-                const uint32_t s0 = (uint32_t)((int)(tm << w.z) >> 31), s1 = (uint32_t)((int)(tm << w.w) >> 31);
-                mask ^= (w.x ^ s0) & (w.y ^ s1);
-            }
-            negate_masked(a, mask);
-            break;
-        }
+        // CZ X^m = X^m CZ with Z on a qubit whose partner is flipped: the signs do not depend on m
+#define ARSO_CZ_MASKS                                                          \
+    {                                                                          \
+        const uint32_t b0 = (c.m >> q0) & 1u, b1 = (c.m >> q1) & 1u;           \
+        c.z ^= (b0 << q1) ^ (b1 << q0);                                        \
+        c.gp ^= (b0 & b1) << 1;                                                \
+    }
+        case OP_CZ_RR + 0: neg_quarter<0, 1, 1, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RR + 1: neg_quarter<0, 2, 1, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RR + 2: neg_quarter<0, 3, 1, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RR + 3: neg_quarter<0, 4, 1, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RR + 4: neg_quarter<1, 2, 1, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RR + 5: neg_quarter<1, 3, 1, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RR + 6: neg_quarter<1, 4, 1, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RR + 7: neg_quarter<2, 3, 1, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RR + 8: neg_quarter<2, 4, 1, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RR + 9: neg_quarter<3, 4, 1, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RT + 0: if ((c.tpart >> q1) & 1u) neg_half<0, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RT + 1: if ((c.tpart >> q1) & 1u) neg_half<1, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RT + 2: if ((c.tpart >> q1) & 1u) neg_half<2, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RT + 3: if ((c.tpart >> q1) & 1u) neg_half<3, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_RT + 4: if ((c.tpart >> q1) & 1u) neg_half<4, 1>(a); ARSO_CZ_MASKS break;
+        case OP_CZ_TT:
+            if ((c.tpart >> q0) & (c.tpart >> q1) & 1u) negate_all(a);
+            ARSO_CZ_MASKS break;
+#undef ARSO_CZ_MASKS
         case OP_OMEGA: rg_omega(a, c, q0, p0, (h.x >> 20) & 7u); break;
         case OP_PHASE: phase_pair(a, bit_mask(c, q0), make_float2(__uint_as_float(u->x), __uint_as_float(u->y))); break;
         case OP_CP: rg_cp(a, c, q0, q1, make_float2(__uint_as_float(u->x), __uint_as_float(u->y))); break;
@@ -863,15 +926,26 @@ __device__ __forceinline__ void apply_macro(Amps &a, TileCtx &c, const uint4 h, 
                     default: break;
                 }
             }
+            uint32_t sg = 0;
+            if ((w.w & 7u) && ((c.z >> (31u - ((w.z >> 16) & 31u))) & 1u)) {
+                // Z on the target: a sign where it flips; for CX, Z on the control
+                if ((w.w & 7u) == 1u) {
+                    const uint32_t qa = 31u - (w.z & 31u);
+                    c.z ^= 1u << qa;
+                    c.gp ^= ((c.m >> qa) & 1u) << 1;
+                } else {
+                    sg = mask;
+                }
+            }
             c.m ^= h.w;
             if (w.w & 0x78u) {
                 const uint32_t pc = w.z >> 24;
                 const uint32_t C = (pc < REG_BITS ? reg_pattern(pc) : 0u) ^
                                    (uint32_t)((int)((c.tpart ^ c.m) << ((w.z >> 16) & 31u)) >> 31);
-                const uint32_t sg = (w.w & 8u ? A & B : 0u) ^ (w.w & 16u ? A & C : 0u) ^ (w.w & 32u ? B & C : 0u) ^
-                                    (w.w & 64u ? A & B & C : 0u);
-                if (sg) negate_masked(a, sg);
+                sg ^= (w.w & 8u ? A & B : 0u) ^ (w.w & 16u ? A & C : 0u) ^ (w.w & 32u ? B & C : 0u) ^
+                      (w.w & 64u ? A & B & C : 0u);
             }
+            if (sg) negate_masked(a, sg);
             break;
         }
         case OP_PARITY:
@@ -890,13 +964,13 @@ __device__ __forceinline__ void apply_macro(Amps &a, TileCtx &c, const uint4 h, 
         case OP_DENSE1: {
             const float2 *M = mats + u->x;
             const uint32_t f = ARSO_FLIP;
-            rg_dense1_lanes(a, M[f ? 3 : 0], M[f ? 2 : 1], M[f ? 1 : 2], M[f ? 0 : 3]);
+            rg_dense1_lanes(a, M[f ? 3 : 0], ARSO_ZS(M[f ? 2 : 1]), ARSO_ZS(M[f ? 1 : 2]), M[f ? 0 : 3]);
             break;
         }
-        case OP_DENSE1 + 1: { const float2 *M = mats + u->x; ARSO_D1(1); break; }
-        case OP_DENSE1 + 2: { const float2 *M = mats + u->x; ARSO_D1(2); break; }
-        case OP_DENSE1 + 3: { const float2 *M = mats + u->x; ARSO_D1(3); break; }
-        case OP_DENSE1 + 4: { const float2 *M = mats + u->x; ARSO_D1(4); break; }
+        case OP_DENSE1 + 1: ARSO_D1Z(1); break;
+        case OP_DENSE1 + 2: ARSO_D1Z(2); break;
+        case OP_DENSE1 + 3: ARSO_D1Z(3); break;
+        case OP_DENSE1 + 4: ARSO_D1Z(4); break;
         case OP_DENSE2: tile_two(a, c, false, q0, q1, mats + u->x, sm, ubuf, t); break;
         case OP_SWAP: tile_two(a, c, true, q0, q1, nullptr, sm, ubuf, t); break;
         default: break;
@@ -904,6 +978,8 @@ __device__ __forceinline__ void apply_macro(Amps &a, TileCtx &c, const uint4 h, 
 }
 #undef ARSO_FLIP
 #undef ARSO_D1
+#undef ARSO_D1Z
+#undef ARSO_ZS
 #undef ARSO_CX
 #undef ARSO_CZ_ALL
 #undef ARSO_P4
@@ -955,7 +1031,12 @@ __device__ __forceinline__ void run_prog(Amps &v, TileCtx &c, const uint4 *u, co
         while (ev_pos(next) < h.y) {
             const float4 e = __ldg(reinterpret_cast<const float4 *>(evs + 2 * ev_pos(next) + ev_slot(next)));
             const uint32_t q = __float_as_uint(e.z), pc = ev_code(next);
-            rg_pauli(v, c, q, pc);
+            if (pc & 2u) {  // Z part (Eq. (2)): on the true bit, so a sign of all where the bit is flipped
+                c.z ^= 1u << q;
+                c.gp ^= ((c.m >> q) & 1u) << 1;
+            }
+            if (pc & 1u) c.m ^= 1u << q;
+            if (pc == 3u) c.gp = (c.gp + 1u) & 3u;  // Y = i X Z
             if ((pc & 1u) && e.x != 1.f) phase_pair(v, ~bit_mask(c, q), make_float2(e.x, e.y));
             ++ev;
             next = ev < ev_end ? *ev : NO_EVENT;
@@ -1156,13 +1237,12 @@ __device__ __forceinline__ LoadAt tile_at(uint32_t base, const uint32_t *__restr
 // register bits: the mask only swaps the branches of its nodes, so a score does not
 // depend on the checkpoint its trajectory started from. The reference is read two
 // neighbours (16 bytes) at a time.
-__device__ __forceinline__ void score_registers(Partial &acc, const DCrit &crit, const Amps &v, uint32_t m,
+__device__ __forceinline__ void score_registers(Partial &acc, const DCrit &crit, const Amps &v,
                                                 const float2 *__restrict__ ref, const LoadAt &at) {
-    const uint32_t flip0 = m & 1u;
     if (crit.kind == ARSO_CRIT_ARGMAX) {
 #pragma unroll
         for (int ri = 0; ri < 32; ++ri)
-            accumulate(acc, crit, amp_get(v, ri), ref, (uint64_t)(at(ri >> 1) + ((ri & 1) ^ flip0)));
+            accumulate(acc, crit, amp_get(v, ri), ref, (uint64_t)(at(ri >> 1) + (ri & 1)));
         return;
     }
     float2 ta[5], tb[5];  // partial sums of the tree's levels
@@ -1172,8 +1252,7 @@ __device__ __forceinline__ void score_registers(Partial &acc, const DCrit &crit,
         float2 sa, sb = make_float2(0.f, 0.f);
         if (crit.kind == ARSO_CRIT_FIDELITY) {
             const float4 w = __ldg(reinterpret_cast<const float4 *>(ref + gi));
-            const float2 rr = flip0 ? make_float2(w.z, w.x) : make_float2(w.x, w.z);
-            const float2 ri = flip0 ? make_float2(w.w, w.y) : make_float2(w.y, w.w);
+            const float2 rr = make_float2(w.x, w.z), ri = make_float2(w.y, w.w);
             sa = fma2(rr, v.re[k], mul2(ri, v.im[k]));
             sb = fma2(rr, v.im[k], mul2(make_float2(-ri.x, -ri.y), v.re[k]));
         } else {
@@ -1181,8 +1260,8 @@ __device__ __forceinline__ void score_registers(Partial &acc, const DCrit &crit,
             if (crit.kind == ARSO_CRIT_OUTCOME) in = gi == (crit.target & ~1ull) ? 1u << (crit.target & 1u) : 0u;
             else in = crit.bitmap[gi >> 5] >> (gi & 31);
             sa = fma2(v.re[k], v.re[k], mul2(v.im[k], v.im[k]));
-            sa.x = (in >> flip0) & 1u ? sa.x : 0.f;
-            sa.y = (in >> (flip0 ^ 1u)) & 1u ? sa.y : 0.f;
+            sa.x = in & 1u ? sa.x : 0.f;
+            sa.y = in & 2u ? sa.y : 0.f;
         }
 #pragma unroll
         for (int l = 0; l < 5; ++l) {
@@ -1210,16 +1289,13 @@ __device__ __forceinline__ void load_tile(Amps &v, const float2 *__restrict__ sr
         v.im[k] = make_float2(w.y, w.w);
     }
 }
-__device__ __forceinline__ void store_tile(const Amps &v, float2 *dst, uint32_t m, const LoadAt &at) {
-    const uint32_t flip0 = m & 1u;
+__device__ __forceinline__ void store_tile(const Amps &v, float2 *dst, const LoadAt &at) {
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const float2 r = flip0 ? swp2(v.re[k]) : v.re[k], i = flip0 ? swp2(v.im[k]) : v.im[k];
-        *reinterpret_cast<float4 *>(dst + at(k)) = make_float4(r.x, i.x, r.y, i.y);
-    }
+    for (int k = 0; k < 16; ++k)
+        *reinterpret_cast<float4 *>(dst + at(k)) = make_float4(v.re[k].x, v.im[k].x, v.re[k].y, v.im[k].y);
 }
 
-// v (in the load mapping, mask c.m) times the frame table (internal.h) and i^gp
+// v (in the load mapping, masks resolved but for c.m without bit 0) times the frame table (internal.h) and i^gp
 __device__ __forceinline__ void apply_frame(Amps &v, TileCtx &c, const float2 *__restrict__ frame, int t) {
     const uint32_t nt = 1u << (t - REG_BITS);
     const float4 *T = reinterpret_cast<const float4 *>(frame + nt);
@@ -1227,13 +1303,12 @@ __device__ __forceinline__ void apply_frame(Amps &v, TileCtx &c, const float2 *_
     if (c.gp & 1u) F = make_float2(-F.y, F.x);
     if (c.gp & 2u) F = make_float2(-F.x, -F.y);
     c.gp = 0;
-    const uint32_t mr = (c.m >> (t - 4)) & 15u, flip0 = c.m & 1u;
+    const uint32_t mr = (c.m >> (t - 4)) & 15u;
     const float2 fr = bc2(F.x), fi = bc2(F.y), nfi = bc2(-F.y);
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
         const float4 w = __ldg(T + ((uint32_t)k ^ mr));
-        const float2 tr = flip0 ? make_float2(w.y, w.x) : make_float2(w.x, w.y);
-        const float2 ti = flip0 ? make_float2(w.w, w.z) : make_float2(w.z, w.w);
+        const float2 tr = make_float2(w.x, w.y), ti = make_float2(w.z, w.w);
         const float2 gr = fma2(nfi, ti, mul2(fr, tr)), gi = fma2(fi, tr, mul2(fr, ti));
         const float2 ngi = make_float2(-gi.x, -gi.y);
         const float2 r = v.re[k], i = v.im[k];
@@ -1242,6 +1317,23 @@ __device__ __forceinline__ void apply_frame(Amps &v, TileCtx &c, const float2 *_
     }
 }
 
+// the signs of z, then the lanes in true order: what is left of the masks is m without bit 0
+__device__ __forceinline__ void resolve_masks(Amps &a, TileCtx &c) {
+    uint32_t mask = __popc(c.tpart & c.z) & 1 ? 0xFFFFFFFFu : 0u;
+#pragma unroll
+    for (int b = 0; b < REG_BITS; ++b)
+        if ((c.z >> rbit(c.R, b)) & 1u) mask ^= reg_pattern((uint32_t)b);
+    if (mask) negate_masked(a, mask);
+    c.z = 0;
+    if (c.m & 1u) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            a.re[k] = swp2(a.re[k]);
+            a.im[k] = swp2(a.im[k]);
+        }
+        c.m ^= 1u;
+    }
+}
 // register set of the load/store mapping {0, t-4, ..., t-1}
 __device__ __forceinline__ uint32_t load_set(int t) {
     return ((uint32_t)(t - 4) << 5) | ((uint32_t)(t - 3) << 10) | ((uint32_t)(t - 2) << 15) | ((uint32_t)(t - 1) << 20);
@@ -1249,6 +1341,7 @@ __device__ __forceinline__ uint32_t load_set(int t) {
 // the true state up to its mask, in the load mapping
 __device__ __forceinline__ void finish_tile(Amps &v, float2 *sm, TileCtx &c, const float2 *__restrict__ frame, int t) {
     if (c.R != load_set(t)) remap(v, sm, c, load_set(t), t);
+    resolve_masks(v, c);
     if (frame) apply_frame(v, c, frame, t);
     else apply_global_phase(v, c);
 }
@@ -1321,21 +1414,22 @@ __device__ __forceinline__ bool pass_source(const PassArgs &a, uint32_t slot, co
 
 // end of a pass: the tile scored against the cached state at the boundary, or stored
 __device__ __forceinline__ void pass_finish(const PassArgs &a, Amps &v, TileCtx &c, uint32_t slot, uint32_t tile,
-                                            uint32_t tiles, Partial *red) {
+                                            uint32_t base, uint32_t tiles, Partial *red) {
     const uint64_t N = 1ull << a.n;
+    resolve_masks(v, c);
     if (a.frame) apply_frame(v, c, a.frame, a.t);
     else apply_global_phase(v, c);
-    const LoadAt at = tile_at((uint32_t)tile_base(a.rest_mask, tile), a.offs, a.t, a.c, c.tid, c.m);
+    const LoadAt at = tile_at(base, a.offs, a.t, a.c, c.tid, c.m);
     if (!a.ideal && !a.store_last && a.pass == a.end_pass[slot]) {
         const float2 *ref = static_cast<const float2 *>(a.ref_cache ? a.ref_cache : a.cache) +
                             (size_t)a.cache_slot[a.pass + 1] * N;
         Partial acc = empty_partial();
-        score_registers(acc, a.crit, v, c.m, ref, at);
+        score_registers(acc, a.crit, v, ref, at);
         acc = group_reduce_partial(acc, red, c.nthr);
         if (c.tid == 0) a.partials[(size_t)slot * tiles + tile] = acc;
         return;
     }
-    store_tile(v, a.ideal ? static_cast<float2 *>(a.ideal_dst) : static_cast<float2 *>(a.work) + (size_t)slot * N, c.m, at);
+    store_tile(v, a.ideal ? static_cast<float2 *>(a.ideal_dst) : static_cast<float2 *>(a.work) + (size_t)slot * N, at);
 }
 
 // One pass over tiles of 2^t amplitudes: a CTA runs THREADS / 2^(t-5) neighbouring tiles
@@ -1347,11 +1441,12 @@ template <int THREADS, int MINB>
 __global__ void __launch_bounds__(THREADS, MINB) pass_rb_kernel(PassArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Partial red[THREADS / 32];
+    __shared__ uint32_t s_base[THREADS / 32];
     __shared__ float2 ubuf[THREADS / 32][16];
     __shared__ uint4 s_ops[2][MAX_PHASE_UNITS];
     const int t = a.t;
     TileCtx c;
-    c.m = 0;
+    c.m = c.z = 0;
     c.gp = 0;
     c.nthr = 1u << (t - REG_BITS);
     c.tid = threadIdx.x & (c.nthr - 1u);
@@ -1362,8 +1457,9 @@ __global__ void __launch_bounds__(THREADS, MINB) pass_rb_kernel(PassArgs a) {
     {
         const float2 *src;
         if (!pass_source(a, blockIdx.y, src, ev, ev_end)) return;
-        const uint32_t tile = blockIdx.x * groups + sg;
-        load_tile<false>(v, src, tile_at((uint32_t)tile_base(a.rest_mask, tile), a.offs, t, a.c, c.tid, 0u));
+        const uint32_t base = (uint32_t)tile_base(a.rest_mask, blockIdx.x * groups + sg);
+        if (c.tid == 0) s_base[sg] = base;  // for the store: the phase loop has no register to keep it
+        load_tile<false>(v, src, tile_at(base, a.offs, t, a.c, c.tid, 0u));
     }
     set_phase(c, load_set(t), t);
     uint32_t next = ev < ev_end ? *ev : NO_EVENT;
@@ -1382,7 +1478,7 @@ __global__ void __launch_bounds__(THREADS, MINB) pass_rb_kernel(PassArgs a) {
         run_prog(v, c, s_ops[buf], s_ops[buf] + (a.ph_pg[ph + 1] - a.ph_pg[ph]), mats, sm, ubuf[sg], t, ev, ev_end, next,
                  a.evs);
     }
-    pass_finish(a, v, c, blockIdx.y, blockIdx.x * groups + sg, gridDim.x * groups, red);
+    pass_finish(a, v, c, blockIdx.y, blockIdx.x * groups + sg, s_base[sg], gridDim.x * groups, red);
 }
 
 // One pass of a probe circuit (kernels.h) over a state in place: CTAs loop over the tiles,
@@ -1398,15 +1494,20 @@ __global__ void __launch_bounds__(THREADS, MINB) probe_kernel(ProbeArgs a) {
     __shared__ float2 ubuf[16];
     __shared__ uint4 s_ops[2][MAX_PHASE_UNITS];
     const int t = a.t;
+    __shared__ uint32_t s_base;
     double *row = a.rows + ((size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * a.row_len;
     for (uint32_t tile = blockIdx.x; tile < a.tiles; tile += gridDim.x) {
         TileCtx c;
-        c.m = 0;
+        c.m = c.z = 0;
         c.gp = 0;
         c.nthr = blockDim.x;
         c.tid = threadIdx.x;
         Amps v;
-        load_tile<true>(v, a.state, tile_at((uint32_t)tile_base(a.rest_mask, tile), a.offs, t, a.c, c.tid, 0u));
+        {
+            const uint32_t base = (uint32_t)tile_base(a.rest_mask, tile);
+            if (c.tid == 0) s_base = base;
+            load_tile<true>(v, a.state, tile_at(base, a.offs, t, a.c, c.tid, 0u));
+        }
         set_phase(c, load_set(t), t);
         if (a.pb < a.pe)
             stage_units(s_ops[0], a.prog + a.ph_pg[a.pb], a.ph_pg[a.pb + 1] - a.ph_pg[a.pb], threadIdx.x, blockDim.x);
@@ -1427,8 +1528,10 @@ __global__ void __launch_bounds__(THREADS, MINB) probe_kernel(ProbeArgs a) {
                 u += h.x >> 24;  // a probe circuit has no fused runs
             }
         }
+        resolve_masks(v, c);
         if (a.frame) apply_frame(v, c, a.frame, t);
-        store_tile(v, a.state, c.m, tile_at((uint32_t)tile_base(a.rest_mask, tile), a.offs, t, a.c, c.tid, c.m));
+        else apply_global_phase(v, c);
+        store_tile(v, a.state, tile_at(s_base, a.offs, t, a.c, c.tid, c.m));
         __syncthreads();  // the shared memory is reused by the next tile
     }
 }
@@ -1490,7 +1593,7 @@ __global__ void __launch_bounds__(512, 1) pass_tensor_kernel(PassArgs a) {
     __shared__ uint4 s_ops[2][2 * MAX_PHASE_OPS];
     const int t = a.t;
     TileCtx c;
-    c.m = 0;
+    c.m = c.z = 0;
     c.gp = 0;
     c.tid = threadIdx.x;
     c.nthr = blockDim.x;
@@ -1561,7 +1664,7 @@ __global__ void __launch_bounds__(512, 1) pass_tensor_kernel(PassArgs a) {
         tmem_free(tmem, nblk * 128u);
     }
     if (c.R != load_set(t)) remap(v, sm, c, load_set(t), t);
-    pass_finish(a, v, c, blockIdx.y, blockIdx.x, gridDim.x, red);
+    pass_finish(a, v, c, blockIdx.y, blockIdx.x, (uint32_t)tile_base(a.rest_mask, blockIdx.x), gridDim.x, red);
 }
 
 // ------------------------------------------------------------- resident ---
@@ -1576,8 +1679,10 @@ __global__ void __launch_bounds__(512, 1) pass_tensor_kernel(PassArgs a) {
 __device__ __forceinline__ void rb_store_linear(Amps &v, float2 *sm, TileCtx &c, float2 *dst, int t,
                                                 const float2 *__restrict__ frame) {
     if (c.R != load_set(t)) remap(v, sm, c, load_set(t), t);
+    resolve_masks(v, c);
     if (frame) apply_frame(v, c, frame, t);
-    store_tile(v, dst, c.m, linear_at(t, c.tid, c.m));
+    else apply_global_phase(v, c);
+    store_tile(v, dst, linear_at(t, c.tid, c.m));
 }
 
 template <int MODE>
@@ -1595,7 +1700,7 @@ __global__ void __launch_bounds__(512, 1) resident_rb_kernel(ResidentArgs a) {
     for (uint64_t b = blockIdx.x; b < count; b += gridDim.x) {
         Amps v;
         TileCtx c;
-        c.m = 0;
+        c.m = c.z = 0;
         c.gp = 0;
         c.tid = threadIdx.x;
         c.nthr = blockDim.x;
@@ -1657,7 +1762,7 @@ __global__ void __launch_bounds__(512, 1) resident_rb_kernel(ResidentArgs a) {
             finish_tile(v, sm, c, frame_end, t);
             const float2 *ref = cache + (size_t)(a.n_ckpt - 1) * N;
             Partial acc = empty_partial();
-            score_registers(acc, a.crit, v, c.m, ref, linear_at(t, c.tid, c.m));
+            score_registers(acc, a.crit, v, ref, linear_at(t, c.tid, c.m));
             acc = block_reduce_partial(acc, red);
             if (threadIdx.x == 0) {
                 const double sc = finish_score(a.crit, acc);
@@ -1707,7 +1812,7 @@ __device__ __forceinline__ void batch_item(const BatchItem &it, const BatchCircu
     const bool active = sg < it.count;
     const uint64_t tr = ids[it.off + (active ? sg : 0)];
     TileCtx c;
-    c.m = 0;
+    c.m = c.z = 0;
     c.gp = 0;
     c.tid = threadIdx.x % gsize;
     c.nthr = gsize;
@@ -1734,7 +1839,7 @@ __device__ __forceinline__ void batch_item(const BatchItem &it, const BatchCircu
     finish_tile(v, sm, c, C.frame + (size_t)(C.n_ckpt - 1) * frame_floats2(t), t);
     const float2 *ref = C.cache + (size_t)(C.n_ckpt - 1) * N;
     Partial acc = empty_partial();
-    score_registers(acc, C.crit, v, c.m, ref, linear_at(t, c.tid, c.m));
+    score_registers(acc, C.crit, v, ref, linear_at(t, c.tid, c.m));
     acc = group_reduce_partial(acc, red, gsize);
     if (c.tid == 0 && active) {
         const double sc = finish_score(C.crit, acc);
@@ -2003,7 +2108,7 @@ __device__ __forceinline__ void mix_tile(const MixArgs &A, const MixStream &S, c
         ev = lo;
     }
     TileCtx c;
-    c.m = 0;
+    c.m = c.z = 0;
     c.gp = 0;
     c.tid = threadIdx.x;
     c.nthr = blockDim.x;
@@ -2033,11 +2138,11 @@ __device__ __forceinline__ void mix_tile(const MixArgs &A, const MixStream &S, c
     if (scored) {
         const float2 *ref = S.ref_cache + (size_t)S.cache_slot[j + 1] * N;
         Partial acc = empty_partial();
-        score_registers(acc, S.crit, v, c.m, ref, at);
+        score_registers(acc, S.crit, v, ref, at);
         acc = group_reduce_partial(acc, red, MIX_THREADS);
         if (threadIdx.x == 0) S.partials[(size_t)k * S.tiles + it.tile] = acc;
     } else {
-        store_tile(v, S.work + (size_t)T.slot * N, c.m, at);
+        store_tile(v, S.work + (size_t)T.slot * N, at);
     }
     // publish: the barrier orders every thread's stores before thread 0's fence and
     // counter increments (the release the waiting CTAs acquire)
@@ -2157,7 +2262,8 @@ void prepare_pass_rb() {
 // (device time of all pass launches): 12-qubit tiles, 24-qubit brickwork, 177 trajectories:
 // five 128-thread CTAs 342 ms, four 353, two tiles in a 256-thread CTA 353 (three per SM) or
 // 376 (two); 13-qubit tiles: three CTAs per SM 6.53 ms against 6.87 with two (16-qubit
-// brickwork, 2,000 trajectories) and 3.12 against 3.41 (20-qubit adder, 500).
+// brickwork, 2,000 trajectories) and 3.12 against 3.41 (20-qubit adder, 500); both sides
+// before the fused runs and the z mask (305 ms, 6.0 ms and 1.7 ms since).
 void launch_pass_rb(const PassArgs &a, bool last, uint32_t slots, double bytes, cudaStream_t st, double flops,
                     double smem_bytes) {
     ProfScope ps_(last && !a.store_last ? ARSO_K_PASS_LAST : ARSO_K_PASS, bytes, st, flops, smem_bytes);
