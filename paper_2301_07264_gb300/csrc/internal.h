@@ -234,10 +234,12 @@ struct Criterion {
     std::vector<uint64_t> set;
 };
 
-// pool.cpp: memory of the library's pool. pool_alloc: usable on `st` from there on;
+// pool.cpp: memory of the library's pools. pool_alloc: usable on `st` from there on and freed
+// on `st`; pool_alloc_list: the same for memory that pool_free_idle frees;
 // pool_alloc_now: usable on any stream after the call; pool_free_idle: no work that uses
 // the memory may be pending.
 void *pool_alloc(size_t bytes, cudaStream_t st);
+void *pool_alloc_list(size_t bytes, cudaStream_t st);
 void *pool_alloc_now(size_t bytes);
 void pool_free_idle(void *ptr) noexcept;
 // circuits and surrogates alive: with the last one freed the pool's memory goes back
@@ -280,7 +282,7 @@ struct ListBuffer {
     ~ListBuffer() { pool_free_idle(ptr); }
     void ensure(size_t b, cudaStream_t st) {  // once; usable on st
         if (ptr) throw Error(ARSO_EINVAL, "internal: a list buffer is allocated once");
-        ptr = pool_alloc(b, st);
+        ptr = pool_alloc_list(b, st);
         bytes = b;
     }
     template <typename T> T *as() const { return static_cast<T *>(ptr); }
