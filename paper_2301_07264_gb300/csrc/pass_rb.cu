@@ -1013,6 +1013,7 @@ __device__ __forceinline__ void run_gates(Amps &v, TileCtx &c, uint32_t g, uint3
 // The macro-ops [u, ue) of one phase with the Pauli events that fall inside them. An X
 // or Y error would turn the frame's diag(1, phi) on its qubit into diag(phi, 1);
 // diag(phi, conj phi) on the flipped state keeps the frame the same for every trajectory.
+// (The float cosine of a phase below 2.4e-4 is 1: both parts of phi tell whether it is.)
 __device__ __forceinline__ void run_prog(Amps &v, TileCtx &c, const uint4 *u, const uint4 *ue,
                                          const float2 *__restrict__ mats, float2 *sm, float2 *ubuf, int t,
                                          const uint32_t *&ev, const uint32_t *ev_end, uint32_t &next,
@@ -1037,7 +1038,7 @@ __device__ __forceinline__ void run_prog(Amps &v, TileCtx &c, const uint4 *u, co
             }
             if (pc & 1u) c.m ^= 1u << q;
             if (pc == 3u) c.gp = (c.gp + 1u) & 3u;  // Y = i X Z
-            if ((pc & 1u) && e.x != 1.f) phase_pair(v, ~bit_mask(c, q), make_float2(e.x, e.y));
+            if ((pc & 1u) && (e.x != 1.f || e.y != 0.f)) phase_pair(v, ~bit_mask(c, q), make_float2(e.x, e.y));
             ++ev;
             next = ev < ev_end ? *ev : NO_EVENT;
         }
