@@ -451,11 +451,17 @@ struct FusedRun {
     cd d[8];            // |x> -> d[x] |x ^ flip>
 };
 
+// A run counts as such within RUN_TOL: above the rounding of a product of 40 matrices (a few
+// 1e-15), and far below what FP32 amplitudes resolve of a small rotation's own amplitude. What
+// was accepted is written with ten times that, so a value at the edge cannot fail there.
+constexpr double RUN_TOL = 1e-13;
+
 static uint32_t run_target(const FusedRun &r, uint32_t x) { return r.c >= 0 && (r.f >> x & 1) ? x ^ (1u << r.c) : x; }
 
 // the phases of a run between the frames phi (in) and out: residual signs by new value y, or,
 // without a flip and on two qubits, theta of one parity phase. False: neither.
-static bool run_phases(const FusedRun &r, const cd *phi, cd &S, cd *out, uint32_t &signs, double &theta) {
+static bool run_phases(const FusedRun &r, const cd *phi, cd &S, cd *out, uint32_t &signs, double &theta,
+                       double tol = RUN_TOL) {
     const uint32_t N = 1u << r.n;
     cd e[8];
     for (uint32_t x = 0; x < N; ++x) {
@@ -478,8 +484,8 @@ static bool run_phases(const FusedRun &r, const cd *phi, cd &S, cd *out, uint32_
         for (int k = 0; k < r.n; ++k)
             if (y >> k & 1) v *= out[k];
         res[y] = e[y] / v;
-        if (std::abs(res[y] + 1.0) < 1e-9) signs |= 1u << y;
-        else ok &= std::abs(res[y] - 1.0) < 1e-9;
+        if (std::abs(res[y] + 1.0) < tol) signs |= 1u << y;
+        else ok &= std::abs(res[y] - 1.0) < tol;
     }
     if (ok) return true;
     if (r.c >= 0 || r.n != 2) return false;
@@ -518,7 +524,7 @@ static void run_apply(cd (*M)[8], const uint32_t *q, int n, const HostGate &h) {
 }
 
 // the gates as a fused run; false when their product is none
-static bool run_of(const cd (*M)[8], FusedRun &r) {
+static bool run_of(const cd (*M)[8], FusedRun &r, double tol = RUN_TOL) {
     const uint32_t N = 1u << r.n;
     uint32_t to[8];
     for (uint32_t x = 0; x < N; ++x) {
@@ -526,9 +532,9 @@ static bool run_of(const cd (*M)[8], FusedRun &r) {
         for (uint32_t y = 0; y < N; ++y) {
             const double a = std::abs(M[x][y]);
             if (a > 0.5) hit = hit < 0 ? (int)y : 8;
-            else if (a > 1e-9) return false;
+            else if (a > tol) return false;
         }
-        if (hit < 0 || hit >= 8 || std::abs(std::abs(M[x][hit]) - 1.0) > 1e-9) return false;
+        if (hit < 0 || hit >= 8 || std::abs(std::abs(M[x][hit]) - 1.0) > tol) return false;
         to[x] = (uint32_t)hit;
         r.d[x] = M[x][hit];
         snap(r.d[x]);
@@ -545,7 +551,7 @@ static bool run_of(const cd (*M)[8], FusedRun &r) {
     cd S, out[3];
     uint32_t signs;
     double theta;
-    return run_phases(r, one, S, out, signs, theta);
+    return run_phases(r, one, S, out, signs, theta, tol);
 }
 
 // what a gate costs the kernels: 2 when it is dispatched, 1 when it may be (a phase that has
@@ -561,8 +567,8 @@ static int run_cost(const HostGate &h) {
 // gates that no run takes: measurements, and those that run through shared memory
 static bool run_takes(const HostGate &h) { return h.cls != GC_PROBE && h.cls != GC_DENSE2 && h.cls != GC_SWAP; }
 
-static bool product_of(const arso_circuit *c, const std::vector<const HostGate *> &gs, FusedRun &r) {
-    (void)c;
+// the run that find_units accepted, from its gates
+static bool product_of(const std::vector<const HostGate *> &gs, FusedRun &r) {
     r.n = 0;
     for (const HostGate *h : gs)
         for (uint32_t q : {h->q0, h->q1})
@@ -571,7 +577,7 @@ static bool product_of(const arso_circuit *c, const std::vector<const HostGate *
     for (uint32_t x = 0; x < 8; ++x)
         for (uint32_t y = 0; y < 8; ++y) M[x][y] = x == y ? 1.0 : 0.0;
     for (const HostGate *h : gs) run_apply(M, r.q, r.n, *h);
-    return run_of(M, r);
+    return run_of(M, r, 10 * RUN_TOL);
 }
 
 // The pass's gates (indices from its first position) as units in an order that keeps the
@@ -890,8 +896,11 @@ struct Frame {
 // scale with a full matrix: G(x) grows a state by sqrt(1 + |x|^2) <= sqrt 2, so FP32's
 // range would end after some 250 gates; 2^40 keeps 2^86 of headroom above it.
 constexpr double FRAME_GROWTH = 1.0 / (1ull << 40);
-// a matrix counts as unitary (and its frame form as exact) within this
-constexpr double UNITARY_TOL = 1e-12;
+// a matrix counts as unitary within UNITARY_TOL, its rows as orthogonal within ORTHO_TOL of
+// the smaller entry (the frame form derives the second row from the first, so that a tiny
+// rotation keeps its own amplitude), and an entry as zero within the rounding of the sine or
+// cosine of a right angle
+constexpr double UNITARY_TOL = 1e-12, ORTHO_TOL = 1e-9, ZERO_TOL = 4.5e-16;
 
 // What a one-qubit gate becomes in a frame.
 struct FrameGate {
@@ -904,11 +913,12 @@ struct FrameGate {
 // U on a qubit with frame phase phi: what remains of it, and the frame after it
 static FrameGate frame_dense(Frame &F, uint32_t q, const cd *u) {
     const cd phi = F.phi(q);
-    const cd u00 = u[0], u01 = u[1] * phi, u10 = u[2], u11 = u[3] * phi;
+    cd u00 = u[0], u01 = u[1] * phi, u10 = u[2], u11 = u[3] * phi;
+    if (std::abs(u01) < ZERO_TOL && std::abs(u10) < ZERO_TOL) u01 = u10 = 0;
+    if (std::abs(u00) < ZERO_TOL && std::abs(u11) < ZERO_TOL) u00 = u11 = 0;
     const double a = std::abs(u00), b = std::abs(u01);
-    const bool unitary = std::abs(a * a + b * b - 1.0) < UNITARY_TOL && std::abs(std::abs(u10) - b) < UNITARY_TOL &&
-                         std::abs(std::abs(u11) - a) < UNITARY_TOL &&
-                         std::abs(u00 * std::conj(u10) + u01 * std::conj(u11)) < UNITARY_TOL;
+    const bool unitary = std::abs(a * a + b * b - 1.0) < UNITARY_TOL && std::abs(std::norm(u10) + std::norm(u11) - 1.0) < UNITARY_TOL &&
+                         std::abs(u00 * std::conj(u10) + u01 * std::conj(u11)) <= ORTHO_TOL * std::min(a, b);
     FrameGate g;
     auto full = [&](cd m00, cd m01, cd m10, cd m11) {
         g.kind = FrameGate::FULL;
@@ -919,13 +929,13 @@ static FrameGate frame_dense(Frame &F, uint32_t q, const cd *u) {
         F.phi(q) = 1;
         return g;
     }
-    if (b < UNITARY_TOL) {  // diagonal
+    if (b == 0.0) {  // diagonal
         F.S() *= u00;
         F.phi(q) = u11 / u00;
         snap(F.phi(q));
         return g;
     }
-    if (a < UNITARY_TOL) {  // diag(u01, u10) X
+    if (a == 0.0) {  // diag(u01, u10) X
         F.S() *= u01;
         F.phi(q) = u10 / u01;
         snap(F.phi(q));
@@ -1116,7 +1126,7 @@ static void emit_run(arso_circuit *c, ProgWriter &W, Frame &F, const std::vector
     std::vector<const HostGate *> gs;
     for (uint32_t p = pos; p < end; ++p) gs.push_back(&c->gates[c->perm[p]]);
     FusedRun r;
-    ARSO_REQUIRE(product_of(c, gs, r), "internal: a fused run that is none");
+    ARSO_REQUIRE(product_of(gs, r), "internal: a fused run that is none");
     uint32_t q[3] = {0, 0, 0}, p[3] = {15, 15, 15};  // tile bits and register positions
     for (int k = 0; k < r.n; ++k) q[k] = (uint32_t)local[r.q[k]];
     for (uint32_t i = pos; i < end; ++i) {
@@ -1132,7 +1142,7 @@ static void emit_run(arso_circuit *c, ProgWriter &W, Frame &F, const std::vector
     for (int k = 0; k < r.n; ++k) phi[k] = F.phi(q[k]);
     uint32_t signs = 0;
     double theta = 0.0;
-    ARSO_REQUIRE(run_phases(r, phi, S, out, signs, theta), "internal: a fused run's phases");
+    ARSO_REQUIRE(run_phases(r, phi, S, out, signs, theta, 10 * RUN_TOL), "internal: a fused run's phases");
     // terms of the flip over (a, b), the other two qubits, and of the signs over (a, b, c)
     const int ci = r.c >= 0 ? r.c : r.n - 1;
     int ab[2] = {ci, ci}, m = 0;

@@ -40,3 +40,19 @@ def test_errors_on_small_phases(n, tile, angle):
     got = out.cpu().numpy()
     for k, ev in enumerate(lists):
         assert np.linalg.norm(got[k] - statevector.simulate(circ, ev)) < 2e-5, ev
+
+
+# one rotation's own amplitude, far below what the rest of the state rounds to
+@pytest.mark.parametrize("n,tile", [(10, 0), (14, 12)])
+@pytest.mark.parametrize("fused,angle", [(False, 1e-6), (False, 1e-9), (False, 1e-12), (False, 1e-14),
+                                         (True, 1e-6), (True, 1e-9), (True, 1e-12)])
+def test_tiny_rotations_keep_their_amplitude(n, tile, fused, angle):
+    from paper_2301_07264_gb300 import arso
+    g = [W.Gate("RX", (1,), (angle,))]
+    if fused:  # between CX gates that a run would take it with
+        g = [W.Gate("CX", (0, 1))] + g + [W.Gate("CX", (0, 1)), W.Gate("CX", (1, 0))]
+    cc = arso.compile_circuit(n, g, tile_qubits=tile)
+    out = torch.empty(1 << n, dtype=torch.complex64, device="cuda")
+    arso.reference_state(cc, out)
+    got = complex(out[3 if fused else 2].item())
+    assert abs(got / (-1j * np.sin(angle / 2)) - 1) < 1e-6, got
