@@ -69,6 +69,11 @@ template <typename T> static void h2d(void *dst, const std::vector<T> &v, cudaSt
 }
 
 // ------------------------------------------------------------ upload -------
+// A copy from pageable memory may return before it has reached the device, and a non-blocking
+// stream does not wait for the legacy stream that carries it: tables copied
+// with cudaMemcpy are waited for before any kernel can read them.
+static void uploads_done() { ARSO_CUDA(cudaStreamSynchronize(cudaStreamLegacy)); }
+
 // tables of the frames (one per pass, or per checkpoint of a resident circuit)
 static void upload_frames(arso_circuit *c, const std::vector<std::vector<std::complex<double>>> &fr) {
     const int t = (int)c->tile_qubits;
@@ -198,6 +203,7 @@ static void upload_circuit(arso_circuit *c) {
             ARSO_CUDA(cudaMemcpy(c->d_phase_of_pos.ptr, c->phase_of_pos.data(), c->phase_of_pos.size() * 4,
                                  cudaMemcpyHostToDevice));
     }
+    uploads_done();
 }
 
 // resident arguments common to every launch
@@ -288,6 +294,7 @@ static void ensure_cache(arso_circuit *c, cudaStream_t st) {
             std::vector<std::vector<std::complex<double>>> fr;
             for (uint64_t k = 0; k < c->n_ckpt; ++k) fr.push_back(c->frame[std::min<uint64_t>(k * every, units)]);
             upload_frames(c, fr);
+            uploads_done();
         }
         launch_resident_any(c, resident_args(c), 2, (double)c->n_ckpt * sb, st);
     } else {

@@ -647,6 +647,7 @@ static void upload_norm(arso_surrogate *s) {
     std::memcpy(h + IN, s->sd, sizeof(s->sd));
     s->norm.ensure(sizeof(h));
     ARSO_CUDA(cudaMemcpy(s->norm.ptr, h, sizeof(h), cudaMemcpyHostToDevice));
+    ARSO_CUDA(cudaStreamSynchronize(cudaStreamLegacy));  // the copy may still be under way (api.cu, uploads_done)
 }
 
 // forward of `rows` gathered rows: xb -> h1 -> h2 -> z (logits); the output layer

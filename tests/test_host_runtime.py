@@ -1,0 +1,65 @@
+"""The library's host side against a runtime without a GPU (fake_cuda.cpp): what is waited for
+before memory is read or freed."""
+import ctypes as C
+
+import pytest
+
+from paper_2301_07264_gb300 import arso
+from workloads import circuits as W
+
+import fake_cuda  # noqa: E402  (beside this file)
+
+
+@pytest.fixture(scope="module")
+def library(tmp_path_factory):
+    return fake_cuda.load(tmp_path_factory.mktemp("fake"))
+
+
+@pytest.fixture
+def lib(library):
+    library.fake_fail_at(-1)
+    library.fake_device(0)
+    library.fake_reset_counts()
+    return library
+
+
+def ok(lib, status):
+    assert status == arso.OK, lib.arso_last_error().decode()
+
+
+def compiled(lib, circ, tile=0, flags=0):
+    arr, keep = arso._gates_array(circ.gates)
+    h = C.c_void_p()
+    o = arso.CompileOpts(0, tile, 0, 0, 0, flags)
+    ok(lib, lib.arso_compile_circuit(circ.n, arr, len(circ.gates), C.byref(o), C.byref(h)))
+    return h
+
+
+def sampled(lib, cc, stream, n=8):
+    e = C.c_void_p()
+    ok(lib, lib.arso_sample_errors(cc, 0.01, 0.01, 0.01, 1, 0, n, stream, C.byref(e)))
+    return e
+
+
+# resident, streaming on 13- and 12-qubit tiles, tensor phases
+CIRCUITS = [(W.brickwork(11, 6, 1), 0, 0), (W.brickwork(14, 6, 1), 0, 0), (W.qaoa_maxcut(14, 1), 12, 0),
+            (W.brickwork(14, 6, 1), 12, arso.OPT_TENSOR_PHASES)]
+
+
+@pytest.mark.parametrize("k", range(len(CIRCUITS)))
+@pytest.mark.parametrize("kind", ["fidelity", "outcome"])
+def test_uploads_are_done_before_kernels_of_other_streams(lib, k, kind):
+    # a copy from pageable memory returns before it has reached the device, and a stream that
+    # does not wait for the legacy stream would read what was there
+    st = lib.fake_stream(0)
+    crit = arso.make_criterion(W.Criterion(kind, target=1, threshold=0.5))
+    cc = compiled(lib, *CIRCUITS[k])
+    e = sampled(lib, cc, st)
+    score = (C.c_double * 8)()
+    ok(lib, lib.arso_run_trajectories(cc, e, C.byref(crit), st, score, None))
+    P = (C.c_double * 4)()
+    ok(lib, lib.arso_exhaustive(cc, C.byref(crit), st, P, None))
+    lib.arso_error_list_free(e)
+    lib.arso_circuit_free(cc)
+    assert lib.fake_launches(b"kernel") > 0
+    assert lib.fake_violation(0) == 0
