@@ -2001,11 +2001,16 @@ arso_status arso_autotune(uint32_t n_qubits, const arso_gate *gates, size_t n_ga
         ARSO_CUDA(cudaEventCreate(&e1));
         double best_ms = INFINITY;
         size_t best_i = 0;
+        // counted as a handle: the pools keep their memory from one candidate to the next
+        struct Counted {
+            Counted() { handle_made(); }
+            ~Counted() { handle_freed(); }
+        } counted;
         for (size_t i = 0; i < cands.size(); ++i) {
             arso_circuit *c = nullptr;
             arso_status s1 = arso_compile_circuit(n_qubits, gates, n_gates, &cands[i], &c);
             if (s1 != ARSO_OK) throw Error(s1, arso_last_error());
-            std::unique_ptr<arso_circuit> hold(c);
+            std::unique_ptr<arso_circuit, void (*)(arso_circuit *)> hold(c, arso_circuit_free);
             DevCrit dc;
             make_crit(c, crit, dc, st);
             Scratch sc(st, n_traj * 8);

@@ -63,3 +63,15 @@ def test_uploads_are_done_before_kernels_of_other_streams(lib, k, kind):
     lib.arso_circuit_free(cc)
     assert lib.fake_launches(b"kernel") > 0
     assert lib.fake_violation(0) == 0
+
+
+def test_autotune_leaves_no_handle_counted(lib):
+    # with the last handle the pools' memory goes back, whether or not one was made by autotune
+    arr, keep = arso._gates_array(CIRCUITS[1][0].gates)
+    crit, best, ms, n = arso.make_criterion(W.Criterion("fidelity")), arso.CompileOpts(), (C.c_double * 16)(), C.c_uint32()
+    ok(lib, lib.arso_autotune(14, arr, len(CIRCUITS[1][0].gates), C.byref(crit), C.c_double(1e-3), C.c_uint64(4),
+                              C.c_uint64(0), None, lib.fake_stream(0), C.byref(best), ms, C.byref(n)))
+    assert n.value > 1
+    before = lib.fake_trims()
+    lib.arso_circuit_free(compiled(lib, *CIRCUITS[0]))
+    assert lib.fake_trims() == before + 2  # both pools
