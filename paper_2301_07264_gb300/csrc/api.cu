@@ -1000,43 +1000,60 @@ static McOut mc_run_memo(arso_circuit *c, const DevCrit &dc, double p, uint64_t 
 // circuit maps psi_g to psi_R). Scores in the exhaustive order (X block, Z
 // block, Y block, each in location order). Returns false where the sweep is
 // not available (streaming complex128), leaving the trajectory route.
-// The sums of every slot of c's probe circuit (kernels.h), swept over `state` in place;
-// passes share a launch of the row sum while their rows fit PROBE_BYTES.
+// The sums of every slot of the probe circuit P (kernels.h), swept over `state` in place.
+// Launches share one sum of their rows while those fit PROBE_BYTES; a pass whose rows do not
+// is cut between phases (the state is stored in its frame there, masks applied), so that the
+// scratch stays bounded however deep a pass is.
 static void run_probes(const arso_circuit *P, bool dual, float2 *state, cudaStream_t st, std::vector<double> &sums) {
     constexpr size_t PROBE_BYTES = 256ull << 20;
-    const uint32_t per = dual ? PROBE_SUMS_DUAL : PROBE_SUMS, n_pass = (uint32_t)P->passes.size();
+    const uint32_t per = dual ? PROBE_SUMS_DUAL : PROBE_SUMS;
     const uint32_t tiles = 1u << (P->n - P->tile_qubits), n_rows = probe_rows((int)P->tile_qubits, tiles, dual);
     sums.assign((size_t)per * P->probe_slots.size() + 1, 0.0);
     Scratch d_sums(st, sums.size() * 8);
-    for (uint32_t j0 = 0; j0 < n_pass;) {
-        uint32_t j1 = j0 + 1;
-        auto len = [&](uint32_t j) { return per * (P->probe_first[j] - P->probe_first[j0]); };
-        while (j1 < n_pass && (size_t)len(j1 + 1) * n_rows * 8 <= PROBE_BYTES) ++j1;
-        const size_t bytes = std::max<size_t>((size_t)len(j1) * n_rows * 8, 8);
+    struct Part {
+        uint32_t pass, pb, pe;  // phases [pb, pe) of the pass
+    };
+    std::vector<Part> parts;    // of one sum of rows, from phase `first` on
+    uint32_t first = 0;
+    auto flush = [&](uint32_t end) {  // the slots of phases [first, end)
+        const std::vector<uint32_t> &at = P->probe_first;
+        const uint32_t len = per * (at[end] - at[first]);
+        const size_t bytes = std::max<size_t>((size_t)len * n_rows * 8, 8);
         Scratch rows(st, bytes);
         ARSO_CUDA(cudaMemsetAsync(rows.ptr, 0, bytes, st));
-        for (uint32_t j = j0; j < j1; ++j) {
-            const PassArgs p = pass_args(P, j);
+        for (const Part &q : parts) {
+            const PassArgs p = pass_args(P, q.pass);
             ProbeArgs a{};
             a.n = p.n, a.t = p.t, a.c = p.c;
             a.tiles = tiles;
             a.rest_mask = p.rest_mask;
             a.offs = p.offs;
             a.state = state;
-            a.pb = P->passes[j].pb, a.pe = P->passes[j].pe;
+            a.pb = q.pb, a.pe = q.pe;
             a.ph_R = P->d_ph_R.as<uint32_t>();
             a.ph_pg = P->d_ph_pg.as<uint32_t>();
             a.prog = P->d_prog.as<uint4>();
             a.mats = P->d_rmats.as<float2>();
-            a.frame = pass_frame(P, j);
-            a.rows = rows.as<double>() + len(j);
-            a.row_len = len(j1);
+            a.frame = q.pe == P->passes[q.pass].pe ? pass_frame(P, q.pass) : nullptr;
+            a.rows = rows.as<double>();
+            a.row_len = len;
+            a.slot0 = at[first];
             launch_probe(a, dual, st);
         }
-        launch_probe_sum(rows.as<double>(), n_rows, len(j1), d_sums.as<double>() + (size_t)per * P->probe_first[j0], st);
+        launch_probe_sum(rows.as<double>(), n_rows, len, d_sums.as<double>() + (size_t)per * at[first], st);
         ARSO_CUDA(cudaStreamSynchronize(st));
-        j0 = j1;
+        parts.clear();
+        first = end;
+    };
+    for (uint32_t j = 0; j < P->passes.size(); ++j) {
+        for (uint32_t ph = P->passes[j].pb; ph < P->passes[j].pe; ++ph) {
+            const size_t len = (size_t)per * (P->probe_first[ph + 1] - P->probe_first[first]);
+            if (ph > first && len * n_rows * 8 > PROBE_BYTES) flush(ph);
+            if (parts.empty() || parts.back().pass != j) parts.push_back({j, ph, ph});
+            parts.back().pe = ph + 1;
+        }
     }
+    flush((uint32_t)P->ph_R.size());
     copy_d2h(sums.data(), d_sums.ptr, (sums.size() - 1) * 8, st);
     ARSO_CUDA(cudaStreamSynchronize(st));
 }

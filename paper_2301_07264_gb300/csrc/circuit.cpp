@@ -976,12 +976,11 @@ struct ProgWriter {
     uint32_t probes = 0;             // register positions being measured (open is false then)
     ProbeSlot probe[REG_BITS];
     std::vector<ProbeSlot> *slots = nullptr;
-    size_t slot0 = 0;                // the pass's first slot
     explicit ProgWriter(std::vector<uint4> &o) : out(o), first(o.size()) {}
     void close() {
         if (probes) {
             last = out.size();
-            out.push_back(make_uint4(OP_PROBE | probes << 8 | 1u << 24, end, (uint32_t)(slots->size() - slot0), 0));
+            out.push_back(make_uint4(OP_PROBE | probes << 8 | 1u << 24, end, (uint32_t)slots->size(), 0));
             for (int p = 0; p < REG_BITS; ++p)
                 if (probes >> p & 1) slots->push_back(probe[p]);
             probes = 0;
@@ -1234,13 +1233,12 @@ static void reg_program(arso_circuit *c) {
         std::vector<int> local(c->n, -1);
         for (size_t i = 0; i < ps.tile_qubits.size(); ++i) local[ps.tile_qubits[i]] = (int)i;
         Frame F(c->tile_qubits);
-        c->probe_first.push_back((uint32_t)c->probe_slots.size());
         for (uint32_t ph = ps.pb; ph < ps.pe; ++ph) {
             if (c->engine == 0) c->frame.push_back(F.f);
             c->ph_pg.push_back((uint32_t)c->prog.size());
+            c->probe_first.push_back((uint32_t)c->probe_slots.size());
             ProgWriter W(c->prog);
             W.slots = &c->probe_slots;
-            W.slot0 = c->probe_first.back();
             auto gate = [&](uint32_t pos) {
                 const HostGate &h = c->gates[c->perm[pos]];
                 const uint32_t q0 = (uint32_t)local[h.q0], q1 = (uint32_t)local[h.q1];

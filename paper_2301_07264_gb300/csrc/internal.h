@@ -145,8 +145,8 @@ enum RegOpCode : uint32_t {
 //   OP_BLOCK: the gates [.., end) fused: z = units after this header and its fused macro-op
 //           that hold the gates one by one. A trajectory with an error event among the gates
 //           runs those, the others the fused macro-op; both end in the same frame
-//   OP_PROBE: bits 8-12 of x the register positions measured, z the first one's slot in
-//           its pass; the slots follow in order of position
+//   OP_PROBE: bits 8-12 of x the register positions measured, z the first one's slot; the
+//           slots follow in order of position
 // Frames: the true state is S * prod_q diag(1, phi_q) * X^m Z^z * stored, with the scalar S
 // and the unit phases phi_q the same for every trajectory and tracked on the host in FP64
 // from gate to gate (reg_program in circuit.cpp), and the masks m and z kept by the kernel:
@@ -220,7 +220,7 @@ struct Pass {
     uint32_t end_remap = 0;            // 1 if the last phase's set differs from the load layout
 };
 
-// One measurement of a probe circuit, in the order of the passes' slots.
+// One measurement of a probe circuit, in the order of the phases' slots.
 struct ProbeSlot {
     uint32_t loc;               // error location
     std::complex<double> phi;   // frame phase of its qubit
@@ -385,7 +385,7 @@ struct arso_circuit {
     std::unique_ptr<arso_circuit> probe, probe_dual;
     std::vector<arso::ProbeSlot> probe_slots;   // of a probe circuit
     std::vector<uint32_t> probe_loc;            // of a probe circuit: location of a GC_PROBE gate
-    std::vector<uint32_t> probe_first;          // of a probe circuit: pass -> its first slot (plus a sentinel)
+    std::vector<uint32_t> probe_first;          // of a probe circuit: phase -> its first slot (plus a sentinel)
     size_t state_bytes() const { return (size_t(1) << n) * (precision == ARSO_C128 ? 16 : 8); }
 };
 

@@ -263,7 +263,7 @@ void launch_dual_expect_resident(const DGate *adj, const void *mats, uint32_t G,
                                  cudaStream_t st);
 
 // Both sweeps of a streaming complex64 circuit, as passes of its probe circuit (build_probe)
-// over one state in place. Every warp adds its sums of the pass's slots, PROBE_SUMS (6 with
+// over one state in place. Every warp adds its sums of the phases' slots, PROBE_SUMS (6 with
 // the dual circuit) values each, to its own row of `rows` (zeroed before); launch_probe_sum
 // adds the rows in order. The raw sums of a measured qubit, per slot, over the pairs (s0, s1)
 // of stored amplitudes along it: |s0|^2 - |s1|^2, Re and Im of conj(s0) s1; dual, with psi in
@@ -282,6 +282,7 @@ struct ProbeArgs {
     const float2 *mats, *frame;
     double *rows;
     uint32_t row_len;   // doubles per row
+    uint32_t slot0;     // the rows' first slot
 };
 uint32_t probe_rows(int t, uint32_t tiles, bool dual);  // rows of one launch
 void launch_probe(const ProbeArgs &a, bool dual, cudaStream_t st);

@@ -797,7 +797,8 @@ template <int P> __device__ __forceinline__ void rg_probe_dual(const Amps &a, ui
 // The measurements of one OP_PROBE: the values of all positions summed over the warp by
 // halving exchanges (one shuffle per value instead of five), then added to the warp's row,
 // one value per lane (pair of lanes).
-template <bool DUAL> __device__ __forceinline__ void run_probe(const Amps &a, const TileCtx &c, const uint4 h, double *row) {
+template <bool DUAL> __device__ __forceinline__ void run_probe(const Amps &a, const TileCtx &c, const uint4 h, uint32_t slot0,
+                                                            double *row) {
     constexpr int SUMS = DUAL ? 6 : 3, N = DUAL ? 32 : 16, P0 = DUAL ? 1 : 0;
     float w[N];
 #pragma unroll
@@ -829,7 +830,7 @@ template <bool DUAL> __device__ __forceinline__ void run_probe(const Amps &a, co
     if constexpr (!DUAL) w[0] += __shfl_xor_sync(0xffffffffu, w[0], 1);
     const uint32_t v = DUAL ? lane : lane >> 1, p = v / SUMS;
     if (((DUAL || !(lane & 1u))) && ((act >> p) & 1u)) {
-        const uint32_t slot = h.z + __popc(act & ((1u << p) - 1u));
+        const uint32_t slot = h.z - slot0 + __popc(act & ((1u << p) - 1u));
         atomicAdd(row + slot * SUMS + v - p * SUMS, (double)w[0]);  // its own row: no result is waited for
     }
 }
@@ -1482,7 +1483,7 @@ __global__ void __launch_bounds__(THREADS, MINB) pass_rb_kernel(PassArgs a) {
     pass_finish(a, v, c, blockIdx.y, blockIdx.x * groups + sg, s_base[sg], gridDim.x * groups, red);
 }
 
-// One pass of a probe circuit (kernels.h) over a state in place: CTAs loop over the tiles,
+// One pass of a probe circuit (kernels.h), or some of its phases, over a state in place: CTAs loop over the tiles,
 // so that each warp keeps one row of sums. Bound by instruction issue: a measurement is 64
 // packed multiply-adds and about 70 instructions of exchange per warp, next to 64 for the
 // gate before it, and a pass reads and writes the state once for some 40 gates. Whole
@@ -1524,7 +1525,7 @@ __global__ void __launch_bounds__(THREADS, MINB) probe_kernel(ProbeArgs a) {
             const uint4 *u = s_ops[buf], *ue = u + (a.ph_pg[ph + 1] - a.ph_pg[ph]);
             while (u < ue) {
                 const uint4 h = *u;
-                if ((h.x & 255u) == OP_PROBE) run_probe<DUAL>(v, c, h, row);
+                if ((h.x & 255u) == OP_PROBE) run_probe<DUAL>(v, c, h, a.slot0, row);
                 else apply_macro(v, c, h, u + 1, a.mats, sm, ubuf, t);
                 u += h.x >> 24;  // a probe circuit has no fused runs
             }

@@ -75,3 +75,19 @@ def test_autotune_leaves_no_handle_counted(lib):
     before = lib.fake_trims()
     lib.arso_circuit_free(compiled(lib, *CIRCUITS[0]))
     assert lib.fake_trims() == before + 2  # both pools
+
+
+@pytest.mark.parametrize("kind", ["fidelity", "outcome"])
+def test_exhaustive_scratch_is_bounded_on_one_deep_pass(lib, kind):
+    # 20,000 one-qubit gates on the qubits of one tile: the sums of one pass would take a
+    # gigabyte (twice that for two states), the state itself 8 MiB
+    n = 20
+    gates = [W.Gate("RY", (k % 12,), (0.1 + k,)) for k in range(20000)]
+    cc = compiled(lib, W.Circuit(n, gates))
+    crit = arso.make_criterion(W.Criterion(kind, target=1, threshold=0.5))
+    P = (C.c_double * 4)()
+    lib.fake_reset_counts()
+    ok(lib, lib.arso_exhaustive(cc, C.byref(crit), lib.fake_stream(0), P, None))
+    lib.arso_circuit_free(cc)
+    assert lib.fake_launches(b"probe_kernel") >= 2
+    assert lib.fake_largest() <= 256 << 20
