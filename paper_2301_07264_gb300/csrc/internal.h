@@ -21,12 +21,16 @@ struct Error : std::runtime_error {
 };
 void set_last_error(const std::string &m);
 
+// An error is thrown once: the runtime's record of it is cleared, or the launch check of the
+// next call would report it again.
 #define ARSO_CUDA(call)                                                                       \
     do {                                                                                      \
         cudaError_t e_ = (call);                                                              \
-        if (e_ != cudaSuccess)                                                                \
+        if (e_ != cudaSuccess) {                                                              \
+            (void)cudaGetLastError();                                                         \
             throw ::arso::Error(e_ == cudaErrorMemoryAllocation ? ARSO_ENOMEM : ARSO_ECUDA,   \
                                 std::string(#call) + ": " + cudaGetErrorString(e_));          \
+        }                                                                                     \
     } while (0)
 #define ARSO_REQUIRE(cond, msg)                                              \
     do {                                                                     \

@@ -91,3 +91,15 @@ def test_exhaustive_scratch_is_bounded_on_one_deep_pass(lib, kind):
     lib.arso_circuit_free(cc)
     assert lib.fake_launches(b"probe_kernel") >= 2
     assert lib.fake_largest() <= 256 << 20
+
+
+def test_a_failed_call_does_not_fail_the_next(lib):
+    stream = lib.fake_stream(0)
+    cc = compiled(lib, *CIRCUITS[1])
+    for k in range(4):
+        lib.fake_fail_at(k)
+        e = C.c_void_p()
+        assert lib.arso_sample_errors(cc, 0.01, 0.01, 0.01, 1, 0, 8, stream, C.byref(e)) == arso.ENOMEM
+        lib.fake_fail_at(-1)
+        lib.arso_error_list_free(sampled(lib, cc, stream))
+    lib.arso_circuit_free(cc)
