@@ -713,7 +713,6 @@ static void sample(const arso_circuit *c, double px, double pz, double py, uint6
     ARSO_REQUIRE(pt <= 1.0, "p_x + p_z + p_y must be <= 1");
     ARSO_REQUIRE(begin + n_traj >= begin, "trajectory range overflows");
     std::unique_ptr<arso_error_list> e = new_list(c, n_traj, st);
-    SyncOnFail wait(st);
     SampleArgs a{};
     a.seed = seed;
     a.traj_begin = begin;
@@ -744,7 +743,6 @@ static void sample(const arso_circuit *c, double px, double pz, double py, uint6
     if (total) launch_sample_fill(a, e->d_offsets.as<uint64_t>(), c->d_loc_key.as<uint32_t>(), e->d_loc.as<uint32_t>(),
                                   e->d_key.as<uint32_t>(), st);
     finish_list(c, e.get(), st);
-    wait.done = true;
     *out = e.release();
 }
 
@@ -776,7 +774,6 @@ static void sample_batch(size_t count, const arso_circuit *const *circuits, cons
                          const double *py, const uint64_t *seeds, const uint64_t *begins, const uint64_t *n_traj,
                          cudaStream_t st, arso_error_list **out) {
     std::vector<std::unique_ptr<arso_error_list>> lists(count);
-    SyncOnFail wait(st);
     std::vector<SampleJob> jobs(count);
     uint64_t total = 0;
     for (size_t i = 0; i < count; ++i) {
@@ -817,7 +814,6 @@ static void sample_batch(size_t count, const arso_circuit *const *circuits, cons
         launch_sample_batch_fill(d_jobs.as<SampleJob>(), (uint32_t)count, total, any, st);
         ARSO_CUDA(cudaStreamSynchronize(st));
     }
-    wait.done = true;
     for (size_t i = 0; i < count; ++i) out[i] = lists[i].release();
 }
 
@@ -837,7 +833,6 @@ static void list_from_host(const arso_circuit *c, uint64_t n_traj, const uint64_
     const uint64_t total = offsets[n_traj];
     ARSO_REQUIRE(total == 0 || events != nullptr, "events is NULL");
     std::unique_ptr<arso_error_list> e = new_list(c, n_traj, st);
-    SyncOnFail wait(st);
     e->n_events = total;
     e->d_loc.ensure(std::max<uint64_t>(total, 1) * 4, st);
     e->d_key.ensure(std::max<uint64_t>(total, 1) * 4, st);
@@ -847,7 +842,6 @@ static void list_from_host(const arso_circuit *c, uint64_t n_traj, const uint64_
         launch_keys_from_loc(e->d_loc.as<uint32_t>(), total, c->d_loc_key.as<uint32_t>(), e->d_key.as<uint32_t>(), st);
     }
     finish_list(c, e.get(), st);
-    wait.done = true;
     *out = e.release();
 }
 
@@ -1808,11 +1802,13 @@ arso_status arso_error_list_copy(const arso_error_list *e, uint64_t *offsets, ui
     return guard([&] {
         ARSO_REQUIRE(e != nullptr, "NULL error list");
         cudaStream_t st = (cudaStream_t)stream;
+        SyncOnFail wait(st);
         if (offsets)
             copy_d2h(offsets, e->d_offsets.ptr, (e->n_traj + 1) * 8, st);
         if (events && e->n_events)
             copy_d2h(events, e->d_loc.ptr, e->n_events * 4, st);
         ARSO_CUDA(cudaStreamSynchronize(st));
+        wait.done = true;
     });
 }
 
@@ -1825,6 +1821,7 @@ arso_status arso_run_trajectories(const arso_circuit *cc, const arso_error_list 
         ARSO_REQUIRE(e->circ == cc, "error list belongs to another circuit");
         arso_circuit *c = const_cast<arso_circuit *>(cc);
         cudaStream_t st = (cudaStream_t)stream;
+        SyncOnFail wait(st);
         DevCrit dc;
         make_crit(c, crit, dc, st);
         const bool sdev = is_device_ptr(score_out), pdev = pass_out && is_device_ptr(pass_out);
@@ -1838,6 +1835,7 @@ arso_status arso_run_trajectories(const arso_circuit *cc, const arso_error_list 
         if (pass_out && !pdev && e->n_traj)
             copy_d2h(pass_out, d_pass, e->n_traj, st);
         ARSO_CUDA(cudaStreamSynchronize(st));
+        wait.done = true;
     });
 }
 
@@ -1873,6 +1871,7 @@ arso_status arso_run_batch(size_t count, arso_circuit *const *circuits, const ar
     return guard([&] {
         ARSO_REQUIRE(count == 0 || (circuits && errors && crits && score_out), "NULL argument");
         cudaStream_t st = (cudaStream_t)stream;
+        SyncOnFail wait(st);
         std::vector<DevCrit> dcs(count);
         std::vector<std::unique_ptr<Scratch>> tmp;
         std::vector<double *> d_score(count);
@@ -1988,6 +1987,7 @@ arso_status arso_run_batch(size_t count, arso_circuit *const *circuits, const ar
             if (pass_out && pass_out[i] && d_pass[i] != pass_out[i]) copy_d2h(pass_out[i], d_pass[i], T, st);
         }
         ARSO_CUDA(cudaStreamSynchronize(st));
+        wait.done = true;
     });
 }
 
@@ -2063,8 +2063,12 @@ arso_status arso_trajectory_states(const arso_circuit *cc, const arso_error_list
         ARSO_REQUIRE(is_device_ptr(amps_out), "amps_out must be device memory");
         arso_circuit *c = const_cast<arso_circuit *>(cc);
         cudaStream_t st = (cudaStream_t)stream;
+        SyncOnFail wait(st);
         ensure_cache(c, st);
-        if (!count) return;
+        if (!count) {
+            wait.done = true;
+            return;
+        }
         if (c->engine == 0) {
             ResidentArgs a = resident_args(c);
             a.first_traj = first;
@@ -2084,6 +2088,7 @@ arso_status arso_trajectory_states(const arso_circuit *cc, const arso_error_list
             run_streaming(c, e, ids, fp, fp, none, nullptr, nullptr, amps_out, st);
         }
         ARSO_CUDA(cudaStreamSynchronize(st));
+        wait.done = true;
     });
 }
 

@@ -5,6 +5,7 @@
 
 #include <complex>
 #include <cstdint>
+#include <exception>
 #include <memory>
 #include <stdexcept>
 #include <string>
@@ -276,14 +277,18 @@ struct DeviceBuffer {
 };
 
 // Memory that only calls which wait for their own work use (error lists, criteria): freed
-// without waiting. A call that fails half-way waits before its buffers go (SyncOnFail).
+// without waiting, except where an exception takes a call's own buffers with work in flight.
+// A call on a list that its caller owns waits when it fails (SyncOnFail).
 struct ListBuffer {
     void *ptr = nullptr;
     size_t bytes = 0;
     ListBuffer() = default;
     ListBuffer(const ListBuffer &) = delete;
     ListBuffer &operator=(const ListBuffer &) = delete;
-    ~ListBuffer() { pool_free_idle(ptr); }
+    ~ListBuffer() {
+        if (ptr && std::uncaught_exceptions()) cudaDeviceSynchronize();
+        pool_free_idle(ptr);
+    }
     void ensure(size_t b, cudaStream_t st) {  // once; usable on st
         if (ptr) throw Error(ARSO_EINVAL, "internal: a list buffer is allocated once");
         ptr = pool_alloc_list(b, st);
@@ -313,6 +318,7 @@ struct StreamBuffer {
     }
     template <typename T> T *as() const { return static_cast<T *>(ptr); }
 };
+// Waits for the stream when a call is left before done is set.
 struct SyncOnFail {
     cudaStream_t st;
     bool done = false;

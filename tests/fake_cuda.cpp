@@ -35,6 +35,7 @@ bool legacy_copy[2] = {false, false};
 std::map<void *, Block> blocks;
 uint64_t violations[4], trims, frees, largest;
 long fail_at = -1, allocs = 0;           // the pool allocation that fails (and its retry)
+long fail_launch = -1, launches = 0;     // the launch that fails
 bool retry_fails = false;
 std::vector<std::string> launched;
 std::map<const void *, std::string> names;
@@ -71,6 +72,7 @@ const Block *block_of(const void *p) {
 cudaError_t launch(const void *f, cudaStream_t s) {
     std::lock_guard<std::recursive_mutex> g(mu);
     const int d = dev_of(s);
+    if (launches++ == fail_launch) return err(cudaErrorLaunchOutOfResources);
     if (legacy_copy[d] && key(s)) ++violations[0];
     launched.push_back(names.count(f) ? names[f] : "?");
     work(s);
@@ -94,6 +96,8 @@ uint64_t fake_launches(const char *part) {
 }
 void fake_reset_counts() { memset(violations, 0, sizeof violations), trims = frees = largest = 0, allocs = 0, launched.clear(); }
 void fake_fail_at(long k) { fail_at = k, allocs = 0, retry_fails = false; }
+void fake_fail_launch_at(long k) { fail_launch = k, launches = 0; }
+uint64_t fake_tried() { return (uint64_t)launches; }
 void fake_device(int d) { cur = d; }
 int fake_current() { return cur; }
 void *fake_stream(int d) { return new Stream{&ctxs[d], ctxs[d].id}; }

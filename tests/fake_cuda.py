@@ -21,10 +21,10 @@ def load(tmp):
         getattr(lib, name).argtypes = args
     for name in ("arso_circuit_free", "arso_error_list_free", "arso_surrogate_free"):
         getattr(lib, name).argtypes, getattr(lib, name).restype = [C.c_void_p], None
-    for name in ("violation", "trims", "frees", "largest", "live", "allocs", "launches"):
+    for name in ("violation", "trims", "frees", "largest", "live", "allocs", "tried", "launches"):
         getattr(lib, "fake_" + name).restype = C.c_uint64
     lib.fake_launches.argtypes = [C.c_char_p]
-    lib.fake_fail_at.argtypes = [C.c_long]
+    lib.fake_fail_at.argtypes = lib.fake_fail_launch_at.argtypes = [C.c_long]
     lib.fake_stream.restype = C.c_void_p
     lib.arso_last_error.restype = C.c_char_p
     return lib

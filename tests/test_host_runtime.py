@@ -18,6 +18,7 @@ def library(tmp_path_factory):
 @pytest.fixture
 def lib(library):
     library.fake_fail_at(-1)
+    library.fake_fail_launch_at(-1)
     library.fake_device(0)
     library.fake_reset_counts()
     return library
@@ -103,3 +104,58 @@ def test_a_failed_call_does_not_fail_the_next(lib):
         lib.fake_fail_at(-1)
         lib.arso_error_list_free(sampled(lib, cc, stream))
     lib.arso_circuit_free(cc)
+
+
+def _calls(lib, stream):
+    """The calls that hold an error list or a criterion's table, each as (name, call)."""
+    circs = {k: compiled(lib, *CIRCUITS[k]) for k in (0, 1)}
+    lists = {k: sampled(lib, cc, stream) for k, cc in circs.items()}
+    crit = arso.make_criterion(W.Criterion("binning", basis_set=(0, 3), threshold=0.5))
+    score, P, res = (C.c_double * 8)(), (C.c_double * 4)(), arso.Result()
+    out = []
+    for k, cc in circs.items():
+        e = lists[k]
+        ptr = lambda *v: C.cast((C.c_void_p * len(v))(*v), C.c_void_p)  # noqa: E731
+        out += [("sample", lambda cc=cc: _sample(lib, cc, stream)),
+                ("trajectories", lambda cc=cc, e=e: lib.arso_run_trajectories(cc, e, C.byref(crit), stream, score, None)),
+                ("batch", lambda cc=cc, e=e: lib.arso_run_batch(C.c_size_t(1), ptr(cc), ptr(e), C.byref(crit),
+                                                                C.c_void_p(stream), ptr(C.addressof(score)), None)),
+                ("exhaustive", lambda cc=cc: lib.arso_exhaustive(cc, C.byref(crit), stream, P, None)),
+                ("success", lambda cc=cc: lib.arso_success_prob(cc, C.byref(crit), 1e-3, 1, 8, 0, stream, C.byref(res)))]
+    return out, circs, lists
+
+
+def _sample(lib, cc, stream):
+    e = C.c_void_p()
+    st = lib.arso_sample_errors(cc, 0.01, 0.01, 0.01, 1, 0, 8, stream, C.byref(e))
+    if st == arso.OK:
+        lib.arso_error_list_free(e)
+    return st
+
+
+@pytest.mark.parametrize("what", ["allocation", "launch"])
+def test_failing_calls_wait_before_lists_are_freed(lib, what):
+    # every allocation, then every launch of every call fails once: memory that kernels in
+    # flight may read is freed only after they have been waited for, by the call itself or,
+    # its own list, by the caller
+    stream = lib.fake_stream(0)
+    fail, tried = (lib.fake_fail_at, lib.fake_allocs) if what == "allocation" else (lib.fake_fail_launch_at, lib.fake_tried)
+    failed = 0
+    for i in range(10):
+        for k in range(60):
+            calls, circs, lists = _calls(lib, stream)
+            lib.fake_reset_counts()
+            fail(k)
+            status = calls[i][1]()
+            done = tried() <= k
+            fail(-1)
+            for e in lists.values():
+                lib.arso_error_list_free(e)
+            for cc in circs.values():
+                lib.arso_circuit_free(cc)
+            assert lib.fake_violation(1) == 0, (calls[i][0], k)
+            failed += status != arso.OK
+            if done:
+                assert status == arso.OK
+                break
+    assert failed > 40
