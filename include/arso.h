@@ -24,7 +24,7 @@
  *  - Pauli codes: 1 = X, 2 = Z, 3 = Y, acting as Eq. (2) prints them:
  *    X (a0, a1) -> (a1, a0); Z -> (a0, -a1); Y -> (-i a1, i a0).
  *  - The library allocates device memory for its own handles and scratch from a
- *    CUDA memory pool of its own (one per device, all streams and threads), which
+ *    CUDA memory pool of its own (one per context, all streams and threads), which
  *    keeps up to 17 GiB of freed memory mapped while a circuit or surrogate is
  *    alive, and at most 256 MiB after the last of them; it never takes ownership
  *    of caller memory.

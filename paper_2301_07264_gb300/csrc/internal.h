@@ -239,14 +239,16 @@ struct Criterion {
     std::vector<uint64_t> set;
 };
 
-// pool.cpp: memory of the library's pools. pool_alloc: usable on `st` from there on and freed
-// on `st`; pool_alloc_list: the same for memory that pool_free_idle frees;
-// pool_alloc_now: usable on any stream after the call; pool_free_idle: no work that uses
-// the memory may be pending.
+// pool.cpp: memory of the library's pools, one set a context. pool_alloc: usable on `st` from
+// there on and freed on `st`; pool_alloc_list: the same for memory that pool_free frees;
+// pool_alloc_now: usable on any stream after the call; pool_free: frees memory of `owner`,
+// whatever device or context is current, after waiting for the owner's device (wait) or when
+// no work that uses the memory is pending.
+struct ContextPools;
 void *pool_alloc(size_t bytes, cudaStream_t st);
-void *pool_alloc_list(size_t bytes, cudaStream_t st);
-void *pool_alloc_now(size_t bytes);
-void pool_free_idle(void *ptr) noexcept;
+void *pool_alloc_list(size_t bytes, cudaStream_t st, ContextPools *&owner);
+void *pool_alloc_now(size_t bytes, ContextPools *&owner);
+void pool_free(void *ptr, ContextPools *owner, bool wait) noexcept;
 // circuits and surrogates alive: with the last one freed the pool's memory goes back
 void handle_made();
 void handle_freed() noexcept;
@@ -255,22 +257,20 @@ void handle_freed() noexcept;
 struct DeviceBuffer {
     void *ptr = nullptr;
     size_t bytes = 0;
+    ContextPools *owner = nullptr;
     DeviceBuffer() = default;
     DeviceBuffer(const DeviceBuffer &) = delete;
     DeviceBuffer &operator=(const DeviceBuffer &) = delete;
     ~DeviceBuffer() { release(); }
     void release() {
-        if (ptr) {
-            cudaDeviceSynchronize();  // kernels of any stream may still use it (as cudaFree waits for them)
-            pool_free_idle(ptr);
-        }
+        if (ptr) pool_free(ptr, owner, true);  // kernels of any stream may still use it (cudaFree waits for them too)
         ptr = nullptr;
         bytes = 0;
     }
     void ensure(size_t b) {
         if (b <= bytes) return;
         release();
-        ptr = pool_alloc_now(b);
+        ptr = pool_alloc_now(b, owner);
         bytes = b;
     }
     template <typename T> T *as() const { return static_cast<T *>(ptr); }
@@ -282,16 +282,16 @@ struct DeviceBuffer {
 struct ListBuffer {
     void *ptr = nullptr;
     size_t bytes = 0;
+    ContextPools *owner = nullptr;
     ListBuffer() = default;
     ListBuffer(const ListBuffer &) = delete;
     ListBuffer &operator=(const ListBuffer &) = delete;
     ~ListBuffer() {
-        if (ptr && std::uncaught_exceptions()) cudaDeviceSynchronize();
-        pool_free_idle(ptr);
+        if (ptr) pool_free(ptr, owner, std::uncaught_exceptions() > 0);
     }
     void ensure(size_t b, cudaStream_t st) {  // once; usable on st
         if (ptr) throw Error(ARSO_EINVAL, "internal: a list buffer is allocated once");
-        ptr = pool_alloc_list(b, st);
+        ptr = pool_alloc_list(b, st, owner);
         bytes = b;
     }
     template <typename T> T *as() const { return static_cast<T *>(ptr); }

@@ -106,8 +106,9 @@ void fake_device_reset(int d) { ctxs[d].id = 100 + next_id++; pending[d].clear()
 // ------------------------------------------------------------------ driver ----
 static CUresult ctx_current(CUcontext *c) { *c = reinterpret_cast<CUcontext>(&ctxs[cur]); return CUDA_SUCCESS; }
 static CUresult ctx_id(CUcontext c, unsigned long long *id) { *id = (c ? reinterpret_cast<Ctx *>(c) : &ctxs[cur])->id; return CUDA_SUCCESS; }
-static CUresult ctx_push(CUcontext c) { static_assert(sizeof(int) == 4, ""); cur = reinterpret_cast<Ctx *>(c)->dev | (cur << 8); return CUDA_SUCCESS; }
-static CUresult ctx_pop(CUcontext *c) { if (c) *c = nullptr; cur >>= 8; return CUDA_SUCCESS; }
+static std::vector<int> below;  // devices under the current one
+static CUresult ctx_push(CUcontext c) { below.push_back(cur), cur = reinterpret_cast<Ctx *>(c)->dev; return CUDA_SUCCESS; }
+static CUresult ctx_pop(CUcontext *c) { *c = reinterpret_cast<CUcontext>(&ctxs[cur]), cur = below.back(), below.pop_back(); return CUDA_SUCCESS; }
 static CUresult encode(...) { return CUDA_SUCCESS; }
 cudaError_t cudaGetDriverEntryPointByVersion(const char *name, void **fn, unsigned int, unsigned long long,
                                              cudaDriverEntryPointQueryResult *q) {

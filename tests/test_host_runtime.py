@@ -159,3 +159,28 @@ def test_failing_calls_wait_before_lists_are_freed(lib, what):
                 assert status == arso.OK
                 break
     assert failed > 40
+
+
+def test_memory_is_freed_in_its_own_context(lib):
+    # handles and lists of device 0 freed while device 1 is current, then of a context that a
+    # reset of its device has ended; calls on the new context work
+    for reset in (False, True):
+        st = lib.fake_stream(0)
+        cc = compiled(lib, *CIRCUITS[1])
+        e = sampled(lib, cc, st)
+        lib.fake_reset_counts()
+        if reset:
+            lib.fake_device_reset(0)
+        else:
+            lib.fake_device(1)
+        live = lib.fake_live()
+        lib.arso_error_list_free(e)
+        lib.arso_circuit_free(cc)
+        assert lib.fake_current() == (0 if reset else 1)
+        assert (lib.fake_live() == live) == reset  # what a reset took is not freed again
+        lib.fake_device(0)
+        cc = compiled(lib, *CIRCUITS[1])
+        e = sampled(lib, cc, lib.fake_stream(0))
+        lib.arso_error_list_free(e)
+        lib.arso_circuit_free(cc)
+        assert [lib.fake_violation(k) for k in (1, 2, 3)] == [0, 0, 0]
