@@ -249,6 +249,7 @@ void *pool_alloc(size_t bytes, cudaStream_t st);
 void *pool_alloc_list(size_t bytes, cudaStream_t st, ContextPools *&owner);
 void *pool_alloc_now(size_t bytes, ContextPools *&owner);
 void pool_free(void *ptr, ContextPools *owner, bool wait) noexcept;
+unsigned long long context_id();  // of the current context; never used twice
 // circuits and surrogates alive: with the last one freed the pool's memory goes back
 void handle_made();
 void handle_freed() noexcept;

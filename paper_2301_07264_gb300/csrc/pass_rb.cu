@@ -21,6 +21,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "prof.h"
 #include "sim_common.cuh"
@@ -2228,10 +2229,10 @@ void launch_mix(const MixArgs &a, double bytes, double flops, double smem_bytes,
     if (!a.n_sub) return;
     ProfScope ps_(ARSO_K_MIX, bytes, st, flops, smem_bytes);
     const size_t smem = (size_t(1) << 13) * sizeof(float2);
-    static bool attr = false;
-    if (!attr) {
+    static std::atomic<unsigned long long> set_for{0};  // the context whose attribute was set last
+    if (const unsigned long long id = context_id(); set_for.load() != id) {
         ARSO_CUDA(cudaFuncSetAttribute(mix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr = true;
+        set_for.store(id);
     }
     int per_sm = 1, dev = 0, sms = 152;
     ARSO_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mix_kernel, MIX_THREADS, smem));
@@ -2242,21 +2243,22 @@ void launch_mix(const MixArgs &a, double bytes, double flops, double smem_bytes,
     ARSO_CUDA(cudaGetLastError());
 }
 
-// Raise the dynamic shared-memory limit of the pass kernels once, before any
+// Raise the dynamic shared-memory limit of the pass kernels once a context, before any
 // launch (and outside stream capture).
 static const auto pass_128 = pass_rb_kernel<128, 5>;  // 96 registers, five CTAs per SM
 static const auto pass_256 = pass_rb_kernel<256, 3>;  // 80 registers, three CTAs per SM
 static const auto pass_512 = pass_rb_kernel<512, 1>;
 void prepare_pass_rb() {
-    static bool done = false;
-    if (done) return;
+    static std::atomic<unsigned long long> set_for{0};  // the context whose attributes were set last
+    const unsigned long long id = context_id();
+    if (set_for.load() == id) return;
     const int tile = (1 << MAX_TILE_QUBITS) * (int)sizeof(float2);
     ARSO_CUDA(cudaFuncSetAttribute(pass_128, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 256));
     ARSO_CUDA(cudaFuncSetAttribute(pass_256, cudaFuncAttributeMaxDynamicSharedMemorySize, 256 * 256));
     ARSO_CUDA(cudaFuncSetAttribute(pass_512, cudaFuncAttributeMaxDynamicSharedMemorySize, tile));
     ARSO_CUDA(cudaFuncSetAttribute(pass_tensor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    tile + 2 * (int)TP_IMAGE_BYTES));
-    done = true;
+    set_for.store(id);
 }
 
 // Tiles of up to 2^12 amplitudes run in 128-thread CTAs (small tiles several side by side),

@@ -171,6 +171,11 @@ void pool_free(void *ptr, ContextPools *owner, bool wait) noexcept {
     cudaFreeAsync(ptr, owner->idle);
 }
 
+unsigned long long context_id() {
+    CUcontext c = nullptr;
+    return current_id(c);
+}
+
 void handle_made() { g_handles.fetch_add(1); }
 void handle_freed() noexcept {
     if (g_handles.fetch_sub(1) != 1) return;

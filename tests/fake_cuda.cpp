@@ -8,6 +8,8 @@
 //   fake_violation(2)  memory freed while a device other than its own is current, on another
 //                      device's stream, or with a runtime call that waits for another device
 //   fake_violation(3)  a use of a pool or stream of a context that is gone
+//   fake_violation(4)  a launch with more than 48 KiB of dynamic shared memory in a context where
+//                      that was not allowed to the kernel
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <sys/mman.h>
@@ -33,12 +35,13 @@ int cur = 0;                             // current device
 std::set<void *> pending[2];             // streams with work not waited for (legacy: nullptr)
 bool legacy_copy[2] = {false, false};
 std::map<void *, Block> blocks;
-uint64_t violations[4], trims, frees, largest;
+uint64_t violations[5], trims, frees, largest;
 long fail_at = -1, allocs = 0;           // the pool allocation that fails (and its retry)
 long fail_launch = -1, launches = 0;     // the launch that fails
 bool retry_fails = false;
 std::vector<std::string> launched;
 std::map<const void *, std::string> names;
+std::map<std::pair<const void *, uint64_t>, int> allowed;  // dynamic shared memory of (kernel, context)
 cudaError_t last = cudaSuccess;
 
 cudaError_t err(cudaError_t e) { if (e != cudaSuccess) last = e; return e; }
@@ -69,11 +72,12 @@ const Block *block_of(const void *p) {
     --it;
     return (const char *)p < (const char *)it->first + it->second.bytes ? &it->second : nullptr;
 }
-cudaError_t launch(const void *f, cudaStream_t s) {
+cudaError_t launch(const void *f, size_t smem, cudaStream_t s) {
     std::lock_guard<std::recursive_mutex> g(mu);
     const int d = dev_of(s);
     if (launches++ == fail_launch) return err(cudaErrorLaunchOutOfResources);
     if (legacy_copy[d] && key(s)) ++violations[0];
+    if (smem > 48 * 1024 && (size_t)allowed[{f, ctxs[d].id}] < smem) ++violations[4];
     launched.push_back(names.count(f) ? names[f] : "?");
     work(s);
     return cudaSuccess;
@@ -132,8 +136,8 @@ cudaError_t __cudaPopCallConfiguration(dim3 *g, dim3 *b, size_t *sm, void *s) {
     return cudaSuccess;
 }
 cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) { *k = (cudaKernel_t)f; return cudaSuccess; }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **, size_t, cudaStream_t s) { return launch((const void *)k, s); }
-cudaError_t cudaLaunchKernel(const void *f, dim3, dim3, void **, size_t, cudaStream_t s) { return launch(f, s); }
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **, size_t sm, cudaStream_t s) { return launch((const void *)k, sm, s); }
+cudaError_t cudaLaunchKernel(const void *f, dim3, dim3, void **, size_t sm, cudaStream_t s) { return launch(f, sm, s); }
 
 cudaError_t cudaGetDevice(int *d) { *d = cur; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { cur = d; return cudaSuccess; }
@@ -158,7 +162,7 @@ cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 1.f; return cudaSuccess; }
-cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute, int v) { allowed[{f, ctxs[cur].id}] = v; return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int *n, const void *, int, size_t) { *n = 2; return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned) { *n = 2; return cudaSuccess; }
 cudaError_t cudaGetLastError() { const cudaError_t e = last; last = cudaSuccess; return e; }

@@ -184,3 +184,21 @@ def test_memory_is_freed_in_its_own_context(lib):
         lib.arso_error_list_free(e)
         lib.arso_circuit_free(cc)
         assert [lib.fake_violation(k) for k in (1, 2, 3)] == [0, 0, 0]
+
+
+def test_shared_memory_is_allowed_on_every_device(lib):
+    crit = arso.make_criterion(W.Criterion("fidelity", threshold=0.5))
+    score = (C.c_double * 8)()
+    outs = (C.c_void_p * 1)(C.addressof(score))
+    for dev in (0, 1, 0):
+        lib.fake_device(dev)
+        st = lib.fake_stream(dev)
+        for k in range(len(CIRCUITS)):
+            cc = compiled(lib, *CIRCUITS[k])
+            e = sampled(lib, cc, st)
+            ok(lib, lib.arso_run_trajectories(cc, e, C.byref(crit), st, score, None))
+            ok(lib, lib.arso_run_batch(C.c_size_t(1), (C.c_void_p * 1)(cc.value), (C.c_void_p * 1)(e.value), C.byref(crit),
+                                       C.c_void_p(st), outs, None))
+            lib.arso_error_list_free(e)
+            lib.arso_circuit_free(cc)
+    assert [lib.fake_violation(k) for k in (2, 3, 4)] == [0, 0, 0]
