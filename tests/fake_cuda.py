@@ -10,11 +10,12 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 
 
 def load(tmp):
+    # bound to its own symbols: another module of the process may have loaded the real runtime
     build.build()
     inc = os.path.join(build._cuda_home(), "include")
     out = os.path.join(str(tmp), "libarso_fake.so")
     objs = [os.path.join(build.OUT_DIR, f) for f in sorted(os.listdir(build.OUT_DIR)) if f.endswith(".o")]
-    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-w", "-I", inc, "-o", out,
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-w", "-Wl,-Bsymbolic", "-I", inc, "-o", out,
                     os.path.join(HERE, "fake_cuda.cpp"), *objs, "-lpthread"], check=True)
     lib = C.CDLL(out)
     for name, args in arso._sigs.items():
