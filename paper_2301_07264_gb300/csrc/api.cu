@@ -251,6 +251,7 @@ static void run_pass(const arso_circuit *c, const PassArgs &a, bool last, uint32
         b.ph_pg = c->d_ph_pg.as<uint32_t>();
         b.evs = c->d_evs.as<EvSlot>();
         b.frame = pass_frame(c, a.pass);
+        b.wide = 32 * c->passes[a.pass].full > c->passes[a.pass].ge - c->passes[a.pass].gb;
         if (c->tensor) {
             b.ph_t = c->d_ph_t.as<uint32_t>();
             b.tmats = c->d_tmats.ptr;

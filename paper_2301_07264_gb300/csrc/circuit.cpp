@@ -1249,10 +1249,11 @@ static void reg_program(arso_circuit *c) {
     c->probe_first.clear();
     c->evs.resize(2 * c->perm.size());
     size_t blk = 0;  // next fused run (they are in engine order)
-    for (const Pass &ps : c->passes) {
+    for (Pass &ps : c->passes) {
         std::vector<int> local(c->n, -1);
         for (size_t i = 0; i < ps.tile_qubits.size(); ++i) local[ps.tile_qubits[i]] = (int)i;
         Frame F(c->tile_qubits);
+        ps.full = 0;
         for (uint32_t ph = ps.pb; ph < ps.pe; ++ph) {
             if (c->engine == 0) c->frame.push_back(F.f);
             c->ph_pg.push_back((uint32_t)c->prog.size());
@@ -1283,6 +1284,7 @@ static void reg_program(arso_circuit *c) {
                             const uint32_t aux[2] = {(uint32_t)c->rmats.size(), 0};
                             for (const cd &v : g.m) c->rmats.push_back(f2(v));
                             W.op(reg_opcode(GC_DENSE1, p0, p1), pos + 1, z, aux);
+                            ++ps.full;
                         }
                         break;
                     }

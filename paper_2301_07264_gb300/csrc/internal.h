@@ -223,6 +223,7 @@ struct Pass {
     double flops_per_amp = 0.0;        // algorithmic FP32 flops per amplitude of one sweep
     uint32_t remaps = 0;               // register-set changes inside the pass (from the load layout)
     uint32_t end_remap = 0;            // 1 if the last phase's set differs from the load layout
+    uint32_t full = 0;                 // one-qubit gates that its register program runs as full matrices
 };
 
 // One measurement of a probe circuit, in the order of the phases' slots.

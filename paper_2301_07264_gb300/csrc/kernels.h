@@ -95,6 +95,7 @@ struct PassArgs {
     const uint32_t *ph_pg;       // phase -> first unit of prog
     const EvSlot *evs;           // 2 per gate position
     const float2 *frame;         // frame table of the pass's end; NULL: the identity
+    int wide;                    // many full one-qubit matrices (launch_pass_rb)
     // tensor-core phases (NULL: every phase runs gate by gate)
     const uint32_t *ph_t;        // phase -> operand-image index or NO_TENSOR
     const void *tmats;           // TENSOR_IMAGE_HALVES fp16 values per image

@@ -2247,6 +2247,7 @@ void launch_mix(const MixArgs &a, double bytes, double flops, double smem_bytes,
 // launch (and outside stream capture).
 static const auto pass_128 = pass_rb_kernel<128, 5>;  // 96 registers, five CTAs per SM
 static const auto pass_256 = pass_rb_kernel<256, 3>;  // 80 registers, three CTAs per SM
+static const auto pass_256_wide = pass_rb_kernel<256, 2>;  // 128 registers, two
 static const auto pass_512 = pass_rb_kernel<512, 1>;
 void prepare_pass_rb() {
     static std::atomic<unsigned long long> set_for{0};  // the context whose attributes were set last
@@ -2255,6 +2256,7 @@ void prepare_pass_rb() {
     const int tile = (1 << MAX_TILE_QUBITS) * (int)sizeof(float2);
     ARSO_CUDA(cudaFuncSetAttribute(pass_128, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 256));
     ARSO_CUDA(cudaFuncSetAttribute(pass_256, cudaFuncAttributeMaxDynamicSharedMemorySize, 256 * 256));
+    ARSO_CUDA(cudaFuncSetAttribute(pass_256_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, 256 * 256));
     ARSO_CUDA(cudaFuncSetAttribute(pass_512, cudaFuncAttributeMaxDynamicSharedMemorySize, tile));
     ARSO_CUDA(cudaFuncSetAttribute(pass_tensor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    tile + 2 * (int)TP_IMAGE_BYTES));
@@ -2268,6 +2270,11 @@ void prepare_pass_rb() {
 // 376 (two); 13-qubit tiles: three CTAs per SM 6.53 ms against 6.87 with two (16-qubit
 // brickwork, 2,000 trajectories) and 3.12 against 3.41 (20-qubit adder, 500); both sides
 // before the fused runs and the z mask (305 ms, 6.0 ms and 1.7 ms since).
+// A full one-qubit matrix does not fit 80 registers: its constants and products spill. Passes
+// of 13-qubit tiles with more of them than one gate in 32 take two CTAs per SM; the single ones
+// that restore a frame's scale, at most one gate in 80, do not (17 qubits, 400 gates, 200
+// trajectories, matrices that have no frame form: 8.72 ms with three CTAs, 3.59 with two; one
+// such gate in eleven: 2.36 and 2.08).
 void launch_pass_rb(const PassArgs &a, bool last, uint32_t slots, double bytes, cudaStream_t st, double flops,
                     double smem_bytes) {
     ProfScope ps_(last && !a.store_last ? ARSO_K_PASS_LAST : ARSO_K_PASS, bytes, st, flops, smem_bytes);
@@ -2280,6 +2287,8 @@ void launch_pass_rb(const PassArgs &a, bool last, uint32_t slots, double bytes, 
         pass_tensor_kernel<<<dim3(tiles, slots), nt, smem + 2 * TP_IMAGE_BYTES, st>>>(a);
     } else if (nt == 512) {
         pass_512<<<dim3(tiles, slots), nt, smem, st>>>(a);
+    } else if (nt == 256 && a.wide) {
+        pass_256_wide<<<dim3(tiles, slots), nt, smem, st>>>(a);
     } else if (nt == 256) {
         pass_256<<<dim3(tiles, slots), nt, smem, st>>>(a);
     } else {

@@ -2,6 +2,7 @@
 before memory is read or freed."""
 import ctypes as C
 
+import numpy as np
 import pytest
 
 from paper_2301_07264_gb300 import arso
@@ -202,3 +203,23 @@ def test_shared_memory_is_allowed_on_every_device(lib):
             lib.arso_error_list_free(e)
             lib.arso_circuit_free(cc)
     assert [lib.fake_violation(k) for k in (2, 3, 4)] == [0, 0, 0]
+
+
+def test_full_matrices_take_the_wide_pass_kernel(lib):
+    # matrices that are unitary only up to their 32-bit rounding, entry by entry, have no frame
+    # form; a long run of rotations holds one full matrix in 80 gates, to restore the scale
+    rng = np.random.default_rng(1)
+    full = [W.Gate("U", (k % 12,), matrix=(W.haar_su2(rng) * np.exp(1j * k)).astype(np.complex64).astype(complex))
+            for k in range(200)]
+    crit = arso.make_criterion(W.Criterion("fidelity", threshold=0.5))
+    score = (C.c_double * 8)()
+    for gates, wide in ((full, True), ([W.Gate("RX", (k % 12,), (1.0 + k,)) for k in range(200)], False)):
+        cc = compiled(lib, W.Circuit(15, gates))
+        st = lib.fake_stream(0)
+        e = sampled(lib, cc, st)
+        lib.fake_reset_counts()
+        ok(lib, lib.arso_run_trajectories(cc, e, C.byref(crit), st, score, None))
+        lib.arso_error_list_free(e)
+        lib.arso_circuit_free(cc)
+        assert (lib.fake_launches(b"pass_rb_kernelILi256ELi2E") > 0) == wide
+        assert (lib.fake_launches(b"pass_rb_kernelILi256ELi3E") > 0) != wide
