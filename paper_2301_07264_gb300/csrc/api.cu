@@ -82,7 +82,7 @@ static void upload_frames(arso_circuit *c, const std::vector<std::vector<std::co
     for (size_t i = 0; i < fr.size(); ++i) {
         frame_table(fr[i], t, tab.data() + i * frame_floats2(t));
         for (const std::complex<double> &v : fr[i])
-            if (v != 1.0) c->frame_trivial[i] = 0;
+            if ((float)v.real() != 1.f || (float)v.imag() != 0.f) c->frame_trivial[i] = 0;
     }
     c->d_frame.ensure(std::max<size_t>(tab.size(), 1) * sizeof(float2));
     if (!tab.empty())

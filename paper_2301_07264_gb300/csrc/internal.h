@@ -94,7 +94,7 @@ struct DGate {
 //   w0  = cls | p0 << 8 | p1 << 12 | q0 << 16 | q1 << 24, with p0/p1 the
 //         register positions of q0/q1 in the gate's phase (15: thread bit)
 //   aux = matrix-pool offset (dense gates) or the exponent k of GC_OMEGA
-//   c0, c1 = inline constants: (a, b) of GC_SU2, (d0, d1) of GC_DIAG1, c0 of OP_CP
+//   c0, c1 = inline constants: (a, b) of GC_SU2, (d0, d1) of GC_DIAG1, (f, d) of OP_CP
 struct __align__(16) RegOp {
     uint32_t w0, aux;
     float2 c0, c1;
@@ -118,7 +118,7 @@ enum RegOpCode : uint32_t {
     OP_X = 71,       // tensor circuits only
     OP_OMEGA = 72,   // diag(1, omega^k), omega = e^{i pi/4}
     OP_DIAG1 = 73,   // tensor circuits only
-    OP_CP = 74,      // diag(1, 1, 1, f)
+    OP_CP = 74,      // diag(1, 1, 1, f (1 + d)), d = what the rounded f lacks of modulus 1
     OP_CX = 75,      // + target position; in a register program a flip under a condition (below)
     OP_DENSE2 = 80,
     OP_SWAP = 81,
@@ -139,7 +139,8 @@ enum RegOpCode : uint32_t {
 //               event commutes with the macro-op's other gates)
 //           z = q0 | q1 << 8 | p0 << 16 | p1 << 20 (tile bits and register positions)
 //           w = tile bits whose index-mask bit flips before the op (X)
-//   second unit where the op has constants: x, y = f, or x = matrix-pool offset
+//   second unit where the op has constants: x, y = f (OP_SCALE: z its residue, see EvSlot; OP_CP:
+//           z = d), or x = matrix-pool offset
 //   OP_LAYER: bits 8-12 of x the register positions that hold a gate G(x), bits 13-17
 //           those whose x is real; one unit (Re x, Re x, Im x, Im x) for each, in order
 //           (position 0: (Re x, -Re x, Im x, Im x), the lanes of a packed register)
@@ -166,8 +167,14 @@ enum RegOpCode : uint32_t {
 // after the gate, and the qubit's tile bit.
 struct __align__(16) EvSlot {
     float2 phi;
-    uint32_t q, pad;
+    uint32_t q, residue;  // residue: what phi, rounded, lacks of modulus 1, in the units of gp
 };
+
+// The power of i that the kernels keep for a trajectory, gp, has two bits; above them it counts,
+// in units of 2^-32, what the moduli of the rounded constants that events brought in lack of
+// the exact ones. Each is the same for all amplitudes, so they would add up over the events;
+// the state is multiplied by 1 + their sum where gp is applied. (Two million events of the
+// largest residue would fill it.)
 
 // A frame as the kernels apply it, in the load/store register mapping of a t-qubit
 // tile: 2^(t-5) thread factors (S times the phases of tile bits 1..t-5), then the 32
@@ -415,7 +422,7 @@ namespace arso {
 // circuit.cpp
 void matrix_for(const arso_gate &g, HostGate &h);  // h.arity must be set
 std::vector<float> circuit_features(const arso_circuit *c, const arso_criterion *crit);
-void frame_table(const std::vector<std::complex<double>> &f, int t, float2 *out);
+std::complex<double> frame_table(const std::vector<std::complex<double>> &f, int t, float2 *out);
 std::unique_ptr<arso_circuit> build_probe(const arso_circuit *c, bool dual);
 void build_circuit(arso_circuit *c, uint32_t n, const arso_gate *gates, size_t n_gates,
                    const arso_compile_opts *opts);

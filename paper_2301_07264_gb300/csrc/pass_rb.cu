@@ -273,7 +273,7 @@ struct TileCtx {
     uint32_t tpart;      // thread part of the local index
     uint32_t m;          // X mask (stored[j] = state[j ^ m])
     uint32_t z;          // Z mask on stored indices (register programs)
-    uint32_t gp;         // global phase i^gp
+    uint32_t gp;         // global phase i^gp, and above its two bits the residues of EvSlot
     uint32_t tid, nthr;  // thread index within the tile's thread group, group size
 };
 
@@ -435,16 +435,18 @@ template <int IDX> __device__ __forceinline__ void cz_case(Amps &a) {
     neg_quarter<cz_pa(IDX >> 2), cz_pb(IDX >> 2), (IDX >> 1) & 1, IDX & 1>(a);
 }
 
-// multiply the registers selected by mask by f
-__device__ __forceinline__ void phase_masked(Amps &a, uint32_t mask, float2 f) {
+// multiply the registers selected by mask by f (1 + d): d is what the rounded f lacks of modulus
+// 1, which every amplitude it meets would lose alike (norm of a 16-qubit QFT: 2.7e-7 short)
+__device__ __forceinline__ void phase_masked(Amps &a, uint32_t mask, float2 f, float d) {
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
         const bool x = (mask >> (2 * k)) & 1u, y = (mask >> (2 * k + 1)) & 1u;
         const float2 fr = make_float2(x ? f.x : 1.f, y ? f.x : 1.f), fi = make_float2(x ? f.y : 0.f, y ? f.y : 0.f);
-        const float2 nfi = make_float2(-fi.x, -fi.y);
+        const float2 nfi = make_float2(-fi.x, -fi.y), dd = make_float2(x ? d : 0.f, y ? d : 0.f);
         const float2 r = a.re[k], i = a.im[k];
-        a.re[k] = fma2(nfi, i, mul2(fr, r));
-        a.im[k] = fma2(fi, r, mul2(fr, i));
+        const float2 nr = fma2(nfi, i, mul2(fr, r)), ni = fma2(fi, r, mul2(fr, i));
+        a.re[k] = fma2(dd, nr, nr);
+        a.im[k] = fma2(dd, ni, ni);
     }
 }
 // multiply the registers selected by mask by f, the others by its conjugate
@@ -461,9 +463,9 @@ __device__ __forceinline__ void phase_pair(Amps &a, uint32_t mask, float2 f) {
     }
 }
 // diag(1, 1, 1, f) on tile bits qa, qb
-__device__ __forceinline__ void rg_cp(Amps &a, const TileCtx &c, uint32_t qa, uint32_t qb, float2 f) {
+__device__ __forceinline__ void rg_cp(Amps &a, const TileCtx &c, uint32_t qa, uint32_t qb, float2 f, float d) {
     const uint32_t mask = bit_mask(c, qa) & bit_mask(c, qb);
-    if (mask) phase_masked(a, mask, f);
+    if (mask) phase_masked(a, mask, f, d);
 }
 
 // Pauli error on tile bit q of the true state (Eq. (2)): Z -> phase -1 on
@@ -477,14 +479,20 @@ __device__ __forceinline__ void rg_pauli(Amps &a, TileCtx &c, uint32_t q, uint32
     if (code == 3u) c.gp = (c.gp + 1u) & 3u;  // Y = i X Z
 }
 
-// multiply every amplitude by i^gp (exact) and reset gp
+// the residue that events and their scales left above gp's two bits (EvSlot); multiplied in
+// unconditionally: a branch around it made the batch kernel spill 700 bytes instead of 364
+__device__ __forceinline__ float2 residue(const TileCtx &c) { return bc2((float)((int)c.gp >> 2) * 2.3283064365386963e-10f); }
+
+// multiply every amplitude by i^gp (exact) and its residue, and reset gp
 __device__ __forceinline__ void apply_global_phase(Amps &a, TileCtx &c) {
     if (!c.gp) return;
+    const float2 x = residue(c);
+    c.gp &= 3u;
     const float2 A = bc2(c.gp == 2 ? -1.f : (c.gp == 0 ? 1.f : 0.f)), B = bc2(c.gp == 1 ? 1.f : (c.gp == 3 ? -1.f : 0.f));
     const float2 nB = make_float2(-B.x, -B.y);
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
-        const float2 r = a.re[k], i = a.im[k];
+        const float2 r = fma2(x, a.re[k], a.re[k]), i = fma2(x, a.im[k], a.im[k]);
         a.re[k] = fma2(nB, i, mul2(A, r));
         a.im[k] = fma2(B, r, mul2(A, i));
     }
@@ -727,7 +735,7 @@ __device__ __forceinline__ void apply_op(Amps &a, TileCtx &c, const RegOp &op, c
         case OP_X: c.m ^= 1u << q0; break;
         case OP_OMEGA: rg_omega(a, c, q0, p0, op.aux); break;
         case OP_DIAG1: rg_diag1(a, c, q0, p0, op.c0, op.c1); break;
-        case OP_CP: rg_cp(a, c, q0, q1, op.c0); break;
+        case OP_CP: rg_cp(a, c, q0, q1, op.c0, op.c1.x); break;
         case OP_CX: ARSO_CX(0); break;
         ARSO_P4(OP_CX, ARSO_CX)
         case OP_DENSE2:
@@ -910,7 +918,7 @@ __device__ __forceinline__ void apply_macro(Amps &a, TileCtx &c, const uint4 h, 
 #undef ARSO_CZ_MASKS
         case OP_OMEGA: rg_omega(a, c, q0, p0, (h.x >> 20) & 7u); break;
         case OP_PHASE: phase_pair(a, bit_mask(c, q0), make_float2(__uint_as_float(u->x), __uint_as_float(u->y))); break;
-        case OP_CP: rg_cp(a, c, q0, q1, make_float2(__uint_as_float(u->x), __uint_as_float(u->y))); break;
+        case OP_CP: rg_cp(a, c, q0, q1, make_float2(__uint_as_float(u->x), __uint_as_float(u->y)), __uint_as_float(u->z)); break;
         case OP_SIGN:
         case OP_CX: case OP_CX + 1: case OP_CX + 2: case OP_CX + 3: case OP_CX + 4: {
             const uint4 w = *u;
@@ -961,6 +969,7 @@ __device__ __forceinline__ void apply_macro(Amps &a, TileCtx &c, const uint4 h, 
                 a.re[k] = fma2(nfi, i, mul2(fr, r));
                 a.im[k] = fma2(fi, r, mul2(fr, i));
             }
+            c.gp += u->z;
             break;
         }
         case OP_DENSE1: {
@@ -1039,8 +1048,11 @@ __device__ __forceinline__ void run_prog(Amps &v, TileCtx &c, const uint4 *u, co
                 c.gp ^= ((c.m >> q) & 1u) << 1;
             }
             if (pc & 1u) c.m ^= 1u << q;
-            if (pc == 3u) c.gp = (c.gp + 1u) & 3u;  // Y = i X Z
-            if ((pc & 1u) && (e.x != 1.f || e.y != 0.f)) phase_pair(v, ~bit_mask(c, q), make_float2(e.x, e.y));
+            if (pc == 3u) c.gp = (c.gp & ~3u) | ((c.gp + 1u) & 3u);  // Y = i X Z
+            if ((pc & 1u) && (e.x != 1.f || e.y != 0.f)) {
+                phase_pair(v, ~bit_mask(c, q), make_float2(e.x, e.y));
+                c.gp += __float_as_uint(e.w);
+            }
             ++ev;
             next = ev < ev_end ? *ev : NO_EVENT;
         }
@@ -1300,6 +1312,7 @@ __device__ __forceinline__ void store_tile(const Amps &v, float2 *dst, const Loa
 
 // v (in the load mapping, masks resolved but for c.m without bit 0) times the frame table (internal.h) and i^gp
 __device__ __forceinline__ void apply_frame(Amps &v, TileCtx &c, const float2 *__restrict__ frame, int t) {
+    const float2 x = residue(c);
     const uint32_t nt = 1u << (t - REG_BITS);
     const float4 *T = reinterpret_cast<const float4 *>(frame + nt);
     float2 F = __ldg(frame + (c.tid ^ ((c.m >> 1) & (nt - 1u))));
@@ -1314,7 +1327,7 @@ __device__ __forceinline__ void apply_frame(Amps &v, TileCtx &c, const float2 *_
         const float2 tr = make_float2(w.x, w.y), ti = make_float2(w.z, w.w);
         const float2 gr = fma2(nfi, ti, mul2(fr, tr)), gi = fma2(fi, tr, mul2(fr, ti));
         const float2 ngi = make_float2(-gi.x, -gi.y);
-        const float2 r = v.re[k], i = v.im[k];
+        const float2 r = fma2(x, v.re[k], v.re[k]), i = fma2(x, v.im[k], v.im[k]);
         v.re[k] = fma2(ngi, i, mul2(gr, r));
         v.im[k] = fma2(gi, r, mul2(gr, i));
     }

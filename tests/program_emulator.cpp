@@ -56,8 +56,8 @@ struct Machine {
             phase *= 1.0 + event_scale(v);
         }
     }
-    double event_scale(const EvSlot &) const { return 0.0; }
-    double op_scale(const uint4 &) const { return 0.0; }
+    double event_scale(const EvSlot &v) const { return ((int32_t)v.residue >> 2) / 4294967296.0; }
+    double op_scale(const uint4 &k) const { return ((int32_t)k.z >> 2) / 4294967296.0; }
     void run(uint32_t ph, const std::vector<Event> &ev, size_t &next) {
         uint32_t R[5];
         for (int b = 0; b < 5; ++b) R[b] = c.ph_R[ph] >> (5 * b) & 31u;
@@ -108,7 +108,7 @@ struct Machine {
                 for (uint32_t j = 0; j < N; ++j) s[j] *= (code == OP_PHASE ? bit(j, q0) : bit(j, q0) ^ bit(j, q1)) ? f : std::conj(f);
             } else if (code == OP_CP) {
                 for (uint32_t j = 0; j < N; ++j)
-                    if (bit(j, q0) && bit(j, q1)) s[j] *= c2(k.x, k.y);
+                    if (bit(j, q0) && bit(j, q1)) s[j] *= c2(k.x, k.y) * (1.0 + c2(k.z, 0).real());
             } else if (code == OP_SCALE) {
                 for (cd &x : s) x *= c2(k.x, k.y);
                 phase *= 1.0 + op_scale(k);

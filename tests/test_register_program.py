@@ -49,3 +49,24 @@ def test_matrices_given_in_32_bits_take_the_frame_form(emulate, n, tile):
     r = emulate(circ, tile, 1, 6)
     assert r["dense"] == 0
     assert r["error"] < 2e-6  # 100 constants of at most 6e-8, as a random walk with a factor of three
+
+
+def _clifford_t(n, G, seed):
+    r = np.random.default_rng(seed)
+    out = []
+    for _ in range(G):
+        a, b = (int(v) for v in r.permutation(n)[:2])
+        name = ("H", "T", "S", "CX", "X", "TDG")[int(r.integers(6))]
+        out.append(W.Gate(name, (a, b) if name == "CX" else (a,)))
+    return W.Circuit(n, out)
+
+
+@pytest.mark.parametrize("circ,tile", [(W.cuccaro_adder(7, 100, 77), 13), (W.cuccaro_adder(7, 100, 77), 10),
+                                       (_clifford_t(14, 600, 1), 10), (_clifford_t(12, 600, 1), 0),
+                                       (W.qft_basis(14, 99), 10), (W.qft_basis(12, 99), 0)])
+@pytest.mark.parametrize("events", [0, 5, 30])
+def test_constants_do_not_add_up(emulate, circ, tile, events):
+    # the scalar of a frame, the phase after an error, the scale of a run and a controlled
+    # phase are rounded constants that many amplitudes share; however many there are, the norm is off by one
+    # rounding of the scalar (2^-24), not by one a pass and an event
+    assert abs(emulate(circ, tile, 3, events)["norm"]) < 2.0 ** -24
