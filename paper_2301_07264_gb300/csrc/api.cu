@@ -1450,10 +1450,8 @@ static void run_mixed(const std::vector<size_t> &sel, arso_circuit *const *circu
                 b.n_phases = (uint32_t)c->ph_R.size();
                 b.n_ckpt = c->n_ckpt;
                 b.ckpt_every = (uint32_t)c->ckpt_every;
-                b.gates = c->d_gates.as<DGate>();
                 b.mats = c->d_rmats.as<float2>();
                 b.ph_R = c->d_ph_R.as<uint32_t>();
-                b.phase_of_pos = c->d_phase_of_pos.as<uint32_t>();
                 b.prog = c->d_prog.as<uint4>();
                 b.ph_pg = c->d_ph_pg.as<uint32_t>();
                 b.evs = c->d_evs.as<EvSlot>();
@@ -1930,10 +1928,8 @@ arso_status arso_run_batch(size_t count, arso_circuit *const *circuits, const ar
                 b.n_phases = (uint32_t)c->ph_R.size();
                 b.n_ckpt = c->n_ckpt;
                 b.ckpt_every = (uint32_t)c->ckpt_every;
-                b.gates = c->d_gates.as<DGate>();
                 b.mats = c->d_rmats.as<float2>();
                 b.ph_R = c->d_ph_R.as<uint32_t>();
-                b.phase_of_pos = c->d_phase_of_pos.as<uint32_t>();
                 b.prog = c->d_prog.as<uint4>();
                 b.ph_pg = c->d_ph_pg.as<uint32_t>();
                 b.evs = c->d_evs.as<EvSlot>();

@@ -111,9 +111,8 @@ void prepare_pass_rb();
 struct BatchCircuit {
     int n;
     uint32_t n_phases, n_ckpt, ckpt_every;
-    const DGate *gates;
     const float2 *mats;
-    const uint32_t *ph_R, *phase_of_pos;
+    const uint32_t *ph_R;
     const uint4 *prog;  // as in ResidentArgs
     const uint32_t *ph_pg;
     const EvSlot *evs;
