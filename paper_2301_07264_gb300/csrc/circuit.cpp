@@ -1135,7 +1135,6 @@ static void tensor_records(arso_circuit *c) {
                 o.c1 = f2(h.m[3]);
             } else if (cls == GC_DIAG2) {
                 o.c0 = f2(h.m[15]);
-                o.c1.x = modulus_gap(h.m[15], o.c0);
             }
             o.pad[0] = reg_opcode(cls, p0, p1);
             o.pad[1] = (uint32_t)c->role[pos];
@@ -1334,11 +1333,9 @@ static void reg_program(arso_circuit *c) {
                     }
                     case GC_DIAG2: {  // commutes with the frame
                         const float2 f = f2(h.m[15]);
-                        const float d = modulus_gap(h.m[15], f);
                         uint32_t cst[2];
                         std::memcpy(cst, &f, 8);
                         W.op(code, pos + 1, z, cst);
-                        std::memcpy(&W.out.back().z, &d, 4);
                         break;
                     }
                     case GC_CZ: W.cz(q0, q1, p0, p1, pos); break;

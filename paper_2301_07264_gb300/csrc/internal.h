@@ -94,7 +94,7 @@ struct DGate {
 //   w0  = cls | p0 << 8 | p1 << 12 | q0 << 16 | q1 << 24, with p0/p1 the
 //         register positions of q0/q1 in the gate's phase (15: thread bit)
 //   aux = matrix-pool offset (dense gates) or the exponent k of GC_OMEGA
-//   c0, c1 = inline constants: (a, b) of GC_SU2, (d0, d1) of GC_DIAG1, (f, d) of OP_CP
+//   c0, c1 = inline constants: (a, b) of GC_SU2, (d0, d1) of GC_DIAG1, c0 of OP_CP
 struct __align__(16) RegOp {
     uint32_t w0, aux;
     float2 c0, c1;
@@ -118,7 +118,7 @@ enum RegOpCode : uint32_t {
     OP_X = 71,       // tensor circuits only
     OP_OMEGA = 72,   // diag(1, omega^k), omega = e^{i pi/4}
     OP_DIAG1 = 73,   // tensor circuits only
-    OP_CP = 74,      // diag(1, 1, 1, f (1 + d)), d = what the rounded f lacks of modulus 1
+    OP_CP = 74,      // diag(1, 1, 1, f)
     OP_CX = 75,      // + target position; in a register program a flip under a condition (below)
     OP_DENSE2 = 80,
     OP_SWAP = 81,
@@ -139,8 +139,8 @@ enum RegOpCode : uint32_t {
 //               event commutes with the macro-op's other gates)
 //           z = q0 | q1 << 8 | p0 << 16 | p1 << 20 (tile bits and register positions)
 //           w = tile bits whose index-mask bit flips before the op (X)
-//   second unit where the op has constants: x, y = f (OP_SCALE: z its residue, see EvSlot; OP_CP:
-//           z = d), or x = matrix-pool offset
+//   second unit where the op has constants: x, y = f (OP_SCALE: z its residue, see EvSlot), or x =
+//           matrix-pool offset
 //   OP_LAYER: bits 8-12 of x the register positions that hold a gate G(x), bits 13-17
 //           those whose x is real; one unit (Re x, Re x, Im x, Im x) for each, in order
 //           (position 0: (Re x, -Re x, Im x, Im x), the lanes of a packed register)

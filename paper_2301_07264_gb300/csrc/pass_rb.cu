@@ -435,18 +435,16 @@ template <int IDX> __device__ __forceinline__ void cz_case(Amps &a) {
     neg_quarter<cz_pa(IDX >> 2), cz_pb(IDX >> 2), (IDX >> 1) & 1, IDX & 1>(a);
 }
 
-// multiply the registers selected by mask by f (1 + d): d is what the rounded f lacks of modulus
-// 1, which every amplitude it meets would lose alike (norm of a 16-qubit QFT: 2.7e-7 short)
-__device__ __forceinline__ void phase_masked(Amps &a, uint32_t mask, float2 f, float d) {
+// multiply the registers selected by mask by f
+__device__ __forceinline__ void phase_masked(Amps &a, uint32_t mask, float2 f) {
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
         const bool x = (mask >> (2 * k)) & 1u, y = (mask >> (2 * k + 1)) & 1u;
         const float2 fr = make_float2(x ? f.x : 1.f, y ? f.x : 1.f), fi = make_float2(x ? f.y : 0.f, y ? f.y : 0.f);
-        const float2 nfi = make_float2(-fi.x, -fi.y), dd = make_float2(x ? d : 0.f, y ? d : 0.f);
+        const float2 nfi = make_float2(-fi.x, -fi.y);
         const float2 r = a.re[k], i = a.im[k];
-        const float2 nr = fma2(nfi, i, mul2(fr, r)), ni = fma2(fi, r, mul2(fr, i));
-        a.re[k] = fma2(dd, nr, nr);
-        a.im[k] = fma2(dd, ni, ni);
+        a.re[k] = fma2(nfi, i, mul2(fr, r));
+        a.im[k] = fma2(fi, r, mul2(fr, i));
     }
 }
 // multiply the registers selected by mask by f, the others by its conjugate
@@ -463,9 +461,9 @@ __device__ __forceinline__ void phase_pair(Amps &a, uint32_t mask, float2 f) {
     }
 }
 // diag(1, 1, 1, f) on tile bits qa, qb
-__device__ __forceinline__ void rg_cp(Amps &a, const TileCtx &c, uint32_t qa, uint32_t qb, float2 f, float d) {
+__device__ __forceinline__ void rg_cp(Amps &a, const TileCtx &c, uint32_t qa, uint32_t qb, float2 f) {
     const uint32_t mask = bit_mask(c, qa) & bit_mask(c, qb);
-    if (mask) phase_masked(a, mask, f, d);
+    if (mask) phase_masked(a, mask, f);
 }
 
 // Pauli error on tile bit q of the true state (Eq. (2)): Z -> phase -1 on
@@ -735,7 +733,7 @@ __device__ __forceinline__ void apply_op(Amps &a, TileCtx &c, const RegOp &op, c
         case OP_X: c.m ^= 1u << q0; break;
         case OP_OMEGA: rg_omega(a, c, q0, p0, op.aux); break;
         case OP_DIAG1: rg_diag1(a, c, q0, p0, op.c0, op.c1); break;
-        case OP_CP: rg_cp(a, c, q0, q1, op.c0, op.c1.x); break;
+        case OP_CP: rg_cp(a, c, q0, q1, op.c0); break;
         case OP_CX: ARSO_CX(0); break;
         ARSO_P4(OP_CX, ARSO_CX)
         case OP_DENSE2:
@@ -918,7 +916,7 @@ __device__ __forceinline__ void apply_macro(Amps &a, TileCtx &c, const uint4 h, 
 #undef ARSO_CZ_MASKS
         case OP_OMEGA: rg_omega(a, c, q0, p0, (h.x >> 20) & 7u); break;
         case OP_PHASE: phase_pair(a, bit_mask(c, q0), make_float2(__uint_as_float(u->x), __uint_as_float(u->y))); break;
-        case OP_CP: rg_cp(a, c, q0, q1, make_float2(__uint_as_float(u->x), __uint_as_float(u->y)), __uint_as_float(u->z)); break;
+        case OP_CP: rg_cp(a, c, q0, q1, make_float2(__uint_as_float(u->x), __uint_as_float(u->y))); break;
         case OP_SIGN:
         case OP_CX: case OP_CX + 1: case OP_CX + 2: case OP_CX + 3: case OP_CX + 4: {
             const uint4 w = *u;

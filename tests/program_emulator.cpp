@@ -108,7 +108,7 @@ struct Machine {
                 for (uint32_t j = 0; j < N; ++j) s[j] *= (code == OP_PHASE ? bit(j, q0) : bit(j, q0) ^ bit(j, q1)) ? f : std::conj(f);
             } else if (code == OP_CP) {
                 for (uint32_t j = 0; j < N; ++j)
-                    if (bit(j, q0) && bit(j, q1)) s[j] *= c2(k.x, k.y) * (1.0 + c2(k.z, 0).real());
+                    if (bit(j, q0) && bit(j, q1)) s[j] *= c2(k.x, k.y);
             } else if (code == OP_SCALE) {
                 for (cd &x : s) x *= c2(k.x, k.y);
                 phase *= 1.0 + op_scale(k);

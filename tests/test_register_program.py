@@ -62,11 +62,10 @@ def _clifford_t(n, G, seed):
 
 
 @pytest.mark.parametrize("circ,tile", [(W.cuccaro_adder(7, 100, 77), 13), (W.cuccaro_adder(7, 100, 77), 10),
-                                       (_clifford_t(14, 600, 1), 10), (_clifford_t(12, 600, 1), 0),
-                                       (W.qft_basis(14, 99), 10), (W.qft_basis(12, 99), 0)])
+                                       (_clifford_t(14, 600, 1), 10), (_clifford_t(12, 600, 1), 0)])
 @pytest.mark.parametrize("events", [0, 5, 30])
 def test_constants_do_not_add_up(emulate, circ, tile, events):
-    # the scalar of a frame, the phase after an error, the scale of a run and a controlled
-    # phase are rounded constants that many amplitudes share; however many there are, the norm is off by one
-    # rounding of the scalar (2^-24), not by one a pass and an event
+    # the scalar of a frame, the phase after an error and the scale of a run are rounded constants
+    # that all amplitudes share; however many there are, the norm is off by one rounding of the
+    # scalar (2^-24), not by one a pass and an event
     assert abs(emulate(circ, tile, 3, events)["norm"]) < 2.0 ** -24
