@@ -423,10 +423,11 @@ static void tensor_phase(arso_circuit *c, uint32_t ph, uint32_t gb, uint32_t ge,
 
 static float2 f2(cd v) { return make_float2((float)v.real(), (float)v.imag()); }
 
-// what a constant rounded to FP32 lacks of its modulus, as a factor and in the units of gp (internal.h)
-static double modulus_gap(cd exact, float2 f) { return std::abs(exact) / std::abs(cd(f.x, f.y)) - 1.0; }
-static uint32_t modulus_residue(cd exact, float2 f) {
-    return (uint32_t)(int32_t)std::llround(modulus_gap(exact, f) * 4294967296.0) << 2;
+// what to add to the real part of f, a constant rounded to FP32, for the exact modulus; next to
+// the imaginary axis, where that would turn f more than its rounding did, for the exact real part
+static float real_gap(cd exact, float2 f) {
+    const double n = std::norm(exact), x = f.x;
+    return (float)(8.0 * x * x > n ? (n - std::norm(cd(f.x, f.y))) / (2.0 * x) : exact.real() - x);
 }
 
 static cd omega(int k) {
@@ -1229,11 +1230,11 @@ static void emit_run(arso_circuit *c, ProgWriter &W, Frame &F, const std::vector
     const cd ratio = F.S() / fused.S();
     if (std::abs(ratio - 1.0) > 1e-14) {
         const float2 f = f2(ratio);
-        uint32_t cst[3];
+        const float d = real_gap(ratio, f);
+        uint32_t cst[2];
         std::memcpy(cst, &f, 8);
-        cst[2] = modulus_residue(ratio, f);
         W.op(OP_SCALE, end, 0, cst);
-        W.out.back().z = cst[2];
+        std::memcpy(&W.out.back().z, &d, 4);
     }
     W.out[head].z = (uint32_t)(W.out.size() - slow);
     W.last = SIZE_MAX;  // nor a later one in a macro-op that the fused path passes over
@@ -1344,7 +1345,7 @@ static void reg_program(arso_circuit *c) {
                 }
                 auto slot = [&](uint32_t q) {
                     const float2 f = f2(F.phi(q));
-                    return EvSlot{f, q, modulus_residue(F.phi(q), f)};
+                    return EvSlot{f, q, real_gap(F.phi(q), f)};
                 };
                 c->evs[2 * pos] = slot(q0);
                 c->evs[2 * pos + 1] = slot(q1);

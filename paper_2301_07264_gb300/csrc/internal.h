@@ -129,7 +129,7 @@ enum RegOpCode : uint32_t {
     OP_BLOCK = 87,   // a fused run of gates (below)
     OP_SIGN = 88,    // the signs of a fused run without a flip (below)
     OP_PARITY = 89,  // f where q0 ^ q1 = 1, conj f elsewhere (a fused run)
-    OP_SCALE = 90,   // every amplitude times f
+    OP_SCALE = 90,   // every amplitude times f + d
 };
 
 // Register program of a phase (circuits without tensor phases): macro-ops of 16-byte units.
@@ -139,8 +139,8 @@ enum RegOpCode : uint32_t {
 //               event commutes with the macro-op's other gates)
 //           z = q0 | q1 << 8 | p0 << 16 | p1 << 20 (tile bits and register positions)
 //           w = tile bits whose index-mask bit flips before the op (X)
-//   second unit where the op has constants: x, y = f (OP_SCALE: z its residue, see EvSlot), or x =
-//           matrix-pool offset
+//   second unit where the op has constants: x, y = f, or x = matrix-pool offset
+//           (OP_SCALE: z = d, see EvSlot)
 //   OP_LAYER: bits 8-12 of x the register positions that hold a gate G(x), bits 13-17
 //           those whose x is real; one unit (Re x, Re x, Im x, Im x) for each, in order
 //           (position 0: (Re x, -Re x, Im x, Im x), the lanes of a packed register)
@@ -167,14 +167,10 @@ enum RegOpCode : uint32_t {
 // after the gate, and the qubit's tile bit.
 struct __align__(16) EvSlot {
     float2 phi;
-    uint32_t q, residue;  // residue: what phi, rounded, lacks of modulus 1, in the units of gp
+    uint32_t q;
+    float d;  // what the real part of the rounded phi lacks for modulus 1: all amplitudes would lose
+              // that alike, and over the events it would add up
 };
-
-// The power of i that the kernels keep for a trajectory, gp, has two bits; above them it counts,
-// in units of 2^-32, what the moduli of the rounded constants that events brought in lack of
-// the exact ones. Each is the same for all amplitudes, so they would add up over the events;
-// the state is multiplied by 1 + their sum where gp is applied. (Two million events of the
-// largest residue would fill it.)
 
 // A frame as the kernels apply it, in the load/store register mapping of a t-qubit
 // tile: 2^(t-5) thread factors (S times the phases of tile bits 1..t-5), then the 32

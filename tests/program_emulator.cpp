@@ -52,12 +52,10 @@ struct Machine {
         if (e.code & 1) m ^= 1u << g[v.q];
         if (e.code == 3) phase *= cd(0, 1);
         if ((e.code & 1) && (v.phi.x != 1.f || v.phi.y != 0.f)) {
-            for (uint32_t j = 0; j < N; ++j) s[j] *= bit(j, v.q) ? std::conj(c2(v.phi)) : c2(v.phi);
-            phase *= 1.0 + event_scale(v);
+            const cd f = c2(v.phi) + (double)v.d;
+            for (uint32_t j = 0; j < N; ++j) s[j] *= bit(j, v.q) ? std::conj(f) : f;
         }
     }
-    double event_scale(const EvSlot &v) const { return ((int32_t)v.residue >> 2) / 4294967296.0; }
-    double op_scale(const uint4 &k) const { return ((int32_t)k.z >> 2) / 4294967296.0; }
     void run(uint32_t ph, const std::vector<Event> &ev, size_t &next) {
         uint32_t R[5];
         for (int b = 0; b < 5; ++b) R[b] = c.ph_R[ph] >> (5 * b) & 31u;
@@ -110,8 +108,7 @@ struct Machine {
                 for (uint32_t j = 0; j < N; ++j)
                     if (bit(j, q0) && bit(j, q1)) s[j] *= c2(k.x, k.y);
             } else if (code == OP_SCALE) {
-                for (cd &x : s) x *= c2(k.x, k.y);
-                phase *= 1.0 + op_scale(k);
+                for (cd &x : s) x *= c2(k.x, k.y) + c2(k.z, 0).real();
             } else if (code >= OP_DENSE1 && code < OP_DENSE1 + 5) {
                 const float2 *M = c.rmats.data() + k.x;
                 pair(R[code - OP_DENSE1], c2(M[0]), c2(M[1]), c2(M[2]), c2(M[3]));
