@@ -480,7 +480,10 @@ arso_status arso_score_state_noalloc(uint32_t n_qubits, const void *amps, const 
  * for a dense one-qubit gate (2x2 complex matrix-vector product), 30 for a
  * dense two-qubit gate, 6 for a diagonal gate, 4 for H, 2 for an odd power
  * of the T phase and 0 for permutations and sign flips (X, CX, SWAP, CZ, Z,
- * S), times the amplitudes each launch sweeps.
+ * S), times the amplitudes each launch sweeps. These are the method's
+ * operations, the same for every way of doing it; the register kernels execute
+ * fewer (8 for a dense one-qubit gate, 4 for one with real entries or H, none
+ * for most diagonal gates and for gates inside a fused run).
  * Launch and host<->device transfer counters run whether or not timing is
  * enabled. Process-wide, thread-safe; reading resolves pending events. */
 enum {

@@ -463,7 +463,7 @@ __device__ __forceinline__ void phase_pair(Amps &a, uint32_t mask, float2 f) {
 // the same with d added to the real part of f (EvSlot), for constants that a trajectory's errors
 // bring in. d is less than a rounding of the product, so it goes in before the last two: a
 // factor 1 + d on the result would round back. Norm of 64 trajectories, largest error: 16-qubit
-// Clifford+T circuit of 3,000 gates, some 80 errors each, 9.9e-7 without d, 2.8e-7 with such a
+// Clifford+T circuit of 3,000 gates, some 70 errors each, 9.9e-7 without d, 2.8e-7 with such a
 // factor, 8.4e-8 so.
 __device__ __forceinline__ void phase_pair_exact(Amps &a, uint32_t mask, float2 f, float d) {
     const float2 fr = bc2(f.x), dd = bc2(d);
@@ -1494,12 +1494,14 @@ __global__ void __launch_bounds__(THREADS, MINB) pass_rb_kernel(PassArgs a) {
     pass_finish(a, v, c, blockIdx.y, blockIdx.x * groups + sg, s_base[sg], gridDim.x * groups, red);
 }
 
-// One pass of a probe circuit (kernels.h), or some of its phases, over a state in place: CTAs loop over the tiles,
-// so that each warp keeps one row of sums. Bound by instruction issue: a measurement is 64
+// One pass of a probe circuit (kernels.h), or some of its phases, over a state in place: CTAs
+// loop over the tiles, so that each warp keeps one row of sums. Bound by instruction issue: a measurement is 64
 // packed multiply-adds and about 70 instructions of exchange per warp, next to 64 for the
 // gate before it, and a pass reads and writes the state once for some 40 gates. Whole
 // single-error analysis, before (one HBM sweep per gate) and after: 24-qubit brickwork, 1,880
-// locations, 88.7 -> 23.7 ms; 20-qubit adder, both states, 25.4 -> 1.16 ms.
+// locations, 88.7 -> 33.0 ms for the first call of a handle, which plans and uploads the probe
+// circuit, and 23.3 ms for the later ones, which find it there; 20-qubit adder, both states,
+// 25.4 -> 1.95 and 0.87 ms.
 template <int THREADS, int MINB, bool DUAL>
 __global__ void __launch_bounds__(THREADS, MINB) probe_kernel(ProbeArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -2,9 +2,10 @@
 // unless a caller makes others), shared by every handle and every call. Allocation is
 // stream-ordered and thread-safe (the driver's), and the pool keeps up to POOL_KEEP freed
 // bytes mapped: mapping and unmapping a call's working states (8 GiB at 24 qubits) took
-// 19 ms of each call, and the five buffers of an error list 0.2 ms with cudaMalloc. When the last circuit or surrogate handle is freed, all but
-// POOL_IDLE goes back: a program that makes one handle at a time would otherwise map its
-// memory anew for each (0.7 ms of a surrogate's 2.8).
+// 19 ms of each call, and the five buffers of an error list 0.2 ms with cudaMalloc. When the
+// last circuit or surrogate handle is freed, all but POOL_IDLE goes back: a program that makes
+// one handle at a time would otherwise map its memory anew for each (0.7 ms of a surrogate's
+// 2.8).
 //
 // Two pools a context. Working memory is freed on the stream (or the idle stream) that
 // allocated it, and only that one reuses it: with the driver's search among the blocks of

@@ -11,7 +11,7 @@ def test_many_events_keep_the_norm():
     from paper_2301_07264_gb300 import arso
     from workloads import circuits as W
     # T gates leave odd powers of e^{i pi/4} as frame phases: the same rounded constant in every
-    # event. Some 80 events a trajectory; their mean stays within one rounding of a scalar
+    # event. Some 70 events a trajectory; their mean stays within one rounding of a scalar
     # (without compensation -8.6e-7, with a factor that rounds back -1.2e-7)
     r = np.random.default_rng(2)
     gates = []
